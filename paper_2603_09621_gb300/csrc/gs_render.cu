@@ -8,17 +8,17 @@
 // in both kernels from the voxel's global index and the Gaussian alone, so forward and
 // adjoint agree on every inclusion decision and no result depends on the brick shape.
 //
-// Forward: the brick is split into 4 x 4 x 4 footprints, one half-warp each; a lane owns one
-// x-row of four voxels. The block stages the brick's list in rounds of about 28 records per
-// footprint (224 for an 8^3 brick), so most lists take one round and smaller bricks, with
-// shorter lists, keep more blocks resident. A half-warp tests 16 staged Gaussians against
-// its footprint with one ballot and three conservative tests: the triangle inequality in
-// whitened space (|M (p - mu)| >= |M (c - mu)| - rho4, with rho4 the whitened radius of the
-// footprint around its centre c, so a footprint whose centre is farther than sqrt(T) + rho4
-// is missed), the truncated ellipsoid's bounding box widened by 3/2 along each axis, and q's
-// lower bound from the smallest eigenvalue at the footprint's nearest point; a margin
-// absorbs FP32 rounding. It evaluates the hits in ascending Gaussian id, accumulating S and W in registers
-// (deterministic; one packed FFMA2 updates a voxel's (S, W) with (v r, r) g).
+// Forward: the brick is split into 4 x 4 x 4 footprints, a quarter-warp each; a lane owns the two
+// x-rows of four voxels at z and z + 1. The block stages the brick's list in rounds of 20 records
+// per footprint (160 for an 8^3 brick); smaller bricks, with shorter lists, take shorter rounds
+// and keep more blocks resident. The thread that stages a record tests it against every footprint
+// (three conservative tests, see foot_mask: the triangle inequality in whitened space
+// |M (p - mu)| >= |M (c - mu)| - rho4, with rho4 the whitened radius of the footprint around its
+// centre c; the truncated ellipsoid's bounding box widened by 3/2 along each axis; and q's lower
+// bound from the smallest eigenvalue at the footprint's nearest point; a margin absorbs FP32
+// rounding). Each warp lists the hits of its footprints and evaluates them in ascending Gaussian
+// id, accumulating S and W in registers (deterministic; one packed FFMA2 updates a voxel's (S, W)
+// with (v r, r) g).
 // Adjoint: one thread per (brick, Gaussian) pair evaluates the brick rows the Gaussian
 // reaches (the row shadow, per z-row a quadratic in dy; z-planes whose section of the
 // ellipsoid misses the brick's x range are skipped), each row as bx predicated voxel slots in
@@ -44,8 +44,8 @@
 
 namespace gs {
 
-constexpr int kFwdChunkPerFoot = 28;  // Gaussians staged per forward round and 4^3 footprint
-                                      // (in steps of a factor 2: 56, 112 or 224 records)
+constexpr int kFwdChunkPerFoot = 20;  // Gaussians staged per forward round and 4^3 footprint
+                                      // (in steps of a factor 2: 40, 80 or 160 records)
 constexpr int kBwdThreads = 128;
 constexpr int kBwdPairs = 256;        // pairs per adjoint block, taken by warps 32 at a time
 constexpr int kBwdStage = 4;          // bricks of per-voxel factors staged per adjoint block
@@ -136,128 +136,202 @@ __device__ __forceinline__ float ux_base(const Rec& R, int x4) {
     return (float(x4) + R.nmhx) + R.nmlx;
 }
 
-// Scaled x offset of voxel x = x4 + k (x4 = x & ~3) from the row minimum, tq = sa (u - dx*),
-// taken as tq = fma(k, sa, tq0) from the group's tq0 = sa (ux_base(R, x4) - dx*); then
-// q = fma(tq, tq, S). Every kernel uses this operation sequence, so forward and adjoint agree
+// The scaled x offset of voxel x = x4 + k (x4 = x & ~3) from the row minimum, tq = sa (u - dx*),
+// is taken as tq = fma(k, sa, tq0) from the group's tq0 = sa (ux_base(R, x4) - dx*); then
+// q = fma(tq, tq, S). Both kernels use this operation sequence, so forward and adjoint agree
 // on every inclusion q <= T.
-__device__ __forceinline__ float tq_base(const Rec& R, int x4, float dxs) {
-    return R.sa * (ux_base(R, x4) - dxs);
-}
 
-__device__ __forceinline__ float q_of_k(const Rec& R, float tq0, int k, float S) {
-    const float tq = (k == 0) ? tq0 : fmaf(float(k), R.sa, tq0);
-    return fmaf(tq, tq, S);
-}
-
-// Footprint cull: may the Gaussian reach a voxel centre within 3/2 of (cx, cy, cz) per axis?
-// Three conservative tests: the whitened triangle inequality; the footprint centre's offset
-// from the mean against the truncated ellipsoid's box widened by the footprint's half-width;
-// and q's lower bound lam |p - mu|^2 at the footprint's voxel box's nearest point (exact for
-// isotropic Gaussians, it drops footprints that only a corner of the ellipsoid grazes between
-// voxel centres). (An approximate square root suffices: Tcull carries a 1 % margin over T.)
-__device__ __forceinline__ bool foot_hit(const float4* s, float cx, float cy, float cz,
-                                         float sqrtTcull) {
-    const Rec R = load_rec(s);
-    float dy, dz, S, dxs;
-    row_terms(R, f2(cy, cz), dy, dz, S, dxs);
-    const float ux = (cx + R.nmhx) + R.nmlx;
-    const float tq = R.sa * (ux - dxs);
-    const float qc = fmaf(tq, tq, S);
-    const float ax = fmaxf(fabsf(ux) - 1.5f, 0.0f), ay = fmaxf(fabsf(dy) - 1.5f, 0.0f);
-    const float az = fmaxf(fabsf(dz) - 1.5f, 0.0f);
-    const float dist2 = fmaf(ax, ax, fmaf(ay, ay, az * az));
-    return (sqrt_approx(fmaxf(qc, 0.0f)) - R.rho4 <= sqrtTcull) & (fabsf(ux) <= R.ex) &
-           (fabsf(dy) <= R.ey) & (fabsf(dz) <= R.ez) & (R.lam * dist2 <= sqrtTcull * sqrtTcull);
+// Footprint cull: bit f of the result is set where the Gaussian of the record may reach a voxel
+// centre of the brick's 4^3 footprint f = (wz FY + wy) FX + wx. Three conservative tests per
+// footprint, at its centre (half-width 3/2 per axis): the whitened triangle inequality; the
+// centre's offset from the mean against the truncated ellipsoid's box widened by the half-width;
+// and q's lower bound lam |p - mu|^2 at the footprint's nearest point (exact for isotropic
+// Gaussians, it drops footprints that only a corner of the ellipsoid grazes between voxel
+// centres). (An approximate square root suffices: Tcull carries a 1 % margin over T.)
+// kFX, kFY, kFZ: footprints per axis at compile time (0: taken from G).
+template <int kFX, int kFY, int kFZ>
+__device__ __forceinline__ unsigned foot_mask(const Rec& R, const RenderGeo& G, int ox, int oy, int oz) {
+    const int fx = kFX > 0 ? kFX : G.fx, fy = kFY > 0 ? kFY : G.fy, fz = kFZ > 0 ? kFZ : G.fz;
+    unsigned mask = 0;
+    int bit = 0;
+#pragma unroll (kFZ > 0 ? kFZ : 1)
+    for (int wz = 0; wz < fz; ++wz)
+#pragma unroll (kFY > 0 ? kFY : 1)
+        for (int wy = 0; wy < fy; ++wy) {
+            float dy, dz, S, dxs;
+            row_terms(R, f2(float(oy + 4 * wy) + 1.5f, float(oz + 4 * wz) + 1.5f), dy, dz, S, dxs);
+            const float ay = fmaxf(fabsf(dy) - 1.5f, 0.0f), az = fmaxf(fabsf(dz) - 1.5f, 0.0f);
+            const float ayz = fmaf(ay, ay, az * az);
+            const bool in_yz = (fabsf(dy) <= R.ey) & (fabsf(dz) <= R.ez);
+#pragma unroll (kFX > 0 ? kFX : 1)
+            for (int wx = 0; wx < fx; ++wx, ++bit) {
+                const float ux = (float(ox + 4 * wx) + 1.5f + R.nmhx) + R.nmlx;
+                const float tq = R.sa * (ux - dxs);
+                const float qc = fmaf(tq, tq, S);
+                const float ax = fmaxf(fabsf(ux) - 1.5f, 0.0f);
+                const bool hit = (sqrt_approx(fmaxf(qc, 0.0f)) - R.rho4 <= G.sqrtTcull) & (fabsf(ux) <= R.ex) &
+                                 in_yz & (R.lam * fmaf(ax, ax, ayz) <= G.sqrtTcull * G.sqrtTcull);
+                mask |= hit ? 1u << bit : 0u;
+            }
+        }
+    return mask;
 }
 
 // ------------------------------------------------------------------------ forward
 
+// One block of 32 or 64 threads per brick. What bounds it is instruction issue (72 % active) and
+// the latency of the gathered records, so work per instruction decides:
+//   - A quarter-warp per 4^3 footprint, a lane owning the x-rows at z and z + 1: the row terms,
+//     offsets and exponents of the two rows run as FP32x2 pairs (element by element the scalar
+//     operations, so results are bit-identical to one row per lane). Against a half-warp per
+//     footprint and one row per lane: 277 -> 241 us (256 x 256 x 128 grid, 500k Gaussians of a fit
+//     in progress, 132M effective pairs, L2 flushed), 6.97 -> 6.13 ms (512 x 512 x 256 grid, 4M
+//     clustered Gaussians).
+//   - The thread that stages a record also culls it against all the brick's footprints from
+//     registers (row terms shared along x). With one lane per (record, footprint) reading the
+//     staged copy, the cull's shared-memory loads were half of all its wavefronts, and staging
+//     and culling took 110 us of the 241. Each warp then lists its footprints' hits of the whole
+//     round, so quarters of unequal hit counts wait for one another once per round instead of
+//     once per 32 records: 241 -> 215 us, 6.13 -> 5.28 ms.
+//   - Four hits per iteration (the lists are padded with a null record): 215 -> 212 us,
+//     5.28 -> 5.17 ms, and 35 -> 27 us where few bricks leave one warp per scheduler (32^3 grid,
+//     4,096 Gaussians). Two hits 217 us, eight 215 us.
+//   - 72 registers, 14 blocks per SM, 20 records per round and footprint: 209 us and 5.23 ms. 16
+//     records 212 us and 5.20 ms; 24 records 207 us but 5.50 ms; 64 registers (spills) 216 us;
+//     96 registers 217 us. Rounds double-buffered with cp.async measured slower (242 against
+//     241 us, 7.06 against 6.13 ms).
+constexpr int kFwdHits = 4;  // hits per iteration of the evaluation loop (one 32-bit list word)
+
 template <bool kStats, int kChunk>
-__global__ void __launch_bounds__(128, 10) k_render_fwd(const int32_t* __restrict__ brick_off,
-                                                    const int32_t* __restrict__ pair_gid,
-                                                    const float4* __restrict__ rec4, RenderGeo G,
-                                                    float* __restrict__ I, float* __restrict__ W,
-                                                    unsigned long long* __restrict__ stats) {
+__global__ void __launch_bounds__(64, 14) k_render_fwd(const int32_t* __restrict__ brick_off,
+                                                       const int32_t* __restrict__ pair_gid,
+                                                       const float4* __restrict__ rec4, RenderGeo G,
+                                                       float* __restrict__ I, float* __restrict__ W,
+                                                       unsigned long long* __restrict__ stats) {
     pdl_enter();
-    __shared__ float4 srec[kChunk][REC_F4];
+    static_assert(kChunk < 256, "hit lists hold record slots in bytes");
+    // quads 0, 1, 2 and 4 of each record; slot kChunk is the null record (v r = r = 0: it adds 0)
+    __shared__ float4 srec[4][kChunk + 1];
+    __shared__ unsigned char sfoot[kChunk];
+    __shared__ __align__(4) unsigned char slist[8][kChunk + kFwdHits];
     const int tid = threadIdx.x, lane = tid & 31;
     const int nthreads = blockDim.x;
     const int b = blockIdx.x;
     int bx, by, bz;
     brick_xyz(b, G, bx, by, bz);
-    // half-warp per 4^3 footprint; a lane owns one x-row of 4 voxels
-    const int foot = tid >> 4, l16 = lane & 15;
+    // quarter-warp per 4^3 footprint; a lane owns two x-rows of 4 voxels, at z and z + 1
+    const int foot = tid >> 3, l8 = lane & 7, foot0 = (tid >> 5) * 4;
     const int n_foot = G.fx * G.fy * G.fz;
     const bool foot_ok = foot < n_foot;
     const int f = foot_ok ? foot : 0;
     const int wx = f % G.fx, wy = (f / G.fx) % G.fy, wz = f / (G.fx * G.fy);
-    const int ox = bx * G.bsx + wx * 4, oy = by * G.bsy + wy * 4, oz = bz * G.bsz + wz * 4;
-    const int y = oy + (l16 & 3), z = oz + (l16 >> 2);
-    const float2 fyz = f2(float(y), float(z));
-    const float cx = float(ox) + 1.5f, cy = float(oy) + 1.5f, cz = float(oz) + 1.5f;
-    const unsigned half_sel = (lane < 16) ? 0x0000ffffu : 0xffff0000u;
+    const int x0 = bx * G.bsx, y0 = by * G.bsy, z0 = bz * G.bsz;
+    const int ox = x0 + wx * 4, oy = y0 + wy * 4, oz = z0 + wz * 4;
+    const int y = oy + (l8 & 3), z = oz + 2 * (l8 >> 2);
+    const float fy = float(y);
+    const float2 fz2 = f2(float(z), float(z + 1));
+    if (tid < 4) srec[tid][kChunk] = make_float4(0.f, 0.f, 0.f, 0.f);
 
-    float2 SW[4];  // (S, W) of the lane's four voxels
+    float2 SWa[4], SWb[4];  // (S, W) of the lane's voxels in its two rows
 #pragma unroll
-    for (int xi = 0; xi < 4; ++xi) SW[xi] = f2(0.f, 0.f);
+    for (int xi = 0; xi < 4; ++xi) SWa[xi] = SWb[xi] = f2(0.f, 0.f);
     unsigned long long n_eff = 0, n_eval = 0;
     const int start = brick_off[b], end = brick_off[b + 1];
     for (int c0 = start; c0 < end; c0 += kChunk) {
         const int cnt = min(kChunk, end - c0);
         if (c0 != start) __syncthreads();  // the previous chunk's records are no longer read
-        for (int k = tid; k < cnt; k += nthreads) {  // a thread stages one record
+        for (int k = tid; k < cnt; k += nthreads) {  // a thread stages and culls one record
             const float4* src = rec4 + int64_t(pair_gid[c0 + k]) * REC_F4;
+            float4 q[REC_F4];
 #pragma unroll
-            for (int part = 0; part < REC_F4; ++part) srec[k][part] = src[part];
+            for (int part = 0; part < REC_F4; ++part) q[part] = src[part];
+            const Rec R = load_rec(q);
+            const unsigned m = (G.fx == 2 && G.fy == 2 && G.fz == 2) ? foot_mask<2, 2, 2>(R, G, x0, y0, z0)
+                               : (G.fx == 2 && G.fy == 2 && G.fz == 1)
+                                   ? foot_mask<2, 2, 1>(R, G, x0, y0, z0)
+                                   : foot_mask<0, 0, 0>(R, G, x0, y0, z0);
+            sfoot[k] = static_cast<unsigned char>(m);
+            srec[0][k] = q[0];
+            srec[1][k] = q[1];
+            srec[2][k] = q[2];
+            srec[3][k] = q[4];
         }
         __syncthreads();
-        for (int k0 = 0; k0 < cnt; k0 += 16) {
-            // lane l16 of each half tests Gaussian k0 + l16 against the half's footprint
-            const int k = k0 + l16;
-            const bool hit = foot_ok && (k < cnt) && foot_hit(srec[k], cx, cy, cz, G.sqrtTcull);
-            const unsigned bal = __ballot_sync(0xffffffffu, hit);
-            unsigned mask = (bal & half_sel) >> (lane & 16);
-            // each half takes its hits in ascending Gaussian id (per voxel the order of Eq. 3);
-            // the halves run their own trip counts and meet again at the next ballot
-            while (mask) {
-                {
-                    const int kk = k0 + __ffs(mask) - 1;
-                    mask &= mask - 1;
-                    const Rec R = load_rec(srec[kk]);
-                    float dy, dz, Sr, dxs;
-                    row_terms(R, fyz, dy, dz, Sr, dxs);
-                    const float tq0 = tq_base(R, ox, dxs);
-                    const float2 vrr = f2(R.vr, R.r);
+        // each warp lists the hits of its four footprints in ascending Gaussian id
+        int n[4] = {0, 0, 0, 0};
+        for (int k0 = 0; k0 < cnt; k0 += 32) {
+            const int k = k0 + lane;
+            const unsigned m = (k < cnt ? static_cast<unsigned>(sfoot[k]) : 0u) >> foot0;
 #pragma unroll
-                    for (int xi = 0; xi < 4; ++xi) {
-                        const float q = q_of_k(R, tq0, xi, Sr);
-                        if (q <= G.T) {
-                            const float g = ex2_approx(-q);
-                            SW[xi] = fma2(vrr, f2(g, g), SW[xi]);
-                        }
-                        if (kStats) {
-                            n_eff += (y < G.ny && z < G.nz && ox + xi < G.nx && q <= G.T) ? 1 : 0;
-                            n_eval += 1;
-                        }
+            for (int j = 0; j < 4; ++j) {
+                const unsigned bal = __ballot_sync(0xffffffffu, (m >> j) & 1u);
+                if ((m >> j) & 1u)
+                    slist[foot0 + j][n[j] + __popc(bal & ((1u << lane) - 1u))] = static_cast<unsigned char>(k);
+                n[j] += __popc(bal);
+            }
+        }
+        const int myn = (lane & 16) ? ((lane & 8) ? n[3] : n[2]) : ((lane & 8) ? n[1] : n[0]);
+        if (l8 < kFwdHits) slist[foot][myn + l8] = static_cast<unsigned char>(kChunk);
+        __syncwarp();
+        for (int i = 0; i < myn; i += kFwdHits) {
+            const unsigned slots = *reinterpret_cast<const unsigned*>(&slist[foot][i]);
+#pragma unroll
+            for (int u = 0; u < kFwdHits; ++u) {
+                const int kk = (slots >> (8 * u)) & 0xff;
+                const float4 ra = srec[0][kk], rb = srec[1][kk], rc = srec[2][kk], re = srec[3][kk];
+                const float dy = (fy + ra.z) + rb.x;
+                const float2 dz = add2(add2(fz2, f2(ra.w, ra.w)), f2(rb.y, rb.y));
+                const float2 dy2 = f2(dy, dy);
+                const float2 t = fma2(f2(rc.x, rc.x), dy2, mul2(f2(rb.z, rb.z), dz));
+                const float2 dxs = fma2(f2(rc.y, rc.y), dy2, mul2(f2(rb.w, rb.w), dz));
+                const float2 Sr = fma2(dy2, t, mul2(mul2(f2(rc.z, rc.z), dz), dz));
+                const float ux = (float(ox) + ra.x) + ra.y;
+                const float2 sa2 = f2(rc.w, rc.w);
+                const float2 tq0 = mul2(sa2, add2(f2(ux, ux), f2(-dxs.x, -dxs.y)));
+                const float2 vrr = f2(re.x, re.y);
+#pragma unroll
+                for (int xi = 0; xi < 4; ++xi) {
+                    const float2 tq = xi == 0 ? tq0 : fma2(f2(float(xi), float(xi)), sa2, tq0);
+                    const float2 q = fma2(tq, tq, Sr);
+                    if (q.x <= G.T) {
+                        const float g = ex2_approx(-q.x);
+                        SWa[xi] = fma2(vrr, f2(g, g), SWa[xi]);
+                    }
+                    if (q.y <= G.T) {
+                        const float g = ex2_approx(-q.y);
+                        SWb[xi] = fma2(vrr, f2(g, g), SWb[xi]);
+                    }
+                    if (kStats) {
+                        const bool live = i + u < myn;
+                        const bool in = live && y < G.ny && ox + xi < G.nx;
+                        n_eff += (in && z < G.nz && q.x <= G.T) ? 1 : 0;
+                        n_eff += (in && z + 1 < G.nz && q.y <= G.T) ? 1 : 0;
+                        n_eval += live ? 2 : 0;
                     }
                 }
             }
         }
     }
-    if (foot_ok && y < G.ny && z < G.nz) {
-        const int64_t row = (int64_t(z) * G.ny + y) * G.nx + ox;
-        float Iv[4];
 #pragma unroll
-        for (int xi = 0; xi < 4; ++xi) Iv[xi] = SW[xi].x / (SW[xi].y > G.eps ? SW[xi].y : G.eps);
+    for (int h = 0; h < 2; ++h) {
+        if (!(foot_ok && y < G.ny && z + h < G.nz)) continue;
+        const int64_t row = (int64_t(z + h) * G.ny + y) * G.nx + ox;
+        float Iv[4], Wv[4];
+#pragma unroll
+        for (int xi = 0; xi < 4; ++xi) {
+            const float S = h ? SWb[xi].x : SWa[xi].x;
+            Wv[xi] = h ? SWb[xi].y : SWa[xi].y;
+            Iv[xi] = S / (Wv[xi] > G.eps ? Wv[xi] : G.eps);
+        }
         if (ox + 3 < G.nx && (G.nx & 3) == 0) {
             *reinterpret_cast<float4*>(I + row) = make_float4(Iv[0], Iv[1], Iv[2], Iv[3]);
-            *reinterpret_cast<float4*>(W + row) = make_float4(SW[0].y, SW[1].y, SW[2].y, SW[3].y);
+            *reinterpret_cast<float4*>(W + row) = make_float4(Wv[0], Wv[1], Wv[2], Wv[3]);
         } else {
 #pragma unroll
             for (int xi = 0; xi < 4; ++xi)
                 if (ox + xi < G.nx) {
                     I[row + xi] = Iv[xi];
-                    W[row + xi] = SW[xi].y;
+                    W[row + xi] = Wv[xi];
                 }
         }
     }
@@ -382,7 +456,7 @@ __device__ __forceinline__ void adjoint_rows(const Rec& R, unsigned long long m,
         float dy, dz, S, dxs;
         row_terms(R, f2(float(y), float(z)), dy, dz, S, dxs);
         const float2 S2 = f2(S, S), nd2 = f2(-dxs, -dxs);
-        float2 tq0[NT];  // tq_base of each group, the forward's sa * (ux - dx*)
+        float2 tq0[NT];  // tq0 of each group, the forward's sa * (ux - dx*)
 #pragma unroll
         for (int j = 0; j < NT; ++j) tq0[j] = mul2(sa2, add2(uxp[j], nd2));
         const bool row_in = kStaged || ((y < G.ny) && (z < G.nz));
@@ -717,7 +791,7 @@ gs_status render_fwd_impl(const gs_bins* bins, const gs_grid* grid, const gs_con
                           float* I, float* W, unsigned long long* stats, cudaStream_t st) {
     RenderGeo G = make_geo(grid, cfg);
     const int n_foot = G.fx * G.fy * G.fz;
-    const int threads = 32 * ((n_foot + 1) / 2);  // a half-warp per footprint
+    const int threads = 32 * ((n_foot + 3) / 4);  // a quarter-warp per footprint
     // records staged per round about in proportion to the footprints (the lists of smaller
     // bricks are shorter), so that smaller bricks keep more blocks resident
     const float4* rec4 = reinterpret_cast<const float4*>(bins->rec);
