@@ -69,8 +69,8 @@ typedef struct {
  *   trunc_sigma: Mahalanobis truncation radius (3.0: the 3-sigma ellipsoids of Sec. 3.3).
  *   eps: floor of the weight sum in the normalisation of Eq. 3 (the paper gives none).
  *   deterministic: 1 = the backward pass reduces per-Gaussian gradients in a fixed order
- *                  (bit-reproducible, no floating-point atomics); 0 = one float atomic
- *                  per (brick, Gaussian, value).
+ *                  (bit-reproducible, no floating-point atomics); 0 = vector float
+ *                  atomics, three per (brick, Gaussian).
  *   signal_mode: 0 (v = A, r = T) or 1 (v = A T, r = 1).
  *   a_act, t_act: 0 = identity, 1 = sigmoid for A and T. */
 typedef struct {
