@@ -2,22 +2,20 @@
 // per-brick Gaussian lists built by count / exclusive scan / stable radix scatter.
 //
 // Pipeline of gs_bin_bricks (all asynchronous on one stream):
-//   k_preprocess   one thread per Gaussian: validity, FP32 brick range (fixed operation order,
-//                  bit-exact against the oracle's binning specification), render record; it
-//                  also clears the radix passes' two digit-count buffers.
-//   scan           exclusive scan of per-Gaussian pair counts -> gm_off; its last thread stores
-//                  the total as d_npairs and flags GS_STATUS_CAPACITY when it exceeds the
-//                  bins' capacity.
-//   k_emit         Gaussian-major pair emission (brick key, owner), staged per block in shared
-//                  memory so the stores are coalesced.
-//   radix passes   stable LSD radix sort of the brick keys, 8 bits per pass: per-tile digit
-//                  counts (the first pass's added up by k_emit, each later pass's by the
-//                  scatter before it), a digit-major scan, and a stable scatter whose in-tile
-//                  ranks come from warp match masks. Stability keeps ascending Gaussian ids inside
-//                  each brick, so the lists are deterministic.
-//                  The last pass stores pair_brick (key), pair_gmj (Gaussian-major position)
-//                  and pair_gid (owner) directly.
-//   k_brick_off    brick_off from the boundaries of the sorted keys.
+//   k_preprocess    one thread per Gaussian: validity, FP32 brick range (fixed operation order,
+//                   bit-exact against the oracle's binning specification), render record. A block
+//                   also counts its 256 Gaussians' pairs and their first radix digits.
+//   k_row_scan      one block per digit: exclusive scan of the digit's counts over the Gaussian
+//                   tiles; one more block scans the tiles' pair counts, stores d_npairs and the
+//                   status word (GS_STATUS_NONFINITE, GS_STATUS_CAPACITY).
+//   k_radix_scatter (first pass) a block writes gm_off of its Gaussians, emits their pairs into
+//                   shared memory and scatters them by digit: the Gaussian-major pair list never
+//                   goes to memory.
+//   later passes    the same scan and scatter over tiles of 2,048 pairs, whose digit counts the
+//                   scatter before added up. Stability keeps ascending Gaussian ids inside each
+//                   brick, so the lists are deterministic. The last pass stores pair_brick (key),
+//                   pair_gmj (Gaussian-major position) and pair_gid directly.
+//   k_brick_off     brick_off from the boundaries of the sorted keys.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -86,98 +84,6 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* smem, T* total) {
     return prefix;
 }
 
-// Per-block sums (64-bit) of kScanTile consecutive values.
-template <typename Tin>
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const Tin* __restrict__ in, int64_t n,
-                                                              long long* __restrict__ sums) {
-    pdl_enter();
-    __shared__ long long sm[32];
-    const int64_t base = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanItems;
-    long long s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i)
-        if (base + i < n) s += static_cast<long long>(in[base + i]);
-    long long tot;
-    block_exclusive_scan(s, sm, &tot);
-    if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-// Exclusive scan of each block, offset by the block sums before it (nullptr: single block).
-// kRaw: offs holds the raw block sums and each block adds up those before its own (few
-// blocks); otherwise offs is already scanned.
-template <typename Tin, typename Tout, bool kRaw>
-__global__ void __launch_bounds__(kScanThreads) k_scan_down(const Tin* __restrict__ in, Tout* out,
-                                                            int64_t n, const long long* __restrict__ offs,
-                                                            long long* total, CapCheck cc) {
-    pdl_enter();
-    __shared__ long long sm[32];
-    long long boff = 0;
-    if (kRaw) {
-        long long o = 0;
-        for (int k = threadIdx.x; k < static_cast<int>(blockIdx.x); k += kScanThreads) o += offs[k];
-        block_exclusive_scan(o, sm, &boff);
-    }
-    const int64_t base = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanItems;
-    long long vals[kScanItems];
-    long long s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        vals[i] = (base + i < n) ? static_cast<long long>(in[base + i]) : 0;
-        s += vals[i];
-    }
-    long long tot;
-    long long run = block_exclusive_scan(s, sm, &tot);
-    if (kRaw) run += boff;
-    else if (offs) run += offs[blockIdx.x];
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        if (base + i < n) out[base + i] = static_cast<Tout>(run);
-        run += vals[i];
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) {
-        if (total) *total = run;
-        if (cc.npairs) {
-            *cc.npairs = run;
-            if (run > cc.capacity) atomicOr(cc.status, GS_STATUS_CAPACITY);
-        }
-    }
-}
-
-template <typename Tin, typename Tout>
-static gs_status scan_rec(const Tin* in, Tout* out, int64_t n, long long* total, long long* tmp,
-                          int64_t tmp_len, cudaStream_t st, CapCheck cc) {
-    if (n <= 0) return GS_OK;
-    if (n <= kScanTile) {
-        launch_k(k_scan_down<Tin, Tout, false>, dim3(1), dim3(kScanThreads), 0, st, in, out, n,
-            nullptr, total, cc);
-        return last_launch_status();
-    }
-    const int64_t nb = (n + kScanTile - 1) / kScanTile;
-    if (nb + 1 > tmp_len) return GS_ERR_WORKSPACE;
-    long long* sums = tmp;
-    launch_k(k_scan_reduce<Tin>, dim3(static_cast<unsigned>(nb)), dim3(kScanThreads), 0, st, in, n,
-        sums);
-    gs_status s = last_launch_status();
-    if (s != GS_OK) return s;
-    if (nb <= kScanTile) {  // few blocks: each adds up the raw sums before its own
-        launch_k(k_scan_down<Tin, Tout, true>, dim3(static_cast<unsigned>(nb)), dim3(kScanThreads),
-            0, st, in, out, n, sums, total, cc);
-        return last_launch_status();
-    }
-    // Scan the block sums in place (64-bit), recursively.
-    s = scan_rec<long long, long long>(sums, sums, nb, nullptr, tmp + nb + 1, tmp_len - nb - 1, st,
-                                       CapCheck{});
-    if (s != GS_OK) return s;
-    launch_k(k_scan_down<Tin, Tout, false>, dim3(static_cast<unsigned>(nb)), dim3(kScanThreads), 0,
-        st, in, out, n, sums, total, cc);
-    return last_launch_status();
-}
-
-gs_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, long long* total,
-                             long long* tmp, int64_t tmp_len, cudaStream_t stream, CapCheck cc) {
-    return scan_rec<int32_t, int32_t>(in, out, n, total, tmp, tmp_len, stream, cc);
-}
-
 // ============================================================================ preprocess
 
 struct GridF {
@@ -197,24 +103,78 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// Six blocks of 256 per SM (42 registers, a few values spilled to L1) measured faster than
-// four (52 registers, no spills): the kernel is latency-bound on its division and square-root
-// sequences, so the extra resident warps pay more than the spills cost.
-__global__ void __launch_bounds__(256, 6) k_preprocess(const float* __restrict__ params, int64_t N, GridF G,
-                                                    float trunc_sigma, int signal_mode, int a_act,
-                                                    int t_act, float* __restrict__ rec,
-                                                    int32_t* __restrict__ brange,
-                                                    int32_t* __restrict__ gm_cnt,
-                                                    int32_t* __restrict__ status,
-                                                    int32_t* __restrict__ hist_zero,
-                                                    int64_t hist_zero_len) {
-    pdl_enter();
-    const int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g == 0) gm_cnt[N] = 0;  // sentinel: gm_off has N + 1 entries
-    // the digit counts of the first two radix passes are accumulated by k_emit and the first
-    // scatter: start them at zero
-    for (int64_t i = g; i < hist_zero_len; i += int64_t(gridDim.x) * blockDim.x) hist_zero[i] = 0;
-    if (g >= N) return;
+// Box of bricks of one Gaussian: first brick and size along each axis; cnt = 0: no brick.
+struct BrickBox {
+    int lo[3], n[3];
+    int cnt;
+};
+
+// Key of the box's j-th brick (x fastest).
+__device__ __forceinline__ int box_key(const BrickBox& B, int j, int nbx, int nby) {
+    const int r = j / B.n[0], x = j - r * B.n[0];
+    const int z = r / B.n[1], y = r - z * B.n[1];
+    return ((B.lo[2] + z) * nby + B.lo[1] + y) * nbx + B.lo[0] + x;
+}
+
+__device__ __forceinline__ BrickBox box_of_lane(const BrickBox& B, int src) {
+    BrickBox o;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        o.lo[k] = __shfl_sync(0xffffffffu, B.lo[k], src);
+        o.n[k] = __shfl_sync(0xffffffffu, B.n[k], src);
+    }
+    o.cnt = __shfl_sync(0xffffffffu, B.cnt, src);
+    return o;
+}
+
+// f(source lane, off + j, key) for the bricks j in [j0, j1) of each lane's box. A lane walks up to
+// kBoxSerial bricks itself; longer ranges (a Gaussian across much of the volume) are shared by
+// the warp. All lanes of the warp call it, lanes without bricks with j0 >= j1.
+constexpr int kBoxSerial = 64;
+
+template <typename F>
+__device__ __forceinline__ void for_box(const BrickBox& B, int j0, int j1, int off, int nbx, int nby, F f) {
+    const int lane = threadIdx.x & 31;
+    unsigned big = __ballot_sync(0xffffffffu, j1 - j0 > kBoxSerial);
+    if (j1 > j0 && j1 - j0 <= kBoxSerial) {
+        int x = 0, y = 0, z = 0;
+        if (j0 > 0) {
+            const int r = j0 / B.n[0];
+            x = j0 - r * B.n[0];
+            z = r / B.n[1];
+            y = r - z * B.n[1];
+        }
+        int key = ((B.lo[2] + z) * nby + B.lo[1] + y) * nbx + B.lo[0] + x;
+        const int next_row = nbx - B.n[0], next_plane = (nby - B.n[1]) * nbx;
+        for (int j = j0; j < j1; ++j) {
+            f(lane, off + j, key);
+            ++key;
+            if (++x == B.n[0]) {
+                x = 0;
+                key += next_row;
+                if (++y == B.n[1]) {
+                    y = 0;
+                    key += next_plane;
+                }
+            }
+        }
+    }
+    while (big) {
+        const int src = __ffs(big) - 1;
+        big &= big - 1;
+        const BrickBox o = box_of_lane(B, src);
+        const int a = __shfl_sync(0xffffffffu, j0, src), e = __shfl_sync(0xffffffffu, j1, src);
+        const int so = __shfl_sync(0xffffffffu, off, src);
+        for (int j = a + lane; j < e; j += 32) f(src, so + j, box_key(o, j, nbx, nby));
+    }
+}
+
+// Range, record and brick box of Gaussian g; returns false where it is invalid (then it has no
+// brick and a zero record).
+__device__ __forceinline__ bool preprocess_one(const float* __restrict__ params, int64_t g, const GridF& G,
+                                               float trunc_sigma, int signal_mode, int a_act, int t_act,
+                                               float* __restrict__ rec, int32_t* __restrict__ brange,
+                                               BrickBox& box) {
     const float4* p4 = reinterpret_cast<const float4*>(params + g * 12);
     float4 a0 = p4[0], a1 = p4[1], a2 = p4[2];
     float p[12] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w, a2.x, a2.y, a2.z, a2.w};
@@ -235,11 +195,9 @@ __global__ void __launch_bounds__(256, 6) k_preprocess(const float* __restrict__
     if (!ok) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) br[k] = 0;
-        gm_cnt[g] = 0;
 #pragma unroll
         for (int k = 0; k < REC_F4; ++k) r4[k] = z4;
-        atomicOr(status, GS_STATUS_NONFINITE);
-        return;
+        return false;
     }
 
     // ---- binning specification (FP32, explicit rounding, fixed order) ----
@@ -289,25 +247,22 @@ __global__ void __launch_bounds__(256, 6) k_preprocess(const float* __restrict__
             hi[k] = static_cast<int>(hc);
         }
     }
-    int cnt = 0;
     if (inside) {
         int b0[3], b1[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             b0[k] = static_cast<int>(fast_div(static_cast<unsigned>(lo[k]), G.db[k]));
             b1[k] = static_cast<int>(fast_div(static_cast<unsigned>(hi[k]), G.db[k]));
-            br[k] = b0[k];
-            br[3 + k] = b1[k];
+            box.lo[k] = b0[k];
+            box.n[k] = b1[k] - b0[k] + 1;
         }
-        cnt = (b1[0] - b0[0] + 1) * (b1[1] - b0[1] + 1) * (b1[2] - b0[2] + 1);
-        br[B_CNT] = cnt;
-        br[B_VALID] = 1;
+        box.cnt = box.n[0] * box.n[1] * box.n[2];
+        reinterpret_cast<int4*>(br)[0] = make_int4(b0[0], b0[1], b0[2], b1[0]);
+        reinterpret_cast<int4*>(br)[1] = make_int4(b1[1], b1[2], box.cnt, 1);
     } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) br[k] = 0;
-        br[B_VALID] = 1;
+        reinterpret_cast<int4*>(br)[0] = make_int4(0, 0, 0, 0);
+        reinterpret_cast<int4*>(br)[1] = make_int4(0, 0, 0, 1);
     }
-    gm_cnt[g] = cnt;
 
     // ---- render record (accuracy only; contraction allowed) ----
     // M = sqrt(log2 e / 2) diag(1/s) R^T H: row k of M is R[:, k]^T H scaled by sqrt(k)/s_k.
@@ -398,229 +353,418 @@ __global__ void __launch_bounds__(256, 6) k_preprocess(const float* __restrict__
     const float hmin = fminf(G.h[0], fminf(G.h[1], G.h[2]));
     const float lam = kHalfLog2e * (1.0f - 1e-3f) * (hmin / smax) * (hmin / smax);
     r4[4] = make_float4(v * r, r, v, lam);
+    return true;
 }
 
-// ============================================================================ capacity / emit
+constexpr long long kBadFlag = 1LL << 62;  // marks a Gaussian tile with an invalid Gaussian
 
-__global__ void k_capacity(const long long* __restrict__ total, int64_t capacity,
-                           int64_t* __restrict__ npairs, int32_t* __restrict__ status) {
+// Six blocks of 256 per SM (42 registers, a few values spilled to L1) measured faster than
+// four (52 registers, no spills): the kernel is latency-bound on its division and square-root
+// sequences, so the extra resident warps pay more than the spills cost.
+// The block also stores its column of the first radix pass's digit counts (hist0[d * stride0 +
+// block]) and its number of pairs (blk[block]), kBadFlag added where a Gaussian was invalid.
+__global__ void __launch_bounds__(kGaussTile, 6) k_preprocess(
+    const float* __restrict__ params, int64_t N, GridF G, float trunc_sigma, int signal_mode, int a_act,
+    int t_act, float* __restrict__ rec, int32_t* __restrict__ brange, int nd, int32_t* __restrict__ hist0,
+    int64_t stride0, long long* __restrict__ blk) {
     pdl_enter();
-    long long t = *total;
-    *npairs = t;
-    if (t > capacity) atomicOr(status, GS_STATUS_CAPACITY);
+    __shared__ int hcnt[kMaxDigits], hdif[kMaxDigits + 1], sscan[32];
+    __shared__ int hall, flags;  // flags: 1 an invalid Gaussian, 2 a box of more than kBoxSerial bricks
+    __shared__ unsigned long long btot;
+    for (int d = threadIdx.x; d <= nd; d += kGaussTile) {
+        if (d < nd) hcnt[d] = 0;
+        hdif[d] = 0;
+    }
+    if (threadIdx.x == 0) {
+        hall = flags = 0;
+        btot = 0;
+    }
+    __syncthreads();
+    const int64_t g = int64_t(blockIdx.x) * kGaussTile + threadIdx.x;
+    BrickBox box;
+    box.cnt = 0;
+    bool bad = false;
+    if (g < N)
+        bad = !preprocess_one(params, g, G, trunc_sigma, signal_mode, a_act, t_act, rec, brange, box);
+    unsigned long long wsum = static_cast<unsigned>(box.cnt);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0 && wsum != 0) atomicAdd(&btot, wsum);
+    for_box(box, 0, box.cnt <= kBoxSerial ? box.cnt : 0, 0, G.nb[0], G.nb[1],
+            [&](int, int, int key) { atomicAdd(&hcnt[key & (nd - 1)], 1); });
+    // larger boxes by rows of consecutive keys, shared by the warp: a row adds a constant to every
+    // digit and 1 to an interval of digits (as differences), so that a cloud whose pairs will
+    // exceed the capacity costs no more than its rows
+    unsigned big = __ballot_sync(0xffffffffu, box.cnt > kBoxSerial);
+    const int warp_flags = (__any_sync(0xffffffffu, bad) ? 1 : 0) | (big != 0 ? 2 : 0);
+    if (lane == 0 && warp_flags != 0) atomicOr(&flags, warp_flags);
+    while (big) {
+        const int src = __ffs(big) - 1;
+        big &= big - 1;
+        const BrickBox o = box_of_lane(box, src);
+        for (int r = lane; r < o.n[1] * o.n[2]; r += 32) {
+            const int z = r / o.n[1], y = r - z * o.n[1];
+            const int a = (((o.lo[2] + z) * G.nb[1] + o.lo[1] + y) * G.nb[0] + o.lo[0]) & (nd - 1);
+            const int rem = o.n[0] & (nd - 1), e = a + rem;
+            if (o.n[0] >= nd) atomicAdd(&hall, o.n[0] / nd);
+            if (rem) {
+                atomicAdd(&hdif[a], 1);
+                if (e <= nd) {
+                    atomicAdd(&hdif[e], -1);
+                } else {
+                    atomicAdd(&hdif[0], 1);
+                    atomicAdd(&hdif[e - nd], -1);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int di = nd > kGaussTile ? nd / kGaussTile : 1;  // thread t stores digits [t di, (t + 1) di)
+    int run = 0;
+    if (flags & 2) {
+        int v = 0, tot;
+        for (int e = 0; e < di; ++e) v += threadIdx.x * di + e < nd ? hdif[threadIdx.x * di + e] : 0;
+        run = block_exclusive_scan(v, sscan, &tot) + hall;
+    }
+    for (int e = 0; e < di; ++e) {
+        const int d = threadIdx.x * di + e;
+        if (d < nd) {
+            if (flags & 2) run += hdif[d];
+            hist0[d * stride0 + blockIdx.x] = hcnt[d] + run;
+        }
+    }
+    if (threadIdx.x == 0) blk[blockIdx.x] = static_cast<long long>(btot) + ((flags & 1) ? kBadFlag : 0);
 }
+
+// ============================================================================ radix sort
 
 __device__ __forceinline__ int64_t valid_pairs(const int64_t* npairs, int64_t capacity) {
     int64_t P = *npairs;
     return (P > capacity || P < 0) ? 0 : P;
 }
 
-// One block per 256 consecutive Gaussians, whose pairs fill the contiguous Gaussian-major
-// range [gm_off[g0], gm_off[g0 + 256]). When that range fits kEmitStage entries, each thread
-// writes its pairs into shared memory and the block then stores the range with consecutive
-// threads on consecutive addresses; otherwise threads write their pairs straight to global
-// memory. Both paths write the same values. The block also adds its pairs to the first radix
-// pass's digit counts (digit-major, hist[d * n_tiles + tile] over tiles of kSortTile
-// Gaussian-major positions), so that pass needs no counting launch of its own: counted in
-// shared memory when the range meets at most kEmitTiles tiles (then one global atomic per
-// nonzero count), else one global atomic per pair.
-constexpr int kEmitThreads = 256;
-constexpr int kEmitStage = 4096;
-constexpr int kEmitTiles = 4;
+constexpr int kRowThreads = 512;
+constexpr int kRowItems = 4;
 
-__global__ void __launch_bounds__(kEmitThreads) k_emit(const int32_t* __restrict__ brange,
-                                                       const int32_t* __restrict__ gm_off, int64_t N,
-                                                       int nbx, int nby,
-                                                       const int64_t* __restrict__ npairs,
-                                                       int64_t capacity, int32_t* __restrict__ keys,
-                                                       int32_t* __restrict__ gm_gid,
-                                                       int32_t* __restrict__ hist, int n_tiles) {
+struct RowScan {
+    int32_t* hist;       // rows of digit counts, scanned in place (exclusive within a row)
+    int64_t stride;
+    int64_t cols;        // columns in use: fixed (first pass), or from npairs where < 0
+    int32_t* rowtot;     // row totals
+    int32_t* zero;       // the next pass's counts, cleared here (nullptr: last pass)
+    int64_t zero_cols;
+    long long* blk;      // first pass: pairs of each Gaussian tile, scanned by the last block
+    int nd;
+    int64_t* npairs;
+    int64_t capacity;
+    int32_t* status;
+};
+
+// Block d scans row d (digit d's counts over the tiles) and clears row d of the next pass's
+// counts; the scatter adds up the row totals before its digits itself, so a pass's scan is one
+// launch of 3.5 us at 1,954 tiles (a reduction and a down-sweep over all rows took two, 9 us).
+// The first pass's block nd scans the Gaussian tiles' pair counts (64-bit).
+__global__ void __launch_bounds__(kRowThreads) k_row_scan(RowScan A) {
     pdl_enter();
-    __shared__ int32_t skey[kEmitStage];
-    __shared__ int32_t sgid[kEmitStage];
-    __shared__ int32_t hcnt[kEmitTiles * kRadix];
-    if (valid_pairs(npairs, capacity) == 0) return;
-    const int64_t g0 = int64_t(blockIdx.x) * kEmitThreads;
-    const int64_t g = g0 + threadIdx.x;
-    const int64_t gl = min(g0 + kEmitThreads, N);
-    const int base = gm_off[g0];
-    const int total = gm_off[gl] - base;
-    const bool staged = total <= kEmitStage;
-    const int t0 = base / kSortTile;
-    const bool local = total == 0 || (base + total - 1) / kSortTile - t0 < kEmitTiles;  // uniform
-    for (int i = threadIdx.x; i < kEmitTiles * kRadix; i += kEmitThreads) hcnt[i] = 0;
-    __syncthreads();
-    int32_t* kdst = staged ? skey : keys + base;
-    int32_t* gdst = staged ? sgid : gm_gid + base;
-    if (g < N) {
-        const int32_t* br = brange + g * 8;
-        if (br[B_CNT] != 0) {
-            int j = gm_off[g] - base;
-            for (int bz = br[B_LOZ]; bz <= br[B_HIZ]; ++bz)
-                for (int by = br[B_LOY]; by <= br[B_HIY]; ++by)
-                    for (int bx = br[B_LOX]; bx <= br[B_HIX]; ++bx) {
-                        const int key = (bz * nby + by) * nbx + bx;
-                        kdst[j] = key;
-                        gdst[j] = static_cast<int32_t>(g);
-                        if (!staged) {  // (staged ranges are counted as they are stored)
-                            const int t = (base + j) / kSortTile;
-                            if (local)
-                                atomicAdd(&hcnt[(t - t0) * kRadix + (key & (kRadix - 1))], 1);
-                            else
-                                atomicAdd(&hist[int64_t(key & (kRadix - 1)) * n_tiles + t], 1);
-                        }
-                        ++j;
-                    }
-        }
-    }
-    __syncthreads();
-    if (staged) {
-        for (int i = threadIdx.x; i < total; i += kEmitThreads) {
-            const int key = skey[i];
-            keys[base + i] = key;
-            gm_gid[base + i] = sgid[i];
-            atomicAdd(&hcnt[((base + i) / kSortTile - t0) * kRadix + (key & (kRadix - 1))], 1);
+    __shared__ long long sm[32];
+    const int row = blockIdx.x, tid = threadIdx.x;
+    long long carry = 0;
+    if (row == A.nd) {
+        __shared__ int bad;
+        if (tid == 0) bad = 0;
+        __syncthreads();
+        for (int64_t c0 = 0; c0 < A.cols; c0 += kRowThreads) {
+            const int64_t c = c0 + tid;
+            long long v = c < A.cols ? A.blk[c] : 0;
+            if (v >= kBadFlag) {
+                v -= kBadFlag;
+                bad = 1;
+            }
+            long long tot;
+            const long long pre = block_exclusive_scan(v, sm, &tot);
+            if (c < A.cols) A.blk[c] = carry + pre;
+            carry += tot;
         }
         __syncthreads();
-    }
-    if (local) {
-        for (int i = threadIdx.x; i < kEmitTiles * kRadix; i += kEmitThreads) {
-            const int c = hcnt[i];
-            if (c != 0) atomicAdd(&hist[int64_t(i % kRadix) * n_tiles + t0 + i / kRadix], c);
+        if (tid == 0) {
+            A.blk[A.cols] = carry;
+            *A.npairs = carry;
+            *A.status = (bad ? GS_STATUS_NONFINITE : 0) | (carry > A.capacity ? GS_STATUS_CAPACITY : 0);
         }
+        return;
     }
+    const int64_t cols = A.cols >= 0 ? A.cols : (valid_pairs(A.npairs, A.capacity) + kSortTile - 1) / kSortTile;
+    int32_t* h = A.hist + row * A.stride;
+    for (int64_t c0 = 0; c0 < cols; c0 += kRowThreads * kRowItems) {
+        const int64_t c = c0 + int64_t(tid) * kRowItems;
+        // (the stride is a multiple of 4, so a 16-byte piece that starts inside the row is whole)
+        int4 v = c < cols ? *reinterpret_cast<const int4*>(h + c) : make_int4(0, 0, 0, 0);
+        if (c + 1 >= cols) v.y = 0;
+        if (c + 2 >= cols) v.z = 0;
+        if (c + 3 >= cols) v.w = 0;
+        long long tot;
+        const int s = v.x + v.y + v.z + v.w;
+        const int pre = static_cast<int>(carry + block_exclusive_scan<long long>(s, sm, &tot));
+        if (c < cols)
+            *reinterpret_cast<int4*>(h + c) = make_int4(pre, pre + v.x, pre + v.x + v.y, pre + v.x + v.y + v.z);
+        carry += tot;
+    }
+    if (tid == 0) A.rowtot[row] = static_cast<int>(carry);
+    if (A.zero)
+        for (int64_t c = int64_t(tid) * 4; c < A.zero_cols; c += kRowThreads * 4)
+            *reinterpret_cast<int4*>(A.zero + row * A.zero_cols + c) = make_int4(0, 0, 0, 0);
 }
 
-// ============================================================================ radix sort
+struct Scatter {
+    const int32_t* keys_in;    // pass input (not the first pass)
+    const int2* vals_in;       // (Gaussian-major position, Gaussian id)
+    int32_t* keys_out;         // the last pass: pair_brick
+    int2* vals_out;            // (not the last pass)
+    int32_t* out_gmj;          // last pass
+    int32_t* out_gid;
+    const int32_t* hist;       // this pass's scanned counts
+    int64_t stride;
+    const int32_t* rowtot;
+    int32_t* hist_next;        // the next pass's counts (not the last pass)
+    int64_t stride_next;
+    int shift, bits;
+    const int64_t* npairs;
+    int64_t capacity;
+    const int32_t* brange;     // first pass: emission
+    int32_t* gm_off;
+    const long long* blk_base;
+    int64_t N;
+    int nbx, nby;
+};
 
-// Stable scatter of one tile of kSortTile keys. Warp w owns the contiguous sub-tile
-// [w * 256, (w + 1) * 256) and visits it in 8 rounds of 32 consecutive keys (kept in
-// registers; with the digit counts accumulated by the launch before, 2,048-key tiles measured
-// faster than 1,024, 1,536, 2,560 and 3,072 at the fitting size). Pass 1 counts each warp's
-// digits. A block-wide prefix then gives, per digit,
-// the tile-local start of its run and each warp's start inside it. Pass 2 places every key in
-// shared memory at its warp's start + its rank among equal digits in lower lanes (warp match
-// masks), so the tile sits in shared memory sorted by digit, ties in tile order. The tile is
-// then written out in that order: digit d's run goes to [hist_off[d][tile], ...), so
-// consecutive threads store consecutive addresses.
-// kLast: the last pass stores the bins' per-pair arrays directly: brick (the key),
-// Gaussian-major position (the value) and owner (gm_gid of the value). Every other pass adds
-// each key to the next pass's digit counts at its output position's tile (one atomic per
-// group of equal (tile, digit) in a warp), so no pass after the first needs a counting launch.
+// Stable scatter of one tile of up to kSortTile keys per round. Warp w owns a contiguous part of
+// the tile and visits it in rounds of 32 consecutive keys, kept in registers with their ranks
+// among the warp's earlier equal digits (warp match masks). A block-wide prefix over the digits
+// then gives each digit's run inside the tile and each warp's start in it; the tile is placed in
+// shared memory sorted by digit, ties in tile order, and written out in that order, so consecutive
+// threads store consecutive addresses of a run.
+// kFirst: the tile is emitted by the block itself from its kGaussTile Gaussians' boxes (in rounds
+// of kSortTile pairs; the digits' output positions advance from round to round), else it is one
+// tile of the previous pass's output. kLast: the pass stores the bins' per-pair arrays; every
+// other pass adds each key to the next pass's digit counts at its output position's tile (one
+// atomic per group of equal (tile, digit) in a warp).
+// Bound by latency (barriers, the gathered loads) at 40-65 % issue-active, far from bandwidth: the
+// pair list is cache-resident at the fitting size. Whole binning, L2 flushed, at 3.26M pairs
+// (256 x 256 x 128 grid, 8^3 bricks): 115 us with the pair list emitted to memory, two scan launches
+// per list and the owners gathered in the last pass; 90 us now (preprocess 23, first pass 32, last
+// pass 20, scans 7, offsets 6). 104M pairs (512 x 512 x 256, two 9-bit passes where 8-bit digits took
+// three): 5.86 -> 3.01 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed
+// by a second match per key and the values held in registers (80 registers) 108 us; the
+// values loaded when the tile is placed 90 us and 3.17 ms; copied to shared memory
+// asynchronously during the ranking (here) 90 us and 3.01 ms; 5 (6) blocks per SM with spills 95
+// (97) us.
 template <bool kFirst, bool kLast>
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
-    const int32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in,
-    int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out,
-    const int32_t* __restrict__ hist_off, const int64_t* __restrict__ npairs, int64_t capacity,
-    int shift, int n_tiles, const int32_t* __restrict__ gm_gid, int32_t* __restrict__ pair_gid,
-    int32_t* __restrict__ hist_next) {
+__global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
     pdl_enter();
     constexpr int kWarps = kSortThreads / 32;
-    constexpr int kPerWarp = kSortTile / kWarps;
-    constexpr int kRounds = kPerWarp / 32;
-    static_assert(kSortThreads == kRadix, "one thread per digit in the block-wide prefix");
-    __shared__ int wcnt[kWarps][kRadix];
-    __shared__ int dstart[kRadix];   // tile-local start of each digit's run
-    __shared__ int gstart[kRadix];   // global start of each digit's run for this tile
-    __shared__ int wsum[kWarps];
+    static_assert(kSortThreads == kGaussTile, "one thread per Gaussian of a tile");
+    extern __shared__ int smem[];
+    const int nd = 1 << A.bits, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int* wcnt = smem;                 // [kWarps][nd]
+    int* goff = wcnt + kWarps * nd;   // output position of tile slot j of digit d: goff[d] + j
     __shared__ int skey[kSortTile];
-    __shared__ int sval[kSortTile];
-    const int64_t P = valid_pairs(npairs, capacity);
-    const int64_t tile0 = int64_t(blockIdx.x) * kSortTile;
-    if (tile0 >= P) return;  // past the last pair: nothing to place
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int d = tid; d < kRadix; d += kSortThreads)
-        for (int w = 0; w < kWarps; ++w) wcnt[w][d] = 0;
-    __syncthreads();
-    const int64_t sub0 = tile0 + int64_t(warp) * kPerWarp;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    int kr[kRounds], vr[kRounds];
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const int64_t idx = sub0 + r * 32 + lane;
-        const bool valid = idx < P;
-        kr[r] = valid ? keys_in[idx] : 0;
-        vr[r] = valid ? (kFirst ? static_cast<int>(idx) : vals_in[idx]) : 0;
-        const int d = (kr[r] >> shift) & (kRadix - 1);
-        const unsigned tag = valid ? static_cast<unsigned>(d) : static_cast<unsigned>(kRadix + lane);
-        const unsigned peers = __match_any_sync(0xffffffffu, tag);
-        if (valid && lane == __ffs(peers) - 1) wcnt[warp][d] += __popc(peers);
-        __syncwarp();
-    }
-    __syncthreads();
-    // thread d: warps' starts inside digit d's run, and the run's length
-    const int d = tid;
-    int run = 0;
-    for (int w = 0; w < kWarps; ++w) {
-        const int c = wcnt[w][d];
-        wcnt[w][d] = run;
-        run += c;
-    }
-    // exclusive prefix of the run lengths over digits (block scan, digit order)
-    int incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    int before = 0;
-    for (int w = 0; w < warp; ++w) before += wsum[w];
-    const int start = before + incl - run;
-    dstart[d] = start;
-    gstart[d] = hist_off[int64_t(d) * n_tiles + blockIdx.x];
-    for (int w = 0; w < kWarps; ++w) wcnt[w][d] += start;
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const int64_t idx = sub0 + r * 32 + lane;
-        const bool valid = idx < P;
-        const int dk = (kr[r] >> shift) & (kRadix - 1);
-        const unsigned tag = valid ? static_cast<unsigned>(dk) : static_cast<unsigned>(kRadix + lane);
-        const unsigned peers = __match_any_sync(0xffffffffu, tag);
-        if (valid) {
-            const int lp = wcnt[warp][dk] + __popc(peers & lt_mask);
-            skey[lp] = kr[r];
-            sval[lp] = vr[r];
+    __shared__ unsigned short sidx[kSortTile];          // sorted: tile index of each key
+    __shared__ unsigned char sowner[kFirst ? kSortTile : 1];  // tile order: Gaussian of the block
+    __shared__ int2 sval[kFirst ? 1 : kSortTile];       // tile order: the keys' values
+    __shared__ long long sscan[32];
+
+    const int64_t P = valid_pairs(A.npairs, A.capacity);
+    int64_t base = int64_t(blockIdx.x) * kSortTile;  // first pair (Gaussian-major in the first pass)
+    int total;                                       // pairs of this block
+    BrickBox box;
+    box.cnt = 0;
+    int loc = 0;                                     // the thread's first pair in the block
+    int gpos[kMaxDigits / kSortThreads] = {};        // the thread's digits' next output positions
+    if (kFirst) {
+        const int64_t g = int64_t(blockIdx.x) * kGaussTile + tid;
+        if (g < A.N) {
+            const int4 lo = reinterpret_cast<const int4*>(A.brange + g * 8)[0];
+            const int4 hi = reinterpret_cast<const int4*>(A.brange + g * 8)[1];
+            box.lo[0] = lo.x; box.lo[1] = lo.y; box.lo[2] = lo.z;
+            box.n[0] = lo.w - lo.x + 1; box.n[1] = hi.x - lo.y + 1; box.n[2] = hi.y - lo.z + 1;
+            box.cnt = hi.z;
         }
-        __syncwarp();
-        if (valid && lane == __ffs(peers) - 1) wcnt[warp][dk] += __popc(peers);
-        __syncwarp();
+        base = A.blk_base[blockIdx.x];
+        // (offsets modulo 2^32: exact where the pairs fit the capacity, which is below 2^31)
+        unsigned tot;
+        const unsigned pre = block_exclusive_scan(static_cast<unsigned>(box.cnt),
+                                                  reinterpret_cast<unsigned*>(sscan), &tot);
+        if (g < A.N) A.gm_off[g] = static_cast<int32_t>(static_cast<unsigned>(base) + pre);
+        if (g == A.N - 1) A.gm_off[A.N] = static_cast<int32_t>(static_cast<unsigned>(base) + pre + box.cnt);
+        if (P == 0) return;  // also when the pairs exceed the capacity
+        loc = static_cast<int>(pre);
+        total = static_cast<int>(tot);
+    } else {
+        if (base >= P) return;  // past the last pair: nothing to place
+        total = static_cast<int>(min(int64_t(kSortTile), P - base));
     }
-    __syncthreads();
-    const int n_here = static_cast<int>(min(int64_t(kSortTile), P - tile0));
-    for (int j = tid; j < n_here; j += kSortThreads) {
-        const int key = skey[j];
-        const int dk = (key >> shift) & (kRadix - 1);
-        const int pos = gstart[dk] + (j - dstart[dk]);
-        keys_out[pos] = key;
-        vals_out[pos] = sval[j];
-        if (kLast) {
-            pair_gid[pos] = gm_gid[sval[j]];
-        } else {
-            const int tag = ((pos / kSortTile) << kRadixBits) | ((key >> (shift + kRadixBits)) & (kRadix - 1));
-            const unsigned peers = __match_any_sync(__activemask(), tag);
-            if (lane == __ffs(peers) - 1)
-                atomicAdd(&hist_next[int64_t(tag & (kRadix - 1)) * n_tiles + (tag >> kRadixBits)],
-                          __popc(peers));
+    for (int c0 = 0; c0 < total; c0 += kSortTile) {
+        const int n = min(kSortTile, total - c0);
+        if (kFirst) {
+            if (c0 > 0) __syncthreads();  // the previous round has been written out
+            for_box(box, max(0, c0 - loc), min(box.cnt, c0 + n - loc), loc - c0, A.nbx, A.nby,
+                    [&](int src, int o, int key) {
+                        skey[o] = key;
+                        sowner[o] = static_cast<unsigned char>(warp * 32 + src);
+                    });
+        }
+        for (int d = tid; d < kWarps * nd; d += kSortThreads) wcnt[d] = 0;
+        __syncthreads();
+        // each warp's part: the same number of 32-key rounds
+        const int rounds = (n + kSortThreads - 1) / kSortThreads;
+        const int sub0 = warp * rounds * 32;
+        int kr[kSortItems];
+        unsigned short rank[kSortItems];
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) {
+            const int idx = sub0 + r * 32 + lane;
+            kr[r] = 0;
+            if (idx < n && r < rounds) {
+                kr[r] = kFirst ? skey[idx] : A.keys_in[base + idx];
+                if (!kFirst)  // read again only when the sorted tile is written out
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                                     static_cast<unsigned>(__cvta_generic_to_shared(&sval[idx]))),
+                                 "l"(A.vals_in + base + idx)
+                                 : "memory");
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) {
+            if (r < rounds) {
+                const bool valid = sub0 + r * 32 + lane < n;
+                const int d = (kr[r] >> A.shift) & (nd - 1);
+                const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : nd + lane);
+                int* w = &wcnt[warp * nd + d];
+                const int before = valid ? *w : 0;
+                __syncwarp();
+                if (valid && lane == __ffs(peers) - 1) *w = before + __popc(peers);
+                __syncwarp();
+                rank[r] = static_cast<unsigned short>(before + __popc(peers & ((1u << lane) - 1u)));
+            }
+        }
+        __syncthreads();
+        // digit runs: thread t owns digits [t di, (t + 1) di)
+        const int di = nd > kSortThreads ? nd / kSortThreads : 1;
+        long long mine = 0;
+        int runs[kMaxDigits / kSortThreads], rows[kMaxDigits / kSortThreads];
+#pragma unroll
+        for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
+            runs[e] = rows[e] = 0;
+            const int d = tid * di + e;
+            if (e < di && d < nd) {
+                int run = 0;
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    const int c = wcnt[w * nd + d];
+                    wcnt[w * nd + d] = run;
+                    run += c;
+                }
+                runs[e] = run;
+                if (c0 == 0) rows[e] = A.rowtot[d];
+            }
+            mine += (static_cast<long long>(rows[e]) << 13) | runs[e];  // (sums of runs: <= 2,048)
+        }
+        long long all;
+        const long long pre = block_exclusive_scan(mine, sscan, &all);
+        int start = static_cast<int>(pre & 8191);
+        int64_t row0 = pre >> 13;
+#pragma unroll
+        for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
+            const int d = tid * di + e;
+            if (e < di && d < nd) {
+                if (c0 == 0) gpos[e] = static_cast<int>(row0) + A.hist[d * A.stride + blockIdx.x];
+                goff[d] = gpos[e] - start;
+                gpos[e] += runs[e];
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) wcnt[w * nd + d] += start;
+                row0 += rows[e];
+                start += runs[e];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) {
+            const int idx = sub0 + r * 32 + lane;
+            if (r < rounds && idx < n) {
+                const int lp = wcnt[warp * nd + ((kr[r] >> A.shift) & (nd - 1))] + rank[r];
+                skey[lp] = kr[r];
+                sidx[lp] = static_cast<unsigned short>(idx);
+            }
+        }
+        if (!kFirst) asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        for (int j = tid; j < n; j += kSortThreads) {
+            const int key = skey[j];
+            const int idx = sidx[j];
+            const int2 v = kFirst ? make_int2(static_cast<int>(base) + c0 + idx,
+                                              static_cast<int>(blockIdx.x) * kGaussTile + sowner[idx])
+                                  : sval[idx];
+            const int pos = goff[(key >> A.shift) & (nd - 1)] + j;
+            A.keys_out[pos] = key;
+            if (kLast) {
+                A.out_gmj[pos] = v.x;
+                A.out_gid[pos] = v.y;
+            } else {
+                A.vals_out[pos] = v;
+                const int tile = pos / kSortTile, dn = (key >> (A.shift + A.bits)) & (nd - 1);
+                const unsigned peers = __match_any_sync(__activemask(), (tile << A.bits) | dn);
+                if (lane == __ffs(peers) - 1)
+                    atomicAdd(&A.hist_next[dn * A.stride_next + tile], __popc(peers));
+            }
         }
     }
 }
 
 // brick_off from the boundaries of the sorted keys (brick_off[b] = first pair of brick b, or
-// the next non-empty brick's first pair; brick_off[nb] = P).
+// the next non-empty brick's first pair; brick_off[nb] = P). Four consecutive keys per thread; runs
+// of empty bricks longer than kGapSerial are filled by the whole warp. (One key per thread with
+// its predecessor loaded beside it, and gaps filled by one thread, took 600 us at 104M pairs and
+// 131,072 bricks.)
+constexpr int kGapSerial = 8;
+
 __global__ void __launch_bounds__(256) k_brick_off(const int32_t* __restrict__ keys,
                                                    const int64_t* __restrict__ npairs,
                                                    int64_t capacity, int nb,
                                                    int32_t* __restrict__ brick_off) {
     pdl_enter();
     const int64_t P = valid_pairs(npairs, capacity);
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i <= P;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const int cur = (i < P) ? keys[i] : nb;
-        const int prev = (i > 0) ? keys[i - 1] : -1;
-        for (int bb = prev + 1; bb <= cur; ++bb) brick_off[bb] = static_cast<int32_t>(i);
+    const int lane = threadIdx.x & 31;
+    const int64_t step = int64_t(gridDim.x) * blockDim.x;
+    // entry i <= P: key i, and the sentinel key nb at i = P
+    for (int64_t q0 = int64_t(blockIdx.x) * blockDim.x + (threadIdx.x & ~31); 4 * q0 <= P; q0 += step) {
+        const int64_t i = 4 * (q0 + lane);
+        int4 k = make_int4(nb, nb, nb, nb);
+        if (i + 3 < P) {
+            k = *reinterpret_cast<const int4*>(keys + i);
+        } else {
+            if (i < P) k.x = keys[i];
+            if (i + 1 < P) k.y = keys[i + 1];
+            if (i + 2 < P) k.z = keys[i + 2];
+        }
+        int prev = __shfl_up_sync(0xffffffffu, k.w, 1);
+        if (lane == 0) prev = i > 0 ? keys[i - 1] : -1;
+        const int cur[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int gap = i + e <= P ? cur[e] - prev : 0;
+            if (gap <= kGapSerial)
+                for (int b = prev + 1; b <= prev + gap; ++b) brick_off[b] = static_cast<int32_t>(i + e);
+            unsigned big = __ballot_sync(0xffffffffu, gap > kGapSerial);
+            while (big) {
+                const int src = __ffs(big) - 1;
+                big &= big - 1;
+                const int b0 = __shfl_sync(0xffffffffu, prev, src), g = __shfl_sync(0xffffffffu, gap, src);
+                const int v = static_cast<int>(4 * (q0 + src) + e);
+                for (int b = lane + 1; b <= g; b += 32) brick_off[b0 + b] = v;
+            }
+            prev = cur[e];
+        }
     }
 }
 
@@ -744,13 +888,6 @@ bool bins_match(const gs_bins* b, const gs_grid* grid, const gs_config* cfg) {
            b->capacity <= kMaxCapacity && b->n_gauss >= 0;
 }
 
-static int radix_passes(int32_t n_bricks) {
-    int bits = 0;
-    while ((int64_t(1) << bits) < n_bricks) ++bits;
-    int passes = (bits + kRadixBits - 1) / kRadixBits;
-    return passes < 1 ? 1 : passes;
-}
-
 gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_config* cfg,
                           gs_bins* bins, const Workspace& ws, cudaStream_t st) {
     const int64_t N = bins->n_gauss;
@@ -767,81 +904,79 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
     G.nb[0] = b.nbx; G.nb[1] = b.nby; G.nb[2] = b.nbz;
     for (int k = 0; k < 3; ++k) G.db[k] = make_fastdiv(static_cast<unsigned>(G.b[k]));
 
-    if (cudaMemsetAsync(bins->d_status, 0, sizeof(int32_t), st) != cudaSuccess) return GS_ERR_CUDA;
-    long long* total = ws.scan_tmp + ws.scan_tmp_len - 1;
-    if (N > 0) {
-        const unsigned gb = static_cast<unsigned>((N + 255) / 256);
-        launch_k(k_preprocess, dim3(gb), dim3(256), 0, st, params, N, G, cfg->trunc_sigma,
-            cfg->signal_mode, cfg->a_act, cfg->t_act, bins->rec, bins->brange, ws.gm_cnt,
-            bins->d_status, ws.hist, 2 * (int64_t(kRadix) * ws.n_tiles + 1));
-        gs_status s = last_launch_status();
-        if (s != GS_OK) return s;
-        // gm_off = exclusive scan of counts (N + 1 entries; gm_cnt[N] = 0 sentinel); the scan's
-        // last thread also stores the total as d_npairs and flags an overflow of the capacity.
-        const CapCheck cc{cap, bins->d_npairs, bins->d_status};
-        s = exclusive_scan_i32(ws.gm_cnt, bins->gm_off, N + 1, total, ws.scan_tmp,
-                               ws.scan_tmp_len - 1, st, cc);
-        if (s != GS_OK) return s;
-    } else {
-        if (cudaMemsetAsync(total, 0, sizeof(long long), st) != cudaSuccess) return GS_ERR_CUDA;
-        if (cudaMemsetAsync(bins->gm_off, 0, sizeof(int32_t), st) != cudaSuccess) return GS_ERR_CUDA;
-        launch_k(k_capacity, dim3(1), dim3(1), 0, st, total, cap, bins->d_npairs, bins->d_status);
-        const gs_status s = last_launch_status();
-        if (s != GS_OK) return s;
-    }
-    gs_status s = GS_OK;
-    if (N > 0) {
-        launch_k(k_emit, dim3(static_cast<unsigned>((N + kEmitThreads - 1) / kEmitThreads)),
-            dim3(kEmitThreads), 0, st, bins->brange, bins->gm_off, N, b.nbx, b.nby, bins->d_npairs,
-            cap, ws.keys0, ws.gm_gid, ws.hist, ws.n_tiles);
-        s = last_launch_status();
-        if (s != GS_OK) return s;
-    }
-    if (cap == 0) {
-        if (cudaMemsetAsync(bins->brick_off, 0, sizeof(int32_t) * (int64_t(bins->n_bricks) + 1), st) !=
-            cudaSuccess)
+    const int64_t off_bytes = sizeof(int32_t) * (int64_t(bins->n_bricks) + 1);
+    if (N == 0) {
+        if (cudaMemsetAsync(bins->d_status, 0, sizeof(int32_t), st) != cudaSuccess ||
+            cudaMemsetAsync(bins->d_npairs, 0, sizeof(int64_t), st) != cudaSuccess ||
+            cudaMemsetAsync(bins->gm_off, 0, sizeof(int32_t), st) != cudaSuccess ||
+            cudaMemsetAsync(bins->brick_off, 0, off_bytes, st) != cudaSuccess)
             return GS_ERR_CUDA;
         return GS_OK;
     }
-
-    // Stable LSD radix sort of brick keys; values are Gaussian-major positions.
-    const int passes = radix_passes(bins->n_bricks);
-    int32_t* kin = ws.keys0;
-    int32_t* vin = ws.vals0;
-    int32_t* kout = ws.keys1;
-    int32_t* vout = ws.vals1;
-    const int nt = ws.n_tiles;
-    const int64_t hist_len = int64_t(kRadix) * nt;
-    // digit counts: pass 0's from k_emit, pass p + 1's from pass p's scatter, in two buffers
-    // that k_preprocess zeroed; a third pass reuses the first buffer, zeroed again here
-    int32_t* hbuf[2] = {ws.hist, ws.hist1};
+    const int nd = 1 << ws.radix_bits, passes = ws.radix_passes;
+    const unsigned gb = static_cast<unsigned>((N + kGaussTile - 1) / kGaussTile);
+    launch_k(k_preprocess, dim3(gb), dim3(kGaussTile), 0, st, params, N, G, cfg->trunc_sigma,
+        cfg->signal_mode, cfg->a_act, cfg->t_act, bins->rec, bins->brange, nd, ws.hist0, ws.stride0,
+        ws.blk_base);
+    gs_status s = last_launch_status();
+    if (s != GS_OK) return s;
+    const size_t smem = sizeof(int) * (kSortThreads / 32 + 1) * nd;
+    const unsigned tiles = static_cast<unsigned>((cap + kSortTile - 1) / kSortTile);
     for (int pass = 0; pass < passes; ++pass) {
-        const int shift = pass * kRadixBits;
-        int32_t* hcur = hbuf[pass & 1];
-        int32_t* hnext = hbuf[(pass + 1) & 1];
-        if (pass >= 1 && pass + 1 < passes &&
-            cudaMemsetAsync(hnext, 0, sizeof(int32_t) * hist_len, st) != cudaSuccess)
-            return GS_ERR_CUDA;
-        s = exclusive_scan_i32(hcur, hcur, hist_len, nullptr, ws.scan_tmp, ws.scan_tmp_len - 1, st);
-        if (s != GS_OK) return s;
-        // the last pass writes the bins' pair arrays (brick, Gaussian-major position, owner)
-        const bool last = pass == passes - 1;
-        int32_t* ko = last ? bins->pair_brick : kout;
-        int32_t* vo = last ? bins->pair_gmj : vout;
-        using ScatterFn = void (*)(const int32_t*, const int32_t*, int32_t*, int32_t*, const int32_t*,
-                                   const int64_t*, int64_t, int, int, const int32_t*, int32_t*,
-                                   int32_t*);
-        ScatterFn kern = pass == 0 ? (last ? k_radix_scatter<true, true> : k_radix_scatter<true, false>)
-                                   : (last ? k_radix_scatter<false, true> : k_radix_scatter<false, false>);
-        launch_k(kern, dim3(nt), dim3(kSortThreads), 0, st, kin, vin, ko, vo, hcur,
-            bins->d_npairs, cap, shift, nt, ws.gm_gid, bins->pair_gid, hnext);
+        const bool first = pass == 0, last = pass == passes - 1;
+        const int cur = (pass + 1) & 1;  // later passes alternate: pass 1 reads buffers 0, pass 2 buffers 1
+        const int nxt = pass & 1;
+        RowScan R = {};
+        R.hist = first ? ws.hist0 : ws.hist[cur];
+        R.stride = first ? ws.stride0 : ws.stride1;
+        R.cols = first ? int64_t(gb) : -1;
+        R.rowtot = ws.rowtot;
+        R.zero = last ? nullptr : ws.hist[nxt];
+        R.zero_cols = ws.stride1;
+        R.blk = ws.blk_base;
+        R.nd = nd;
+        R.npairs = bins->d_npairs;
+        R.capacity = cap;
+        R.status = bins->d_status;
+        launch_k(k_row_scan, dim3(nd + (first ? 1 : 0)), dim3(kRowThreads), 0, st, R);
         s = last_launch_status();
         if (s != GS_OK) return s;
-        int32_t* t = kin; kin = kout; kout = t;
-        t = vin; vin = vout; vout = t;
+        Scatter A = {};
+        A.keys_in = first ? nullptr : ws.keys[cur];
+        A.vals_in = first ? nullptr : ws.vals[cur];
+        A.keys_out = last ? bins->pair_brick : ws.keys[nxt];
+        A.vals_out = last ? nullptr : ws.vals[nxt];
+        A.out_gmj = bins->pair_gmj;
+        A.out_gid = bins->pair_gid;
+        A.hist = R.hist;
+        A.stride = R.stride;
+        A.rowtot = ws.rowtot;
+        A.hist_next = R.zero;
+        A.stride_next = ws.stride1;
+        A.shift = pass * ws.radix_bits;
+        A.bits = ws.radix_bits;
+        A.npairs = bins->d_npairs;
+        A.capacity = cap;
+        A.brange = bins->brange;
+        A.gm_off = bins->gm_off;
+        A.blk_base = ws.blk_base;
+        A.N = N;
+        A.nbx = b.nbx;
+        A.nby = b.nby;
+        void (*kern)(Scatter) = first ? (last ? k_radix_scatter<true, true> : k_radix_scatter<true, false>)
+                                      : (last ? k_radix_scatter<false, true> : k_radix_scatter<false, false>);
+        if (first || tiles > 0) {
+            launch_k(kern, dim3(first ? gb : tiles), dim3(kSortThreads), smem, st, A);
+            s = last_launch_status();
+            if (s != GS_OK) return s;
+        }
     }
-    launch_k(k_brick_off, dim3(1184), dim3(256), 0, st, bins->pair_brick, bins->d_npairs, cap,
-        bins->n_bricks, bins->brick_off);
+    if (cap == 0)
+        return cudaMemsetAsync(bins->brick_off, 0, off_bytes, st) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
+    // enough threads for four keys each, at most eight blocks per SM
+    const int64_t ob = (cap / 4 + 256) / 256;
+    launch_k(k_brick_off, dim3(static_cast<unsigned>(ob < 152 * 8 ? ob : 152 * 8)), dim3(256), 0, st,
+        bins->pair_brick, bins->d_npairs, cap, bins->n_bricks, bins->brick_off);
     return last_launch_status();
 }
 

@@ -72,12 +72,9 @@ enum BrangeField : int { B_LOX = 0, B_LOY, B_LOZ, B_HIX, B_HIY, B_HIZ, B_CNT, B_
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
-constexpr int kRadixBits = 8;
-constexpr int kRadix = 1 << kRadixBits;
-
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;  // 1024 values per block
+constexpr int kMaxRadixBits = 9;
+constexpr int kMaxDigits = 1 << kMaxRadixBits;
+constexpr int kGaussTile = 256;   // Gaussians per block of the preprocess and emission kernels
 
 constexpr int kL1Blocks = 1024;  // fixed block count of the L1 reduction (deterministic)
 
@@ -85,35 +82,33 @@ constexpr int64_t kMaxCapacity = (int64_t(1) << 31) - 4096;
 
 // ------------------------------------------------------------------ workspace layout
 struct Workspace {
-    int32_t* keys0;
-    int32_t* vals0;
-    int32_t* keys1;
-    int32_t* vals1;
-    int32_t* gm_gid;
-    int32_t* gm_cnt;
-    int32_t* hist;           // digit counts / offsets of the radix passes: two buffers
-    int32_t* hist1;          // of hist_len + 1, contiguous (hist1 = hist + hist_len + 1)
-    long long* scan_tmp;     // block sums of the multi-level scan
+    int32_t* keys[2];        // brick keys between the radix passes; the second of each pair is
+    int2* vals[2];           // bound for three passes and more. vals: (Gaussian-major position, id)
+    int32_t* hist0;          // first pass's digit counts: one row per digit, a column per
+                             // kGaussTile Gaussians (row stride stride0)
+    int32_t* hist[2];        // later passes': a column per kSortTile pairs (row stride stride1)
+    int32_t* rowtot;         // [kMaxDigits] totals of the digits of the pass being scanned
+    long long* blk_base;     // [Gaussian tiles + 1] pairs of each tile, then their exclusive sums
+    int64_t stride0, stride1;
+    int32_t radix_bits, radix_passes;
     float* part;             // [capacity, 12] per-pair partial gradients (deterministic mode)
     float* gacc;             // [n_gauss, 12] render-space gradient per Gaussian
     float2* aip;             // [n_voxels] (alpha, alpha I'), alpha = dL/dI / max(W, eps)
     float* l1_part;          // [kL1Blocks]
-    int64_t scan_tmp_len;
-    int32_t n_tiles;
     size_t bytes;
 };
 
-inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
-inline int64_t scan_tmp_len_for(int64_t n) {
-    // Space for every level of the recursive block-sum scan of n values.
-    int64_t total = 0;
-    while (n > kScanTile) {
-        n = (n + kScanTile - 1) / kScanTile;
-        total += n + 1;
-    }
-    return total + 8;
+// Stable LSD radix sort of the brick keys: as few passes of at most kMaxRadixBits bits as the
+// keys need, with equal digit widths (16,384 bricks: 2 x 7 bits; 131,072: 2 x 9; 524,288: 3 x 7).
+// Narrow digits give longer runs per tile and digit, and fewer count rows to scan.
+inline void radix_plan(int32_t n_bricks, int32_t* passes, int32_t* bits) {
+    int need = 1;
+    while ((int64_t(1) << need) < n_bricks) ++need;
+    *passes = (need + kMaxRadixBits - 1) / kMaxRadixBits;
+    *bits = (need + *passes - 1) / *passes;
 }
+
+inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Carve (or size, if base == nullptr) the workspace. Returns false on overflow.
 inline bool carve_workspace(void* base, int64_t n_gauss, int64_t capacity, int32_t n_bricks,
@@ -126,21 +121,20 @@ inline bool carve_workspace(void* base, int64_t n_gauss, int64_t capacity, int32
     };
     const int64_t cap = capacity > 0 ? capacity : 1;
     const int64_t n = n_gauss > 0 ? n_gauss : 1;
-    ws->n_tiles = static_cast<int32_t>((cap + kSortTile - 1) / kSortTile);
-    int64_t hist_len = int64_t(kRadix) * ws->n_tiles;
-    int64_t max_scan = hist_len;
-    if (n + 1 > max_scan) max_scan = n + 1;
-    if (int64_t(n_bricks) + 1 > max_scan) max_scan = int64_t(n_bricks) + 1;
-    ws->scan_tmp_len = scan_tmp_len_for(max_scan);
-    ws->keys0 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * cap));
-    ws->vals0 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * cap));
-    ws->keys1 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * cap));
-    ws->vals1 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * cap));
-    ws->gm_gid = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * cap));
-    ws->gm_cnt = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * (n + 1)));
-    ws->hist = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * 2 * (hist_len + 1)));
-    ws->hist1 = ws->hist ? ws->hist + hist_len + 1 : nullptr;
-    ws->scan_tmp = reinterpret_cast<long long*>(take(sizeof(long long) * ws->scan_tmp_len));
+    radix_plan(n_bricks, &ws->radix_passes, &ws->radix_bits);
+    const int64_t nd = int64_t(1) << ws->radix_bits;
+    const int64_t g_tiles = (n + kGaussTile - 1) / kGaussTile;
+    ws->stride0 = (g_tiles + 3) / 4 * 4;  // rows are scanned in 16-byte pieces
+    ws->stride1 = ((cap + kSortTile - 1) / kSortTile + 3) / 4 * 4;
+    for (int k = 0; k < 2; ++k) {
+        const bool used = k == 0 ? ws->radix_passes > 1 : ws->radix_passes > 2;
+        ws->keys[k] = reinterpret_cast<int32_t*>(take(used ? sizeof(int32_t) * cap : 256));
+        ws->vals[k] = reinterpret_cast<int2*>(take(used ? sizeof(int2) * cap : 256));
+        ws->hist[k] = reinterpret_cast<int32_t*>(take(used ? sizeof(int32_t) * nd * ws->stride1 : 256));
+    }
+    ws->hist0 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * nd * ws->stride0));
+    ws->rowtot = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * kMaxDigits));
+    ws->blk_base = reinterpret_cast<long long*>(take(sizeof(long long) * (g_tiles + 1)));
     ws->part = reinterpret_cast<float*>(
         take(deterministic ? sizeof(float) * GRAD_FLOATS * cap : 256));
     ws->gacc = reinterpret_cast<float*>(take(sizeof(float) * GRAD_FLOATS * n));
@@ -222,20 +216,6 @@ inline gs_status last_launch_status() {
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
-
-// Optional check of a scan's grand total against a pair capacity: with npairs set, the total
-// is stored there and GS_STATUS_CAPACITY is or-ed into *status when it exceeds capacity.
-struct CapCheck {
-    int64_t capacity = 0;
-    int64_t* npairs = nullptr;
-    int32_t* status = nullptr;
-};
-
-// Device-wide exclusive scan of int32 values (n <= kMaxCapacity + 1); 64-bit accumulation.
-// out may alias in. If total != nullptr, the grand total is written there (device int64).
-gs_status exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, long long* total,
-                             long long* tmp, int64_t tmp_len, cudaStream_t stream,
-                             CapCheck cc = CapCheck{});
 
 // Parameter chain + render-space gradient -> raw-parameter gradient (gs_param.cu).
 gs_status launch_param_bwd(const float* params, const float* gacc, int64_t n,

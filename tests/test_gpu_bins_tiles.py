@@ -1,0 +1,69 @@
+"""Brick lists where the binning's tiles can go wrong, bit for bit against the oracle's
+specification: Gaussian tiles of 256, rounds of 2,048 pairs per tile, boxes of more than 64 bricks
+(counted by rows and emitted by a warp), digit widths from one narrow pass to three passes."""
+import numpy as np
+import pytest
+
+from helpers import cloud_params
+from paper_2603_09621_gb300 import inputs
+from test_gpu_bins import _bin
+
+pytestmark = pytest.mark.gpu
+
+def _check(params, og, brick=(8, 8, 8)):
+    import oracle
+    ref = oracle.brick_lists(params, og, oracle.Config(brick=brick))
+    P = ref["pair_gid"].size
+    bins = _bin(params, og, brick, capacity=P + 1)
+    assert bins.npairs() == P and bins.status() == 0
+    for name, got in (("brick_off", bins.brick_off()), ("pair_gid", bins.pair_gid(P)), ("gm_off", bins.gm_off())):
+        np.testing.assert_array_equal(got.cpu().numpy(), ref[name])
+    bm_brick = np.repeat(np.arange(ref["brick_off"].size - 1), np.diff(ref["brick_off"]))
+    np.testing.assert_array_equal(bins.pair_brick(P).cpu().numpy(), bm_brick)
+    gmj = bins.pair_gmj(P).cpu().numpy()
+    assert np.array_equal(np.sort(gmj), np.arange(P))
+    np.testing.assert_array_equal(ref["gm_brick"][gmj], bm_brick)
+
+
+# grid (x, y, z) and brick: 1 brick; 2 x 2 x 2; 315 (one 9-bit pass); 512 (one full pass);
+# 513 x 1 x 1 (two passes, rows longer than their 32 digits); 4,096 and 131,072 (two passes of 6 and 9 bits);
+# 266,240 (three passes)
+GRIDS = [((8, 8, 8), (8, 8, 8)), ((13, 11, 10), (8, 8, 8)), ((50, 33, 71), (8, 8, 8)),
+         ((64, 64, 64), (8, 8, 8)), ((4104, 8, 8), (8, 8, 8)), ((64, 64, 64), (4, 4, 4)),
+         ((512, 512, 256), (8, 8, 8)), ((512, 512, 64), (4, 4, 4))]
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 1500])
+@pytest.mark.parametrize("dims,brick", GRIDS)
+def test_bins_tiles(dims, brick, n):
+    import oracle
+    og = oracle.Grid(*dims)
+    d = inputs.gaussian_cloud(n + dims[0], n, dims[::-1])
+    # a few wide Gaussians: boxes of tens to thousands of bricks, some clipped by the grid, next to
+    # narrow ones in the same warp
+    wide = np.arange(0, n, 97)
+    d["log_s"][wide] += np.log(np.linspace(3.0, 12.0, wide.size))[:, None].astype(np.float32)
+    _check(cloud_params(d), og, brick)
+
+
+def test_bins_rounds_exact_fill():
+    """Tiles of exactly 2,048 and 4,096 pairs, and one more: 256 Gaussians that all meet the same
+    8 (16) bricks, plus one."""
+    import oracle
+    og = oracle.Grid(16, 16, 32)
+    for z, n in ((8.0, 256), (8.0, 257), (16.0, 256), (16.0, 513)):
+        p = np.zeros((n, 12), np.float32)
+        p[:, :3] = (8.0, 8.0, z)
+        p[:, 3:6] = np.log(2.0) if z == 8.0 else np.log(np.array([2.0, 2.0, 4.0]))
+        p[:, 6], p[:, 10:] = 1.0, 0.5
+        _check(p, og)
+
+
+def test_bins_overflow_with_wide_gaussians():
+    """Every Gaussian covers the whole grid: the count is exact, nothing is listed."""
+    params = np.zeros((700, 12), np.float32)
+    params[:, :3], params[:, 3:6], params[:, 6], params[:, 10:] = 100.0, 8.0, 1.0, 0.5
+    import oracle
+    bins = _bin(params, oracle.Grid(200, 160, 120), capacity=5000)
+    assert bins.npairs() == 700 * 25 * 20 * 15 and bins.status() == 1
+    assert int(bins.brick_off().abs().sum().item()) == 0
