@@ -108,6 +108,8 @@ inline void radix_plan(int32_t n_bricks, int32_t* passes, int32_t* bits) {
     *bits = (need + *passes - 1) / *passes;
 }
 
+inline bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Carve (or size, if base == nullptr) the workspace. Returns false on overflow.
@@ -217,11 +219,6 @@ inline gs_status last_launch_status() {
     return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
-// Parameter chain + render-space gradient -> raw-parameter gradient (gs_param.cu).
-gs_status launch_param_bwd(const float* params, const float* gacc, int64_t n,
-                           const gs_grid* grid, const gs_config* cfg, float* dparams,
-                           cudaStream_t stream);
-
 // L1 loss with optional sign gradient into dpred (gs_volume.cu).
 gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t snx, float* dst,
                             int32_t dnz, int32_t dny, int32_t dnx, cudaStream_t st);
@@ -286,6 +283,34 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     float y;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// Four values, as one 16-byte access (kVec) or one by one.
+template <bool kVec>
+__device__ __forceinline__ void load4(const float* src, float (&d)[4]) {
+    if (kVec) {
+        const float4 a = *reinterpret_cast<const float4*>(src);
+        d[0] = a.x; d[1] = a.y; d[2] = a.z; d[3] = a.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = src[k];
+    }
+}
+
+template <bool kVec>
+__device__ __forceinline__ void store4(float* dst, const float (&d)[4]) {
+    if (kVec) {
+        *reinterpret_cast<float4*>(dst) = make_float4(d[0], d[1], d[2], d[3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dst[k] = d[k];
+    }
+}
+
+// Adjoint render's factors of one voxel (see k_bwd_prep).
+__device__ __forceinline__ float2 adj_factor(float gI, float w, float iv, float eps) {
+    const float al = gI / (w > eps ? w : eps);
+    return make_float2(al, (w > eps) ? al * iv : 0.0f);
 }
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + expf(-x)); }

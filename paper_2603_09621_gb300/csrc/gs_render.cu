@@ -403,17 +403,30 @@ __device__ __forceinline__ unsigned long long brick_row_mask(const Rec& R, const
 // Per-voxel adjoint factors (alpha, alpha I'): dL/dw_i = v_i alpha - alpha I' with
 // alpha = dL/dI / max(W, eps) and I' = I where W > eps, else 0 (Eq. 5; below the floor
 // I = S / eps, so dI/dw_i = v_i / eps).
+// kVec: four voxels per thread by 16-byte accesses (aligned volumes), the last n mod 4 voxels by
+// one thread each. Bound by HBM (20 bytes per voxel): one voxel per thread took 27 us at 4.7M
+// voxels, 14 us now.
+template <bool kVec>
 __global__ void __launch_bounds__(256) k_bwd_prep(const float* __restrict__ Iv,
                                                   const float* __restrict__ Wv,
                                                   const float* __restrict__ dIv, int64_t n,
                                                   float eps, float2* __restrict__ aip) {
     pdl_enter();
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const float w = Wv[i], gI = dIv[i];
-        const float al = gI / (w > eps ? w : eps);
-        aip[i] = make_float2(al, (w > eps) ? al * Iv[i] : 0.0f);
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t step = int64_t(gridDim.x) * blockDim.x;
+    if (kVec) {
+        for (int64_t q = t; q < n / 4; q += step) {
+            const float4 w = reinterpret_cast<const float4*>(Wv)[q];
+            const float4 g = reinterpret_cast<const float4*>(dIv)[q];
+            const float4 iv = reinterpret_cast<const float4*>(Iv)[q];
+            const float2 a0 = adj_factor(g.x, w.x, iv.x, eps), a1 = adj_factor(g.y, w.y, iv.y, eps);
+            const float2 a2 = adj_factor(g.z, w.z, iv.z, eps), a3 = adj_factor(g.w, w.w, iv.w, eps);
+            reinterpret_cast<float4*>(aip)[2 * q] = make_float4(a0.x, a0.y, a1.x, a1.y);
+            reinterpret_cast<float4*>(aip)[2 * q + 1] = make_float4(a2.x, a2.y, a3.x, a3.y);
+        }
     }
+    for (int64_t i = (kVec ? n / 4 * 4 : 0) + t; i < n; i += step)
+        aip[i] = adj_factor(dIv[i], Wv[i], Iv[i], eps);
 }
 
 // Adjoint sums of one (brick, Gaussian) pair, with h = gamma g (gamma = dL/dw) per voxel.
@@ -741,36 +754,6 @@ __global__ void __launch_bounds__(kBwdThreads, (BX == 16 ? 7 : 8)) k_render_bwd(
     }
 }
 
-// Deterministic reduction: per Gaussian, sum its per-brick partials in Gaussian-major order
-// (ascending brick index).
-__global__ void __launch_bounds__(256) k_pair_reduce(const float* __restrict__ part,
-                                                     const int32_t* __restrict__ gm_off,
-                                                     const int64_t* __restrict__ npairs,
-                                                     int64_t capacity, int64_t N,
-                                                     float* __restrict__ gacc) {
-    pdl_enter();
-    const int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g >= N) return;
-    float acc[12];
-#pragma unroll
-    for (int m = 0; m < 12; ++m) acc[m] = 0.f;
-    const int64_t P = *npairs;
-    if (P >= 0 && P <= capacity) {
-        const int a = gm_off[g], e = gm_off[g + 1];
-        for (int j = a; j < e; ++j) {
-            const float4* src = reinterpret_cast<const float4*>(part + int64_t(j) * GRAD_FLOATS);
-            const float4 p0 = src[0], p1 = src[1], p2 = src[2];
-            acc[0] += p0.x; acc[1] += p0.y; acc[2] += p0.z; acc[3] += p0.w;
-            acc[4] += p1.x; acc[5] += p1.y; acc[6] += p1.z; acc[7] += p1.w;
-            acc[8] += p2.x; acc[9] += p2.y; acc[10] += p2.z;
-        }
-    }
-    float4* dst = reinterpret_cast<float4*>(gacc + g * GRAD_FLOATS);
-    dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-    dst[2] = make_float4(acc[8], acc[9], acc[10], 0.f);
-}
-
 // ------------------------------------------------------------------------ host side
 
 RenderGeo make_geo(const gs_grid* grid, const gs_config* cfg) {
@@ -819,9 +802,10 @@ bool bins_match(const gs_bins* b, const gs_grid* grid, const gs_config* cfg);
 gs_status launch_bwd_prep(const float* I, const float* W, const float* dI, const RenderGeo& G,
                           const Workspace& ws, cudaStream_t st) {
     const int64_t nv = int64_t(G.nx) * G.ny * G.nz;
-    const int64_t pb = (nv + 255) / 256;
-    launch_k(k_bwd_prep, dim3(static_cast<unsigned>(pb < 65536 ? pb : 65536)), dim3(256), 0, st, I,
-        W, dI, nv, G.eps, ws.aip);
+    const bool vec = aligned16(I) && aligned16(W) && aligned16(dI);
+    const int64_t pb = ((vec ? nv / 4 : nv) + 256) / 256;
+    launch_k(vec ? k_bwd_prep<true> : k_bwd_prep<false>, dim3(static_cast<unsigned>(pb < 65536 ? pb : 65536)),
+        dim3(256), 0, st, I, W, dI, nv, G.eps, ws.aip);
     return last_launch_status();
 }
 
@@ -855,24 +839,6 @@ gs_status launch_adjoint_pairs(const gs_bins* bins, const gs_grid* grid, const g
     return GS_ERR_INVALID_ARG;
 }
 
-// Render-space adjoint into ws.gacc [N, 12] (no parameter chain).
-static gs_status render_bwd_geo(const gs_bins* bins, const gs_grid* grid, const gs_config* cfg,
-                                const float* I, const float* W, const float* dI,
-                                const Workspace& ws, cudaStream_t st) {
-    RenderGeo G = make_geo(grid, cfg);
-    gs_status s = launch_bwd_prep(I, W, dI, G, ws, st);
-    if (s != GS_OK) return s;
-    s = launch_adjoint_pairs(bins, grid, cfg, ws, st);
-    if (s != GS_OK) return s;
-    const int64_t N = bins->n_gauss;
-    if (cfg->deterministic && N > 0) {
-        launch_k(k_pair_reduce, dim3(static_cast<unsigned>((N + 255) / 256)), dim3(256), 0, st,
-            ws.part, bins->gm_off, bins->d_npairs, bins->capacity, N, ws.gacc);
-        s = last_launch_status();
-    }
-    return s;
-}
-
 }  // namespace gs
 
 using namespace gs;
@@ -898,8 +864,11 @@ extern "C" gs_status gs_render_bwd(const float* params, const gs_bins* bins, con
     s = bind_workspace(ws, ws_bytes, bins->n_gauss, bins->capacity, grid, cfg, &w);
     if (s != GS_OK) return s;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = render_bwd_geo(bins, grid, cfg, I, W, dI, w, st);
+    s = launch_bwd_prep(I, W, dI, make_geo(grid, cfg), w, st);
     if (s != GS_OK) return s;
-    if (bins->n_gauss == 0) return GS_OK;
-    return launch_param_bwd(params, w.gacc, bins->n_gauss, grid, cfg, dparams, st);
+    s = launch_adjoint_pairs(bins, grid, cfg, w, st);
+    if (s != GS_OK || bins->n_gauss == 0) return s;
+    // (the reduction over a Gaussian's pairs and the chain to its raw parameters in one kernel; as
+    // two, with the sums through memory, 42 us against 39 us at 375,000 Gaussians and 2.1M pairs)
+    return launch_chain_grad(params, dparams, w.part, w.gacc, bins, bins->n_gauss, grid, cfg, st);
 }
