@@ -454,7 +454,8 @@ struct RowScan {
     int32_t* rowtot;     // row totals
     int32_t* zero;       // the next pass's counts, cleared here (nullptr: last pass)
     int64_t zero_cols;
-    long long* blk;      // first pass: pairs of each Gaussian tile, scanned by the last block
+    long long* blk;      // first pass: pairs of each Gaussian tile, scanned by the last block,
+    int32_t* ticket;     // which also clears the loss kernel's block counter
     int nd;
     int64_t* npairs;
     int64_t capacity;
@@ -489,6 +490,7 @@ __global__ void __launch_bounds__(kRowThreads) k_row_scan(RowScan A) {
         __syncthreads();
         if (tid == 0) {
             A.blk[A.cols] = carry;
+            *A.ticket = 0;
             *A.npairs = carry;
             *A.status = (bad ? GS_STATUS_NONFINITE : 0) | (carry > A.capacity ? GS_STATUS_CAPACITY : 0);
         }
@@ -934,6 +936,7 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         R.zero = last ? nullptr : ws.hist[nxt];
         R.zero_cols = ws.stride1;
         R.blk = ws.blk_base;
+        R.ticket = ws.ticket;
         R.nd = nd;
         R.npairs = bins->d_npairs;
         R.capacity = cap;

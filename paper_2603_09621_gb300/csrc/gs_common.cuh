@@ -95,6 +95,8 @@ struct Workspace {
     float* gacc;             // [n_gauss, 12] render-space gradient per Gaussian
     float2* aip;             // [n_voxels] (alpha, alpha I'), alpha = dL/dI / max(W, eps)
     float* l1_part;          // [kL1Blocks]
+    int32_t* ticket;         // finished blocks of the fitting step's loss kernel, cleared by the
+                             // binning's first scan
     size_t bytes;
 };
 
@@ -142,6 +144,7 @@ inline bool carve_workspace(void* base, int64_t n_gauss, int64_t capacity, int32
     ws->gacc = reinterpret_cast<float*>(take(sizeof(float) * GRAD_FLOATS * n));
     ws->aip = reinterpret_cast<float2*>(take(sizeof(float2) * (n_voxels > 0 ? n_voxels : 1)));
     ws->l1_part = reinterpret_cast<float*>(take(sizeof(float) * kL1Blocks));
+    ws->ticket = reinterpret_cast<int32_t*>(take(sizeof(int32_t)));
     ws->bytes = off;
     return true;
 }
@@ -219,14 +222,11 @@ inline gs_status last_launch_status() {
     return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
-// L1 loss with optional sign gradient into dpred (gs_volume.cu).
 gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t snx, float* dst,
                             int32_t dnz, int32_t dny, int32_t dnx, cudaStream_t st);
 gs_status resample_adj_prep_impl(const float* dlr, int32_t lnz, int32_t lny, int32_t lnx,
                                  const float* I, const float* W, int32_t nz, int32_t ny, int32_t nx,
                                  float eps, float2* aip, cudaStream_t st);
-gs_status launch_l1(const float* pred, const float* target, int64_t n, float* d_loss,
-                    float* dpred, float* partials, cudaStream_t stream, int64_t n_norm = 0);
 // Fitting-step tails (gs_param.cu): chain without Adam; Adam with an optional device skip flag.
 gs_status launch_chain_grad(const float* params, float* grad, const float* part,
                             const float* gacc, const gs_bins* bins, int64_t n,

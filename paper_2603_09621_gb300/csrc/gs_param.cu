@@ -162,8 +162,9 @@ struct AdamCoef {
     float bc1, rs_bc2;
 };
 
-__device__ __forceinline__ AdamCoef adam_coef(const AdamLr& hp, const int32_t* d_step) {
-    const int t = *d_step + 1;
+// Coefficients of the step after `taken` steps.
+__device__ __forceinline__ AdamCoef adam_coef(const AdamLr& hp, int taken) {
+    const int t = taken + 1;
     // bias corrections 1 - beta^t = -expm1(t log beta), accurate for small t (1 - beta ~ 1e-3)
     AdamCoef c;
     c.bc1 = -expm1f(float(t) * hp.log_b1);
@@ -193,7 +194,7 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ params, const 
                                               const int32_t* __restrict__ d_skip) {
     pdl_enter();
     if (d_skip && *d_skip != 0) return;  // the step was declared a no-op (see gs_fit_apply)
-    const AdamCoef c = adam_coef(hp, d_step);
+    const AdamCoef c = adam_coef(hp, *d_step);
     float lrb[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) lrb[k] = hp.lr[k] / c.bc1;
@@ -224,7 +225,9 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ params, const 
 
 // Fitting step tail, one thread per Gaussian: sum the per-brick partials in Gaussian-major
 // order (deterministic mode) or take the atomically accumulated gradient, chain it to the
-// raw parameters (written to grad), and (kAdam) apply Adam to params, m, v.
+// raw parameters (written to grad), and (kAdam) apply Adam to params, m, v; d_step already counts
+// this step. A step whose binning overflowed rendered nothing: it leaves parameters and moments as
+// they are and zeroes grad (the caller grows the bins and repeats the step).
 template <bool kDet, bool kAdam>
 __global__ void __launch_bounds__(256, 4) k_chain_adam(
     float* __restrict__ params, float* __restrict__ grad, float* __restrict__ m,
@@ -237,8 +240,6 @@ __global__ void __launch_bounds__(256, 4) k_chain_adam(
     float gv[12];
     const int64_t P = *npairs;
     if (P < 0 || P > capacity) {
-        // The binning overflowed: this step rendered nothing, so it leaves the parameters and
-        // moments as they are (the caller grows the bins and repeats the step).
 #pragma unroll
         for (int k = 0; k < 12; ++k) gv[k] = 0.f;
         store12(grad + g * 12, gv);
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(256, 4) k_chain_adam(
     if (!kAdam) return;
     load12(m + g * 12, mm);
     load12(v + g * 12, vv);
-    const AdamCoef c = adam_coef(hp, d_step);
+    const AdamCoef c = adam_coef(hp, *d_step - 1);
 #pragma unroll
     for (int k = 0; k < 12; ++k) adam_one(p[k], out[k], mm[k], vv[k], hp.lr[lr_group(k)] / c.bc1, hp, c);
     store12(params + g * 12, p);
@@ -272,16 +273,10 @@ __global__ void __launch_bounds__(256, 4) k_chain_adam(
     store12(v + g * 12, vv);
 }
 
-// Counts a step, unless npairs is given and the step's binning overflowed the pair capacity
-// (then the fitting step was a no-op), or d_skip is given and nonzero.
-__global__ void k_step_inc(int32_t* d_step, const int64_t* __restrict__ npairs, int64_t capacity,
-                           const int32_t* __restrict__ d_skip) {
+// Counts a step, unless d_skip is given and nonzero.
+__global__ void k_step_inc(int32_t* d_step, const int32_t* __restrict__ d_skip) {
     pdl_enter();
     if (d_skip && *d_skip != 0) return;
-    if (npairs) {
-        const int64_t P = *npairs;
-        if (P < 0 || P > capacity) return;
-    }
     *d_step += 1;
 }
 
@@ -367,7 +362,7 @@ static bool adam_ok(const gs_adam* hp) {
 gs_status launch_chain_adam(float* params, float* grad, float* m, float* v, const float* part,
                             const float* gacc, const gs_bins* bins, int64_t n,
                             const gs_grid* grid, const gs_config* cfg, const gs_adam* hp,
-                            int32_t* d_step, cudaStream_t st) {
+                            const int32_t* d_step, cudaStream_t st) {
     if (!adam_ok(hp)) return GS_ERR_INVALID_ARG;
     ChainGeo C;
     for (int k = 0; k < 3; ++k) C.h[k] = grid->h[k];
@@ -382,10 +377,6 @@ gs_status launch_chain_adam(float* params, float* grad, float* m, float* v, cons
     else
         launch_k(k_chain_adam<false, true>, dim3(gb), dim3(256), 0, st, params, grad, m, v, part,
             gacc, bins->gm_off, bins->d_npairs, bins->capacity, n, C, a, d_step);
-    gs_status s = last_launch_status();
-    if (s != GS_OK) return s;
-    launch_k(k_step_inc, dim3(1), dim3(1), 0, st, d_step, bins->d_npairs, bins->capacity,
-        static_cast<const int32_t*>(nullptr));
     return last_launch_status();
 }
 
@@ -430,8 +421,7 @@ gs_status launch_adam(float* params, const float* grad, float* m, float* v, int6
         gs_status s = last_launch_status();
         if (s != GS_OK) return s;
     }
-    launch_k(k_step_inc, dim3(1), dim3(1), 0, st, d_step, static_cast<const int64_t*>(nullptr),
-        int64_t(0), d_skip);
+    launch_k(k_step_inc, dim3(1), dim3(1), 0, st, d_step, d_skip);
     return last_launch_status();
 }
 }  // namespace gs

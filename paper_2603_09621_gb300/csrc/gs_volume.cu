@@ -86,74 +86,178 @@ __global__ void __launch_bounds__(256) k_downsample_bwd(const float* __restrict_
     }
 }
 
-// Stage 1: fixed grid of kL1Blocks blocks; each thread sums |pred - target| over a fixed
-// stride, then a fixed-shape block tree. Optionally writes sign(pred - target) / n.
-__global__ void __launch_bounds__(256) k_l1_partial(const float* __restrict__ pred,
-                                                    const float* __restrict__ target, int64_t n,
-                                                    float inv_n, float* __restrict__ dpred,
-                                                    float* __restrict__ partials) {
-    pdl_enter();
-    __shared__ float sm[256];
-    float acc = 0.f;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const float d = pred[i] - target[i];
-        acc += fabsf(d);
-        if (dpred) dpred[i] = (d > 0.f) ? inv_n : ((d < 0.f) ? -inv_n : 0.f);
-    }
+// L1 sums: a fixed grid of kL1Blocks blocks of kL1Threads; thread t sums |pred - target| over the
+// quads of consecutive values t, t + 131,072, ..., then a fixed-shape tree over the block (partials)
+// and over the blocks, so the loss does not depend on which kernel forms it or on alignment. The
+// last tree runs in a launch of its own (k_l1_final) or in the block that finishes last (ticket: a
+// counter cleared earlier on the stream).
+constexpr int kL1Threads = 128;
+
+__device__ __forceinline__ float l1_block_sum(float acc, float* sm) {
     sm[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
+    for (int o = kL1Threads / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partials[blockIdx.x] = sm[0];
+    return sm[0];
 }
 
-__global__ void __launch_bounds__(1024) k_l1_final(const float* __restrict__ partials, float inv_n,
-                                                   float* __restrict__ loss) {
-    pdl_enter();
-    __shared__ float sm[kL1Blocks];
-    sm[threadIdx.x] = partials[threadIdx.x];
+// Tree over the kL1Blocks partials by one block of kL1Threads.
+__device__ __forceinline__ void l1_total(const float* partials, float inv_n, float* loss, float* sm) {
+    constexpr int kPer = kL1Blocks / kL1Threads;  // partials per thread: the tree's first levels
+    const int t = threadIdx.x;
+    float p[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) p[k] = __ldcg(partials + t + k * kL1Threads);
+#pragma unroll
+    for (int o = kPer / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < o; ++k) p[k] += p[k + o];
+    const float sum = l1_block_sum(p[0], sm);
+    if (t == 0) *loss = sum * inv_n;
+}
+
+__device__ __forceinline__ void l1_finish(float acc, float inv_n, float* partials, int* ticket, float* loss) {
+    __shared__ float sm[kL1Threads];
+    __shared__ bool last;
+    const float sum = l1_block_sum(acc, sm);
+    if (threadIdx.x == 0) partials[blockIdx.x] = sum;
+    if (!ticket) return;
+    if (threadIdx.x == 0) {
+        __threadfence();  // the partial is visible before the ticket is taken
+        last = atomicAdd(ticket, 1) == kL1Blocks - 1;
+    }
     __syncthreads();
-    for (int o = kL1Blocks / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
-        __syncthreads();
+    if (!last) return;
+    __threadfence();
+    l1_total(partials, inv_n, loss, sm);
+}
+
+__device__ __forceinline__ float l1_sign(float d, float inv_n) {
+    return (d > 0.f) ? inv_n : ((d < 0.f) ? -inv_n : 0.f);
+}
+
+// The fitting step's counter: one thread of the loss kernel counts the step (d_step, or nullptr),
+// unless the binning overflowed the capacity and the step will change nothing.
+struct StepCount {
+    int32_t* d_step;
+    const int64_t* npairs;
+    int64_t capacity;
+};
+
+__device__ __forceinline__ void count_step(const StepCount& c) {
+    if (c.d_step && blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t P = *c.npairs;
+        if (P >= 0 && P <= c.capacity) *c.d_step += 1;
     }
-    if (threadIdx.x == 0) *loss = sm[0] * inv_n;
 }
 
-static unsigned grid_for(int64_t n) {
-    int64_t b = (n + 255) / 256;
-    if (b < 1) b = 1;
-    return static_cast<unsigned>(b < 65536 ? b : 65536);
-}
-
-// The slice profile's adjoint fused with the adjoint render's factors over a 2D grid (blockIdx.y =
-// HR slice) with four voxels per thread, for planes of a multiple of 4 voxels and at most 65,535
-// slices. Same arithmetic, same results as k_profile_adj_prep.
-__global__ void __launch_bounds__(256) k_profile_adj_prep4(const float4* __restrict__ dlr,
-                                                           const float4* __restrict__ Iv,
-                                                           const float4* __restrict__ Wv,
-                                                           int plane4, int zmax, int s, float inv_s,
-                                                           float eps, float4* __restrict__ aip) {
+// Optionally writes sign(pred - target) / n. kVec: 16-byte accesses of aligned arrays.
+template <bool kVec>
+__global__ void __launch_bounds__(kL1Threads) k_l1_partial(const float* __restrict__ pred,
+                                                           const float* __restrict__ target, int64_t n,
+                                                           float inv_n, float* dpred, float* partials,
+                                                           int* ticket, float* loss, StepCount count) {
     pdl_enter();
-    const int z = blockIdx.y;
-    const bool in = z < zmax;
-    const int64_t base = int64_t(z) * plane4;
-    const float4* g4 = dlr + int64_t(in ? z / s : 0) * plane4;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < plane4; r += gridDim.x * blockDim.x) {
-        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (in) {
-            const float4 d = g4[r];
-            g = make_float4(d.x * inv_s, d.y * inv_s, d.z * inv_s, d.w * inv_s);
+    count_step(count);
+    float acc = 0.f;
+    for (int64_t i = 4 * (int64_t(blockIdx.x) * kL1Threads + threadIdx.x); i < n; i += 4 * kL1Blocks * kL1Threads) {
+        if (i + 3 < n) {
+            float p[4], t[4];
+            load4<kVec>(pred + i, p);
+            load4<kVec>(target + i, t);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float d = p[e] - t[e];
+                acc += fabsf(d);
+                p[e] = l1_sign(d, inv_n);
+            }
+            if (dpred) store4<kVec>(dpred + i, p);
+        } else {
+            for (int64_t e = i; e < n; ++e) {
+                const float d = pred[e] - target[e];
+                acc += fabsf(d);
+                if (dpred) dpred[e] = l1_sign(d, inv_n);
+            }
         }
-        const float4 w = Wv[base + r], iv = Iv[base + r];
-        const float2 a0 = adj_factor(g.x, w.x, iv.x, eps), a1 = adj_factor(g.y, w.y, iv.y, eps);
-        const float2 a2 = adj_factor(g.z, w.z, iv.z, eps), a3 = adj_factor(g.w, w.w, iv.w, eps);
-        aip[2 * (base + r)] = make_float4(a0.x, a0.y, a1.x, a1.y);
-        aip[2 * (base + r) + 1] = make_float4(a2.x, a2.y, a3.x, a3.y);
     }
+    l1_finish(acc, inv_n, partials, ticket, loss);
+}
+
+__global__ void __launch_bounds__(kL1Threads) k_l1_final(const float* partials, float inv_n, float* loss) {
+    pdl_enter();
+    __shared__ float sm[kL1Threads];
+    l1_total(partials, inv_n, loss, sm);
+}
+
+// The fitting step's z box model in one pass: slice profile, L1 and its sign gradient (to lr_pred),
+// profile adjoint and the adjoint render's factors (alpha, alpha I') of the s HR voxels below each
+// LR voxel, with dL/dI = dL/dLR / s (0 in the trailing slices, which no LR slice covers). Bound by
+// HBM: I, W, target read once, dL/dLR and the factors written once. kS: slices per LR slice at
+// compile time (their I values stay in registers), 0: read again from the cache. A thread owns a
+// quad of LR voxels as in k_l1_partial, so loss and gradient equal the separate entry points' bit for
+// bit; kVec: planes of a multiple of 4 voxels and aligned volumes, by 16-byte accesses.
+// As four kernels (profile, L1, its tree, factors) 16 us at 128^3, s = 2, and 33 us at
+// 256 x 256 x 128, s = 4; here 9 and 27 us (151 MB). All 1,024 blocks of 128 threads are resident at
+// once; with 256 threads and 3 (4) blocks per SM 12 and 32 (28) us; one LR voxel per thread with
+// 4-byte accesses 9 and 48 us.
+template <int kS, bool kVec>
+__global__ void __launch_bounds__(kL1Threads, 7) k_profile_loss(
+    const float* __restrict__ Iv, const float* __restrict__ Wv, const float* __restrict__ target, unsigned plane,
+    FastDiv by_plane, int64_t n_lr, int64_t n_hr, int s_, float inv_s, float inv_n, float eps,
+    float* __restrict__ lr_pred, float2* __restrict__ aip, float* partials, int* ticket, float* loss,
+    StepCount count) {
+    pdl_enter();
+    count_step(count);
+    constexpr int kV = kVec ? 4 : 1;  // consecutive LR voxels taken at once
+    const int s = kS > 0 ? kS : s_;
+    const int64_t t0 = int64_t(blockIdx.x) * kL1Threads + threadIdx.x;
+    float acc = 0.f;
+    for (int64_t q = 4 * t0; q < n_lr; q += 4 * kL1Blocks * kL1Threads) {
+#pragma unroll
+        for (int64_t i = q; i < q + 4; i += kV) {
+            if (i >= n_lr) break;
+            const unsigned k = fast_div(static_cast<unsigned>(i), by_plane);
+            // first HR voxel of the column: (k s) plane + (i - k plane)
+            const int64_t v0 = i + int64_t(k) * (s - 1) * plane;
+            Voxels<kV> col[kS > 0 ? kS : 1], sum = {}, g;
+#pragma unroll
+            for (int j = 0; j < s; ++j) {
+                const Voxels<kV> x = load_voxels<kV>(Iv + v0 + int64_t(j) * plane);
+                if (kS > 0) col[kS > 0 ? j : 0] = x;
+#pragma unroll
+                for (int e = 0; e < kV; ++e) sum.v[e] += x.v[e];
+            }
+            const Voxels<kV> t = load_voxels<kV>(target + i);
+#pragma unroll
+            for (int e = 0; e < kV; ++e) {
+                // (the profile's mean rounds before the difference, as when it is stored)
+                const float d = __fmul_rn(sum.v[e], inv_s) - t.v[e];
+                acc += fabsf(d);
+                g.v[e] = l1_sign(d, inv_n);
+            }
+            store_voxels<kV>(lr_pred + i, g);
+#pragma unroll
+            for (int j = 0; j < s; ++j) {
+                const int64_t v = v0 + int64_t(j) * plane;
+                const Voxels<kV> w = load_voxels<kV>(Wv + v);
+                const Voxels<kV> x = kS > 0 ? col[kS > 0 ? j : 0] : load_voxels<kV>(Iv + v);
+                float2 a[kV];
+#pragma unroll
+                for (int e = 0; e < kV; ++e) a[e] = adj_factor(g.v[e] * inv_s, w.v[e], x.v[e], eps);
+                if constexpr (kV == 4) {
+                    reinterpret_cast<float4*>(aip + v)[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+                    reinterpret_cast<float4*>(aip + v)[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
+                } else {
+                    aip[v] = a[0];
+                }
+            }
+        }
+    }
+    for (int64_t v = n_lr * s + t0; v < n_hr; v += kL1Blocks * kL1Threads)
+        aip[v] = adj_factor(0.f, Wv[v], Iv[v], eps);
+    l1_finish(acc, inv_n, partials, ticket, loss);
 }
 
 static dim3 grid2d(int64_t per_plane, int64_t slices) {
@@ -165,16 +269,41 @@ static bool vec_ok(const void* a, const void* b, int64_t plane) {
     return plane % 4 == 0 && aligned16(a) && aligned16(b);
 }
 
-gs_status launch_l1(const float* pred, const float* target, int64_t n, float* d_loss, float* dpred,
-                    float* partials, cudaStream_t st, int64_t n_norm) {
-    // the mean's normaliser: n, or n_norm > 0 when these values are one part of a larger mean
+// The mean's normaliser: n, or n_norm > 0 when these values are one part of a larger mean.
+static float l1_inv_n(int64_t n, int64_t n_norm) {
     const int64_t nn = n_norm > 0 ? n_norm : n;
-    const float inv_n = nn > 0 ? 1.0f / float(nn) : 0.0f;
-    launch_k(k_l1_partial, dim3(kL1Blocks), dim3(256), 0, st, pred, target, n, inv_n, dpred,
-        partials);
+    return nn > 0 ? 1.0f / float(nn) : 0.0f;
+}
+
+static gs_status launch_l1(const float* pred, const float* target, int64_t n, float* d_loss, float* dpred,
+                    float* partials, cudaStream_t st, int64_t n_norm, int* ticket, const StepCount& count) {
+    const float inv_n = l1_inv_n(n, n_norm);
+    const bool vec = aligned16(pred) && aligned16(target) && (!dpred || aligned16(dpred));
+    launch_k(vec ? k_l1_partial<true> : k_l1_partial<false>, dim3(kL1Blocks), dim3(kL1Threads), 0, st, pred,
+        target, n, inv_n, dpred, partials, ticket, d_loss, count);
     gs_status s = last_launch_status();
-    if (s != GS_OK) return s;
-    launch_k(k_l1_final, dim3(1), dim3(kL1Blocks), 0, st, partials, inv_n, d_loss);
+    if (s != GS_OK || ticket) return s;
+    launch_k(k_l1_final, dim3(1), dim3(kL1Threads), 0, st, partials, inv_n, d_loss);
+    return last_launch_status();
+}
+
+template <bool kVec>
+static gs_status launch_profile_loss(const float* I, const float* W, const float* target, int nz, int ny, int nx,
+                                     int s, float eps, float* lr_pred, float* d_loss, int64_t n_norm,
+                                     const Workspace& ws, const StepCount& count, cudaStream_t st) {
+    const int64_t plane = int64_t(ny) * nx, n_lr = plane * (nz / s);
+    auto go = [&](auto kernel) {
+        launch_k(kernel, dim3(kL1Blocks), dim3(kL1Threads), 0, st, I, W, target, static_cast<unsigned>(plane),
+            make_fastdiv(static_cast<unsigned>(plane)), n_lr, plane * nz, s, 1.0f / float(s),
+            l1_inv_n(n_lr, n_norm), eps, lr_pred, ws.aip, ws.l1_part, ws.ticket, d_loss, count);
+    };
+    switch (s) {
+        case 1: go(k_profile_loss<1, kVec>); break;
+        case 2: go(k_profile_loss<2, kVec>); break;
+        case 3: go(k_profile_loss<3, kVec>); break;
+        case 4: go(k_profile_loss<4, kVec>); break;
+        default: go(k_profile_loss<0, kVec>);
+    }
     return last_launch_status();
 }
 
@@ -218,29 +347,7 @@ gs_status launch_adjoint_pairs(const gs_bins* bins, const gs_grid* grid, const g
 gs_status launch_chain_adam(float* params, float* grad, float* m, float* v, const float* part,
                             const float* gacc, const gs_bins* bins, int64_t n,
                             const gs_grid* grid, const gs_config* cfg, const gs_adam* hp,
-                            int32_t* d_step, cudaStream_t st);
-
-// Slice-profile adjoint fused with the adjoint render's per-voxel factors: for each HR voxel
-// dL/dI = dL/dLR[z / s] / s (0 below the last full slab), alpha = dL/dI / max(W, eps) and
-// I' = I where W > eps, else 0; stored as (alpha, alpha I').
-__global__ void __launch_bounds__(256) k_profile_adj_prep(const float* __restrict__ dlr,
-                                                          const float* __restrict__ Iv,
-                                                          const float* __restrict__ Wv, int nz,
-                                                          int ny, int nx, int s, float inv_s,
-                                                          float eps, float2* __restrict__ aip) {
-    pdl_enter();
-    const int64_t plane = int64_t(ny) * nx;
-    const int64_t n = plane * nz;
-    const int zmax = s * (nz / s);
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t z = i / plane, r = i - z * plane;
-        const float gI = (z < zmax) ? dlr[(z / s) * plane + r] * inv_s : 0.0f;
-        const float w = Wv[i];
-        const float al = gI / (w > eps ? w : eps);
-        aip[i] = make_float2(al, (w > eps) ? al * Iv[i] : 0.0f);
-    }
-}
+                            const int32_t* d_step, cudaStream_t st);
 
 }  // namespace gs
 
@@ -269,7 +376,7 @@ extern "C" gs_status gs_l1_loss(const float* pred, const float* target, int64_t 
     if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return GS_ERR_INVALID_ARG;
     if (ws_bytes < sizeof(float) * kL1Blocks) return GS_ERR_WORKSPACE;
     return launch_l1(pred, target, n, d_loss, dpred, static_cast<float*>(ws),
-                     reinterpret_cast<cudaStream_t>(stream));
+                     reinterpret_cast<cudaStream_t>(stream), 0, nullptr, StepCount{});
 }
 
 namespace {
@@ -327,13 +434,16 @@ gs_status fit_prepare(gs_fit_state* st, gs_stream stream, FitRun* run) {
 
 // Bin, render, LR forward model, L1 (normalised by n_norm LR values when n_norm > 0, else by
 // the state's own count), its adjoint with the adjoint render's per-voxel factors, and the
-// adjoint render kernel; phase events 0-4.
-gs_status fit_front(const FitRun& run, int64_t n_norm) {
+// adjoint render kernel; phase events 0-4. The loss kernel counts the step in d_step unless that is
+// nullptr: the Adam kernel behind it reads the counter already advanced, and no launch is left that
+// only counts.
+gs_status fit_front(const FitRun& run, int64_t n_norm, int32_t* d_step) {
     gs_fit_state* st = run.st;
     const Workspace& w = run.w;
     cudaStream_t cs = run.cs;
     const bool trilinear = st->lr_model == GS_LR_TRILINEAR;
     const gs_grid& g = st->grid;
+    const StepCount count{d_step, st->bins.d_npairs, st->bins.capacity};
     if (!run.mark(0)) return GS_ERR_CUDA;
     gs_status s = bin_bricks_impl(st->params, &g, &st->cfg, &st->bins, w, cs);
     if (s != GS_OK) return s;
@@ -342,37 +452,24 @@ gs_status fit_front(const FitRun& run, int64_t n_norm) {
     if (s != GS_OK) return s;
     if (!run.mark(2)) return GS_ERR_CUDA;
     if (run.lr_ready && cudaStreamWaitEvent(cs, run.lr_ready, 0) != cudaSuccess) return GS_ERR_CUDA;
-    if (trilinear)
-        s = resample_fwd_impl(st->I, g.nz, g.ny, g.nx, st->lr_pred, st->lr_nz, st->lr_ny, st->lr_nx, cs);
-    else
-        s = downsample_fwd_impl(st->I, g.nz, g.ny, g.nx, st->s, st->lr_pred, cs);
-    if (s != GS_OK) return s;
-    const int64_t n_lr = trilinear ? int64_t(st->lr_nz) * st->lr_ny * st->lr_nx
-                                   : int64_t(g.nz / st->s) * g.ny * g.nx;
-    // L1 loss; its gradient overwrites lr_pred in place.
-    s = launch_l1(st->lr_pred, st->lr_target, n_lr, st->d_loss, st->lr_pred, w.l1_part, cs, n_norm);
-    if (s != GS_OK) return s;
     if (trilinear) {
+        s = resample_fwd_impl(st->I, g.nz, g.ny, g.nx, st->lr_pred, st->lr_nz, st->lr_ny, st->lr_nx, cs);
+        if (s != GS_OK) return s;
+        const int64_t n_lr = int64_t(st->lr_nz) * st->lr_ny * st->lr_nx;
+        // L1 loss; its gradient overwrites lr_pred in place.
+        s = launch_l1(st->lr_pred, st->lr_target, n_lr, st->d_loss, st->lr_pred, w.l1_part, cs, n_norm, w.ticket,
+                      count);
+        if (s != GS_OK) return s;
         s = resample_adj_prep_impl(st->lr_pred, st->lr_nz, st->lr_ny, st->lr_nx, st->I, st->W, g.nz,
                                    g.ny, g.nx, st->cfg.eps, w.aip, cs);
-        if (s != GS_OK) return s;
     } else {
-        const int64_t nv = int64_t(g.nz) * g.ny * g.nx;
-        const int64_t plane = int64_t(g.ny) * g.nx;
-        if (vec_ok(st->lr_pred, st->I, plane) && vec_ok(st->W, w.aip, plane) && g.nz <= 65535) {
-            const int plane4 = static_cast<int>(plane / 4);
-            launch_k(k_profile_adj_prep4, dim3(grid2d(plane4, g.nz)), dim3(256), 0, cs,
-                reinterpret_cast<const float4*>(st->lr_pred),
-                reinterpret_cast<const float4*>(st->I), reinterpret_cast<const float4*>(st->W),
-                plane4, st->s * (g.nz / st->s), st->s, 1.0f / float(st->s), st->cfg.eps,
-                reinterpret_cast<float4*>(w.aip));
-        } else {
-            launch_k(k_profile_adj_prep, dim3(grid_for(nv)), dim3(256), 0, cs, st->lr_pred, st->I,
-                st->W, g.nz, g.ny, g.nx, st->s, 1.0f / float(st->s), st->cfg.eps, w.aip);
-        }
-        s = last_launch_status();
-        if (s != GS_OK) return s;
+        const bool vec = vec_ok(st->I, st->W, int64_t(g.ny) * g.nx) && aligned16(st->lr_target) &&
+                         aligned16(st->lr_pred);
+        s = (vec ? launch_profile_loss<true> : launch_profile_loss<false>)(
+            st->I, st->W, st->lr_target, g.nz, g.ny, g.nx, st->s, st->cfg.eps, st->lr_pred, st->d_loss, n_norm, w,
+            count, cs);
     }
+    if (s != GS_OK) return s;
     if (!run.mark(3)) return GS_ERR_CUDA;
     s = launch_adjoint_pairs(&st->bins, &g, &st->cfg, w, cs);
     if (s != GS_OK) return s;
@@ -386,7 +483,7 @@ extern "C" gs_status gs_fit_step(gs_fit_state* st, gs_stream stream) {
     FitRun run;
     gs_status s = fit_prepare(st, stream, &run);
     if (s != GS_OK) return s;
-    s = fit_front(run, 0);
+    s = fit_front(run, 0, st->d_step);
     if (s != GS_OK) return s;
     s = launch_chain_adam(st->params, st->grad, st->m, st->v, run.w.part, run.w.gacc, &st->bins,
                           st->n_gauss, &st->grid, &st->cfg, &st->adam, st->d_step, run.cs);
@@ -456,7 +553,7 @@ extern "C" gs_status gs_fit_step_host(gs_fit_state* st, const float* h_params,
             return GS_ERR_CUDA;
         run.lr_ready = r->lr_done;
     }
-    s = fit_front(run, 0);
+    s = fit_front(run, 0, st->d_step);
     if (s != GS_OK) return s;
     s = launch_chain_adam(st->params, st->grad, st->m, st->v, run.w.part, run.w.gacc, &st->bins,
                           st->n_gauss, &st->grid, &st->cfg, &st->adam, st->d_step, cs);
@@ -473,7 +570,7 @@ extern "C" gs_status gs_fit_grad(gs_fit_state* st, int64_t n_lr_total, gs_stream
     FitRun run;
     gs_status s = fit_prepare(st, stream, &run);
     if (s != GS_OK) return s;
-    s = fit_front(run, n_lr_total);
+    s = fit_front(run, n_lr_total, nullptr);
     if (s != GS_OK) return s;
     s = launch_chain_grad(st->params, st->grad, run.w.part, run.w.gacc, &st->bins, st->n_gauss,
                           &st->grid, &st->cfg, run.cs);
