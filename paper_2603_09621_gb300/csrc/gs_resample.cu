@@ -48,34 +48,54 @@ __device__ __forceinline__ void res_range(const ResAxis& A, int i, int& jlo, int
     jhi = min(A.n_dst - 1, static_cast<int>(ceilf((float(i) + 1.5f) * A.inv - 0.5f)) + 1);
 }
 
+// A thread owns one destination column x of a plane z and walks kRows rows y: its x and z taps are
+// formed once, and an element offset (T: 32 bits where the source allows) is a sum of precomputed
+// parts. Bound by instruction issue: one voxel per thread with three index remainders and 64-bit
+// addresses took 170 instructions a voxel. L2 flushed, before -> one row -> four rows per thread:
+// 240 x 240 x 155 to 100^3 14.3 -> 13.6 -> 18.4 us (too few warps in flight), to 200 x 200 x 129
+// 40.5 -> 31.2 -> 31.3, 100^3 to 240 x 240 x 155 63.8 -> 45.0 -> 34.9.
+constexpr int64_t kFwdRowsMin = 5 << 20;  // destination voxels from which a thread walks four rows
+
+template <typename T, int kRows>
 __global__ void __launch_bounds__(256) k_resample_fwd(const float* __restrict__ src, ResGeo G,
                                                       float* __restrict__ dst) {
     pdl_enter();
     const ResAxis &AX = G.a[0], &AY = G.a[1], &AZ = G.a[2];
-    const int64_t n = int64_t(AX.n_dst) * AY.n_dst * AZ.n_dst;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n;
-         t += int64_t(gridDim.x) * blockDim.x) {
-        const int x = static_cast<int>(t % AX.n_dst);
-        const int y = static_cast<int>((t / AX.n_dst) % AY.n_dst);
-        const int z = static_cast<int>(t / (int64_t(AX.n_dst) * AY.n_dst));
-        int x0, x1, y0, y1, z0, z1;
-        float wx, wy, wz;
-        res_map(AX, x, x0, x1, wx);
-        res_map(AY, y, y0, y1, wy);
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= AX.n_dst) return;
+    int x0, x1;
+    float wx;
+    res_map(AX, x, x0, x1, wx);
+    const float ux = 1.0f - wx;
+    const T sx = T(AX.n_src), sxy = sx * T(AY.n_src);
+    for (int z = blockIdx.z; z < AZ.n_dst; z += gridDim.z) {
+        int z0, z1;
+        float wz;
         res_map(AZ, z, z0, z1, wz);
-        const int64_t sx = AX.n_src, sxy = int64_t(AX.n_src) * AY.n_src;
-        const float* p00 = src + z0 * sxy + y0 * sx;
-        const float* p01 = src + z0 * sxy + y1 * sx;
-        const float* p10 = src + z1 * sxy + y0 * sx;
-        const float* p11 = src + z1 * sxy + y1 * sx;
-        const float ux = 1.0f - wx, uy = 1.0f - wy, uz = 1.0f - wz;
-        const float r00 = fmaf(wx, p00[x1], ux * p00[x0]);
-        const float r01 = fmaf(wx, p01[x1], ux * p01[x0]);
-        const float r10 = fmaf(wx, p10[x1], ux * p10[x0]);
-        const float r11 = fmaf(wx, p11[x1], ux * p11[x0]);
-        const float s0 = fmaf(wy, r01, uy * r00);
-        const float s1 = fmaf(wy, r11, uy * r10);
-        dst[t] = fmaf(wz, s1, uz * s0);
+        const float uz = 1.0f - wz;
+        const T a0 = T(z0) * sxy + T(x0), a1 = T(z1) * sxy + T(x0);  // sample x0 of row 0 in each plane
+        const T dx = T(x1) - T(x0);
+        const int64_t out = int64_t(z) * AY.n_dst * AX.n_dst + x;
+        for (int yb = (blockIdx.y * blockDim.y + threadIdx.y) * kRows; yb < AY.n_dst;
+             yb += gridDim.y * blockDim.y * kRows) {
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                const int y = yb + r;
+                if (y >= AY.n_dst) break;
+                int y0, y1;
+                float wy;
+                res_map(AY, y, y0, y1, wy);
+                const T b0 = T(y0) * sx, b1 = T(y1) * sx;
+                const float uy = 1.0f - wy;
+                const float r00 = fmaf(wx, src[a0 + b0 + dx], ux * src[a0 + b0]);
+                const float r01 = fmaf(wx, src[a0 + b1 + dx], ux * src[a0 + b1]);
+                const float r10 = fmaf(wx, src[a1 + b0 + dx], ux * src[a1 + b0]);
+                const float r11 = fmaf(wx, src[a1 + b1 + dx], ux * src[a1 + b1]);
+                const float s0 = fmaf(wy, r01, uy * r00);
+                const float s1 = fmaf(wy, r11, uy * r10);
+                dst[out + int64_t(y) * AX.n_dst] = fmaf(wz, s1, uz * s0);
+            }
+        }
     }
 }
 
@@ -287,18 +307,35 @@ static unsigned res_blocks(int64_t n) {
 gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t snx, float* dst,
                             int32_t dnz, int32_t dny, int32_t dnx, cudaStream_t st) {
     const ResGeo G = make_res(snz, sny, snx, dnz, dny, dnx);
-    launch_k(k_resample_fwd, dim3(res_blocks(int64_t(dnz) * dny * dnx)), dim3(256), 0, st, src, G,
-        dst);
+    // columns in whole warps, the rest of the block's threads over rows
+    const bool narrow = int64_t(snz) * sny * snx <= (int64_t(1) << 31) - 1;
+    const bool rows4 = int64_t(dnz) * dny * dnx >= kFwdRowsMin;
+    const int tx = dnx >= 256 ? 256 : (dnx + 31) / 32 * 32, ty = 256 / tx, per = ty * (rows4 ? 4 : 1);
+    const int64_t gx = (int64_t(dnx) + tx - 1) / tx, gy = (int64_t(dny) + per - 1) / per;
+    const dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy < 65535 ? gy : 65535),
+                    static_cast<unsigned>(dnz < 65535 ? dnz : 65535));
+    launch_k(narrow ? (rows4 ? k_resample_fwd<unsigned, 4> : k_resample_fwd<unsigned, 1>)
+                    : (rows4 ? k_resample_fwd<int64_t, 4> : k_resample_fwd<int64_t, 1>),
+        grid, dim3(tx, ty), 0, st, src, G, dst);
     return last_launch_status();
 }
 
-// Separable form of the adjoint for one source plane z and a tile of kPlaneRows source rows:
-// first U[y][jx] = sum over the z and y runs of w_z w_y dL/dLR[jz][jy][jx] for every LR column
-// jx (shared memory), then each voxel sums its x run over U[y]. Fixed order: z, then y
-// (inside U), then x.
-template <bool kPrep, int K, int kPlaneRows>
+// Separable form of the adjoint for a tile of kRows source rows on each of up to kPlanes source planes
+// z, in shared memory: V[j][jx] = sum over the z run of w_z dL/dLR[jz][jy][jx] for the LR rows jy that the tile's
+// rows read (each LR value is loaded once per tile), U[y][jx] = sum over the y run of w_y V, then
+// each voxel sums its x run over U[y]. Fixed order: z, then y, then x. A thread owns kV consecutive x
+// of every (256 / threads per row)-th row: its x runs stay in registers, and with kV = 4 (rows of
+// whole, aligned quads) I, W and the factors move by 16-byte accesses. Bound by HBM where it forms
+// the adjoint render's factors (143 MB at 240 x 240 x 155 from 100^3: 21 us at the copy bandwidth).
+// With z and y taps gathered per (y, jx) from global memory, one voxel per thread, an index
+// division per voxel and 1,240 blocks for 1,216 resident ones it took 62 us (26 us without the
+// factors); 36 (16) us now. Tiles of 16 (24, 48) rows took 41 (43, 44) us; one plane per block,
+// which forms the x runs twice as often, 38 us; kept where two would leave SMs idle.
+constexpr int kPlanes = 2;
+
+template <bool kPrep, int K, int kRows, int kV>
 __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restrict__ ddst, ResGeo G,
-                                                            const float* __restrict__ Iv,
+                                                            int v_rows, int per, const float* __restrict__ Iv,
                                                             const float* __restrict__ Wv, float eps,
                                                             float* __restrict__ dsrc,
                                                             float2* __restrict__ aip) {
@@ -308,13 +345,15 @@ __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restr
     const int nx = AX.n_src, ny = AY.n_src;
     const int lnx = AX.n_dst, lny = AY.n_dst;
     ResRun<K>* xt = reinterpret_cast<ResRun<K>*>(res_smem);
-    ResRun<K>* yt = xt + nx;                                // kPlaneRows entries
-    float* U = reinterpret_cast<float*>(yt + kPlaneRows);  // [kPlaneRows][lnx]
-    __shared__ ResRun<K> zr;
-    const int z = blockIdx.x;
-    const int y0 = blockIdx.y * kPlaneRows;
-    const int rows = min(kPlaneRows, ny - y0);
-    for (int e = threadIdx.x; e < nx + rows + 1; e += blockDim.x) {
+    ResRun<K>* yt = xt + nx;                           // kRows entries
+    float* U = reinterpret_cast<float*>(yt + kRows);  // [kRows][lnx]
+    float* V = U + kRows * lnx;                       // [v_rows][lnx]
+    __shared__ ResRun<K> zt[kPlanes];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int y0 = blockIdx.y * kRows;
+    const int rows = min(kRows, ny - y0);
+    const int zb = blockIdx.x * per, planes = min(per, AZ.n_src - zb);  // per <= kPlanes
+    for (int e = tid; e < nx + rows + planes; e += 256) {
         ResRun<K> rr;
         if (e < nx) {
             res_list<K>(AX, e, rr.j0, rr.n, rr.w);
@@ -323,69 +362,110 @@ __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restr
             res_list<K>(AY, y0 + (e - nx), rr.j0, rr.n, rr.w);
             yt[e - nx] = rr;
         } else {
-            res_list<K>(AZ, z, rr.j0, rr.n, rr.w);
-            zr = rr;
+            res_list<K>(AZ, zb + (e - nx - rows), rr.j0, rr.n, rr.w);
+            zt[e - nx - rows] = rr;
         }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < rows * lnx; e += blockDim.x) {
-        const int r = e / lnx, jx = e - r * lnx;
-        const ResRun<K>& ry = yt[r];
-        float acc = 0.0f;
+    const int groups = (nx + kV - 1) / kV;  // kV divides nx where kV > 1
+    const int per_row = groups >= 256 ? 256 : (groups + 31) / 32 * 32;
+    const int step = 256 / per_row, ty = tid / per_row;
+    for (int z = zb; z < zb + planes; ++z) {
+        const ResRun<K> zr = zt[z - zb];
+        // LR rows of the tile: runs start in ascending order, so rows jf .. jf + nv - 1 (v_rows bounds them)
+        const int jf = min(yt[0].j0, lny - 1);
+        const int nv = min(min(yt[rows - 1].j0 + K, lny) - jf, v_rows);
+        for (int r = warp; r < nv; r += 8)
+            for (int jx = lane; jx < lnx; jx += 32) {
+                float acc = 0.0f;
 #pragma unroll
-        for (int a = 0; a < K; ++a) {
-            if (a >= zr.n) break;
+                for (int a = 0; a < K; ++a)
+                    if (a < zr.n) acc = fmaf(zr.w[a], ddst[(int64_t(zr.j0 + a) * lny + jf + r) * lnx + jx], acc);
+                V[r * lnx + jx] = acc;
+            }
+        __syncthreads();
+        for (int r = warp; r < rows; r += 8) {
+            const ResRun<K> ry = yt[r];
+            for (int jx = lane; jx < lnx; jx += 32) {
+                float acc = 0.0f;
 #pragma unroll
-            for (int b = 0; b < K; ++b) {
-                if (b >= ry.n) break;
-                acc = fmaf(zr.w[a] * ry.w[b], ddst[(int64_t(zr.j0 + a) * lny + (ry.j0 + b)) * lnx + jx], acc);
+                for (int b = 0; b < K; ++b)
+                    if (b < ry.n) acc = fmaf(ry.w[b], V[min(ry.j0 + b - jf, v_rows - 1) * lnx + jx], acc);
+                U[r * lnx + jx] = acc;
             }
         }
-        U[e] = acc;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < rows * nx; e += blockDim.x) {
-        const int r = e / nx, x = e - r * nx;
-        const ResRun<K>& rx = xt[x];
-        const float* u = U + r * lnx + rx.j0;
-        float acc = 0.0f;
+        __syncthreads();
+        for (int gx = tid - ty * per_row; ty < step && gx < groups; gx += per_row) {
+            ResRun<K> rx[kV];
 #pragma unroll
-        for (int c = 0; c < K; ++c) {
-            if (c >= rx.n) break;
-            acc = fmaf(rx.w[c], u[c], acc);
-        }
-        const int64_t v = (int64_t(z) * ny + (y0 + r)) * nx + x;
-        if (kPrep) {
-            const float w = Wv[v];
-            const float al = acc / (w > eps ? w : eps);
-            aip[v] = make_float2(al, (w > eps) ? al * Iv[v] : 0.0f);
-        } else {
-            dsrc[v] = acc;
+            for (int e = 0; e < kV; ++e) rx[e] = xt[gx * kV + e];
+#pragma unroll 2
+            for (int r = ty; r < rows; r += step) {
+                const float* u = U + r * lnx;
+                float acc[kV];
+#pragma unroll
+                for (int e = 0; e < kV; ++e) {
+                    acc[e] = 0.0f;
+#pragma unroll
+                    for (int c = 0; c < K; ++c)
+                        if (c < rx[e].n) acc[e] = fmaf(rx[e].w[c], u[rx[e].j0 + c], acc[e]);
+                }
+                const int64_t v = (int64_t(z) * ny + (y0 + r)) * nx + gx * kV;
+                if constexpr (kPrep) {
+                    float w[kV], iv[kV];
+                    float2 a[kV];
+                    if constexpr (kV == 4) {
+                        load4<true>(Wv + v, w);
+                        load4<true>(Iv + v, iv);
+                    } else {
+                        w[0] = Wv[v];
+                        iv[0] = Iv[v];
+                    }
+#pragma unroll
+                    for (int e = 0; e < kV; ++e) a[e] = adj_factor(acc[e], w[e], iv[e], eps);
+                    if constexpr (kV == 4) {
+                        reinterpret_cast<float4*>(aip + v)[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+                        reinterpret_cast<float4*>(aip + v)[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
+                    } else {
+                        aip[v] = a[0];
+                    }
+                } else if constexpr (kV == 4) {
+                    store4<true>(dsrc + v, acc);
+                } else {
+                    dsrc[v] = acc[0];
+                }
+            }
         }
     }
 }
 
-constexpr int kPlaneSmem = 48 * 1024;
+constexpr int kPlaneSmem = 48 * 1024 - 512;  // (the kernel also holds the z run)
+
+// Rows per tile: the more, the fewer LR values are read again, but the fewer blocks there are and the
+// more shared memory each takes.
+template <bool kPrep, int K, int kRows>
+static bool launch_adj_plane_rows(const float* dd, const ResGeo& G, const float* I, const float* W, float eps,
+                                  float* dsrc, float2* aip, cudaStream_t st) {
+    const int nx = G.a[0].n_src, ny = G.a[1].n_src, nz = G.a[2].n_src, lnx = G.a[0].n_dst;
+    // LR rows that a tile's rows read: first samples of consecutive rows are n_dst / n_src apart on
+    // average, each within two samples of its exact position
+    const int v_rows = static_cast<int>((kRows - 1) * G.a[1].inv) + 5 + K;
+    const size_t smem = sizeof(ResRun<K>) * (size_t(nx) + kRows) + sizeof(float) * lnx * (size_t(kRows) + v_rows);
+    const int64_t tiles = (ny + kRows - 1) / kRows;
+    if (smem > size_t(kPlaneSmem) || tiles > 65535) return false;
+    const int per = nz * tiles >= 152 * 6 ? kPlanes : 1;
+    const bool vec = nx % 4 == 0 && (kPrep ? aligned16(I) && aligned16(W) && aligned16(aip) : aligned16(dsrc));
+    launch_k(vec ? k_resample_adj_plane<kPrep, K, kRows, 4> : k_resample_adj_plane<kPrep, K, kRows, 1>,
+        dim3(static_cast<unsigned>((nz + per - 1) / per), static_cast<unsigned>(tiles)), dim3(256), smem, st, dd,
+        G, v_rows, per, I, W, eps, dsrc, aip);
+    return true;
+}
 
 template <bool kPrep, int K>
 static bool launch_adj_plane_k(const float* dd, const ResGeo& G, const float* I, const float* W,
                                float eps, float* dsrc, float2* aip, cudaStream_t st) {
-    const int nx = G.a[0].n_src, ny = G.a[1].n_src, nz = G.a[2].n_src, lnx = G.a[0].n_dst;
-    const size_t base = sizeof(ResRun<K>) * size_t(nx);
-    if (nz > 65535) return false;
-    if (base + (sizeof(ResRun<K>) + sizeof(float) * lnx) * 32 <= size_t(kPlaneSmem)) {
-        const size_t smem = base + (sizeof(ResRun<K>) + sizeof(float) * lnx) * 32;
-        launch_k(k_resample_adj_plane<kPrep, K, 32>, dim3(dim3(nz, (ny + 31) / 32)), dim3(256),
-            smem, st, dd, G, I, W, eps, dsrc, aip);
-        return true;
-    }
-    if (base + (sizeof(ResRun<K>) + sizeof(float) * lnx) * 8 <= size_t(kPlaneSmem)) {
-        const size_t smem = base + (sizeof(ResRun<K>) + sizeof(float) * lnx) * 8;
-        launch_k(k_resample_adj_plane<kPrep, K, 8>, dim3(dim3(nz, (ny + 7) / 8)), dim3(256), smem,
-            st, dd, G, I, W, eps, dsrc, aip);
-        return true;
-    }
-    return false;
+    return launch_adj_plane_rows<kPrep, K, 32>(dd, G, I, W, eps, dsrc, aip, st) ||
+           launch_adj_plane_rows<kPrep, K, 8>(dd, G, I, W, eps, dsrc, aip, st);
 }
 
 template <bool kPrep>
