@@ -158,6 +158,18 @@ gs_status gs_bin_bricks(const float* params, const gs_grid* grid, const gs_confi
 gs_status gs_render_fwd(const gs_bins* bins, const gs_grid* grid, const gs_config* cfg,
                         float* I, float* W, unsigned long long* d_stats, gs_stream stream);
 
+/* gs_bin_bricks and gs_render_fwd for a caller that has to know whether the pairs fitted: bins,
+ * renders, and returns when the pair count is known on the host (*h_npairs, host int64), without
+ * waiting for the render. Up to 2^25 voxels the render is queued before the count is known, so the
+ * GPU does not wait for the host. Returns GS_ERR_CAPACITY when *h_npairs exceeds bins->capacity: the
+ * lists are then empty, and I, W and d_stats hold nothing of use (grow the bins and call again).
+ * Arguments as in the two calls. Not for use under stream capture (it waits for an event). The first
+ * call of a thread on a device creates 8 bytes of page-locked memory and an event, which the thread
+ * keeps until it ends. */
+gs_status gs_render_cloud(const float* params, const gs_grid* grid, const gs_config* cfg,
+                          gs_bins* bins, void* ws, size_t ws_bytes, float* I, float* W,
+                          unsigned long long* d_stats, int64_t* h_npairs, gs_stream stream);
+
 /* Eq. 5-6 adjoint of the forward render and the chain to the raw parameters.
  * params: device float [n_gauss, 12] (the ones binned); I, W: the forward outputs;
  * dI: device float [nz, ny, nx], dL/dI; dparams: device float [n_gauss, 12], overwritten

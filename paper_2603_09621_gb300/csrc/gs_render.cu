@@ -852,6 +852,65 @@ extern "C" gs_status gs_render_fwd(const gs_bins* bins, const gs_grid* grid, con
     return render_fwd_impl(bins, grid, cfg, I, W, d_stats, reinterpret_cast<cudaStream_t>(stream));
 }
 
+namespace {
+
+// A thread's page-locked word and event of each device, for reading a pair count back while later
+// work of the stream runs on; given back when the thread ends.
+constexpr int kMaxDevices = 64;
+
+struct CountSlot {
+    int64_t* host = nullptr;
+    cudaEvent_t copied = nullptr;
+    ~CountSlot() {
+        if (copied) (void)cudaEventDestroy(copied);
+        if (host) (void)cudaFreeHost(host);
+    }
+};
+
+CountSlot* count_slot() {
+    static thread_local CountSlot slots[kMaxDevices];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    CountSlot& s = slots[dev];
+    if (!s.host && cudaMallocHost(reinterpret_cast<void**>(&s.host), sizeof(int64_t)) != cudaSuccess) {
+        s.host = nullptr;
+        return nullptr;
+    }
+    if (!s.copied && cudaEventCreateWithFlags(&s.copied, cudaEventDisableTiming) != cudaSuccess) {
+        s.copied = nullptr;
+        return nullptr;
+    }
+    return &s;
+}
+
+// Voxels up to which the forward is queued before the pairs are known to fit: if they do not, it
+// writes 8 bytes per voxel in vain (about 40 us at this size), else the GPU does not idle while the host
+// reads the count and launches it (about 15 us).
+constexpr int64_t kSpeculateVoxels = int64_t(1) << 25;
+
+}  // namespace
+
+extern "C" gs_status gs_render_cloud(const float* params, const gs_grid* grid, const gs_config* cfg,
+                                     gs_bins* bins, void* ws, size_t ws_bytes, float* I, float* W,
+                                     unsigned long long* d_stats, int64_t* h_npairs, gs_stream stream) {
+    if (!h_npairs || !I || !W) return GS_ERR_INVALID_ARG;
+    gs_status s = gs_bin_bricks(params, grid, cfg, bins, ws, ws_bytes, stream);
+    if (s != GS_OK) return s;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    CountSlot* slot = count_slot();
+    if (!slot ||
+        cudaMemcpyAsync(slot->host, bins->d_npairs, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaEventRecord(slot->copied, st) != cudaSuccess)
+        return GS_ERR_CUDA;
+    const bool early = int64_t(grid->nx) * grid->ny * grid->nz <= kSpeculateVoxels;
+    if (early) s = render_fwd_impl(bins, grid, cfg, I, W, d_stats, st);
+    if (cudaEventSynchronize(slot->copied) != cudaSuccess) return GS_ERR_CUDA;
+    *h_npairs = *static_cast<volatile int64_t*>(slot->host);
+    if (s != GS_OK) return s;
+    if (*h_npairs > bins->capacity) return GS_ERR_CAPACITY;
+    return early ? GS_OK : render_fwd_impl(bins, grid, cfg, I, W, d_stats, st);
+}
+
 extern "C" gs_status gs_render_bwd(const float* params, const gs_bins* bins, const gs_grid* grid,
                                    const gs_config* cfg, const float* I, const float* W,
                                    const float* dI, float* dparams, void* ws, size_t ws_bytes,

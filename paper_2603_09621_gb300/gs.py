@@ -123,6 +123,7 @@ SIGNATURES = {
     "gs_signal_proxy": (ctypes.c_int, [_P, _P, _I64, _F, _F, _P, _P]),
     "gs_bin_bricks": (ctypes.c_int, [_P, _P, _P, _P, _P, _SZ, _P]),
     "gs_render_fwd": (ctypes.c_int, [_P, _P, _P, _P, _P, _P, _P]),
+    "gs_render_cloud": (ctypes.c_int, [_P, _P, _P, _P, _P, _SZ, _P, _P, _P, _P, _P]),
     "gs_render_bwd": (ctypes.c_int, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _SZ, _P]),
     "gs_downsample_fwd": (ctypes.c_int, [_P, _I32, _I32, _I32, _I32, _P, _P]),
     "gs_downsample_bwd": (ctypes.c_int, [_P, _I32, _I32, _I32, _I32, _P, _P]),
@@ -289,8 +290,7 @@ class Bins:
     def _view(self, addr, count, dtype):
         base = self.arena.data_ptr()
         off = addr - base
-        esz = torch.empty((), dtype=dtype).element_size()
-        return self.arena[off:off + count * esz].view(dtype)
+        return self.arena[off:off + count * dtype.itemsize].view(dtype)
 
     def brick_off(self):
         return self._view(self.c.brick_off, self.c.n_bricks + 1, torch.int32)
@@ -484,22 +484,42 @@ def gs_status_read(bins: Bins, stream=None) -> tuple[int, int]:
 
 
 # ---------------------------------------------------------------------- composite helpers
+def gs_render_cloud(params: torch.Tensor, grid: Grid, cfg: Config, bins: Bins, ws: Workspace, I, W,
+                    stats=None, stream=None) -> int:
+    """Bin and render; returns the pairs needed once they are known (the render may still run).
+    More than bins.capacity: nothing was rendered."""
+    assert params.is_contiguous() and params.dtype == torch.float32
+    g, c = grid.c(), cfg.c()
+    need = ctypes.c_int64(0)
+    rc = load().gs_render_cloud(_ptr(params), ctypes.byref(g), ctypes.byref(c), ctypes.byref(bins.c),
+                                _ptr(ws.buf), ws.nbytes, _ptr(I), _ptr(W), _ptr(stats),
+                                ctypes.byref(need), _stream(stream))
+    if STATUS.get(rc) != "GS_ERR_CAPACITY":
+        _check(rc, "gs_render_cloud")
+    return need.value
+
+
 def render(params: torch.Tensor, grid: Grid, cfg: Config = Config(), capacity: int | None = None,
            stats: torch.Tensor | None = None, stream=None):
     """Bin and render a cloud. Grows the pair capacity (one host read) if it overflows.
     Returns (I, W, bins, workspace)."""
-    n = params.shape[0]
-    cap = capacity if capacity is not None else max(1024, 16 * n)
+    n, dev = params.shape[0], params.device
+    # 16 pairs per Gaussian; small clouds, whose retry costs more than their memory (72 bytes per
+    # pair), get up to 64
+    cap = capacity if capacity is not None else max(1024, 16 * n, min(64 * n, 1 << 20))
+    I = torch.empty(grid.shape, dtype=torch.float32, device=dev)
+    W = torch.empty(grid.shape, dtype=torch.float32, device=dev)
+    spent = None
     while True:
-        bins = Bins(n, cap, grid, cfg, params.device)
-        ws = Workspace(n, cap, grid, cfg, params.device)
-        gs_bin_bricks(params, grid, cfg, bins, ws, stream)
-        need = bins.npairs()
+        bins = Bins(n, cap, grid, cfg, dev)
+        ws = Workspace(n, cap, grid, cfg, dev)
+        need = gs_render_cloud(params, grid, cfg, bins, ws, I, W, stats, stream)
         if need <= cap:
-            break
+            return I, W, bins, ws
+        # on a stream that is not the allocator's, kernels may still read the small bins until the
+        # next count is known
+        spent = (bins, ws) if stream is not None else None  # noqa: F841 (kept alive)
         cap = int(need * 1.25) + 1024
-    I, W = gs_render_fwd(bins, grid, cfg, stats=stats, stream=stream)
-    return I, W, bins, ws
 
 
 class GaussianRender(torch.autograd.Function):
