@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
 
 #include "gs_common.cuh"
 
@@ -179,7 +180,7 @@ __device__ __forceinline__ unsigned foot_mask(const Rec& R, const RenderGeo& G, 
 
 // ------------------------------------------------------------------------ forward
 
-// One block of 32 or 64 threads per brick. What bounds it is instruction issue (72 % active) and
+// One block of 32 or 64 threads per brick (kWide: a warp per footprint, below). What bounds it is instruction issue (72 % active) and
 // the latency of the gathered records, so work per instruction decides:
 //   - A quarter-warp per 4^3 footprint, a lane owning the x-rows at z and z + 1: the row terms,
 //     offsets and exponents of the two rows run as FP32x2 pairs (element by element the scalar
@@ -200,10 +201,19 @@ __device__ __forceinline__ unsigned foot_mask(const Rec& R, const RenderGeo& G, 
 //     records 212 us and 5.20 ms; 24 records 207 us but 5.50 ms; 64 registers (spills) 216 us;
 //     96 registers 217 us. Rounds double-buffered with cp.async measured slower (242 against
 //     241 us, 7.06 against 6.13 ms).
+// A grid of few bricks leaves most schedulers with one warp or none, and a brick's time is the latency
+// of its lists. There (kWide) a footprint gets a whole warp, each lane the two voxels at z and z + 1,
+// and a thread fetches its record of the next round while the present one is evaluated. Forward us,
+// narrow -> wide: 8 bricks of 8^3 25 -> 21, 64 bricks 33-38 -> 26-28 (random and clustered clouds), 216
+// bricks 35-46 -> 34-36, but 512 bricks 41-53 -> 51-56 and 4,096 bricks 146 -> 270: a lane with one
+// voxel per row repeats the row terms four times as often. 8 x 8 x 4 bricks: 128 of them 36-42 ->
+// 24-26, 1,024 43-64 -> 48-54. So wide where all footprints' warps are resident at once (152 SMs of 2
+// blocks of 8 warps: 304 bricks of 8^3, 608 of 8 x 8 x 4). Eight hits per iteration 1-2 us slower.
+constexpr int64_t kWideFootprints = 152 * 16;
 constexpr int kFwdHits = 4;  // hits per iteration of the evaluation loop (one 32-bit list word)
 
-template <bool kStats, int kChunk>
-__global__ void __launch_bounds__(64, 14) k_render_fwd(const int32_t* __restrict__ brick_off,
+template <bool kStats, int kChunk, bool kWide>
+__global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd(const int32_t* __restrict__ brick_off,
                                                        const int32_t* __restrict__ pair_gid,
                                                        const float4* __restrict__ rec4, RenderGeo G,
                                                        float* __restrict__ I, float* __restrict__ W,
@@ -219,59 +229,78 @@ __global__ void __launch_bounds__(64, 14) k_render_fwd(const int32_t* __restrict
     const int b = blockIdx.x;
     int bx, by, bz;
     brick_xyz(b, G, bx, by, bz);
-    // quarter-warp per 4^3 footprint; a lane owns two x-rows of 4 voxels, at z and z + 1
-    const int foot = tid >> 3, l8 = lane & 7, foot0 = (tid >> 5) * 4;
+    // quarter-warp per 4^3 footprint, a lane owns two x-rows of 4 voxels, at z and z + 1; kWide: a
+    // warp per footprint, a lane owns voxel lx of the two rows
+    constexpr int kFoot = kWide ? 1 : 4;  // footprints per warp
+    constexpr int kX = kWide ? 1 : 4;     // voxels of a row per lane
+    const int foot = tid / (32 / kFoot), foot0 = (tid >> 5) * kFoot;
+    const int lx = kWide ? lane & 3 : 0, lyz = kWide ? lane >> 2 : lane & 7;
     const int n_foot = G.fx * G.fy * G.fz;
     const bool foot_ok = foot < n_foot;
     const int f = foot_ok ? foot : 0;
     const int wx = f % G.fx, wy = (f / G.fx) % G.fy, wz = f / (G.fx * G.fy);
     const int x0 = bx * G.bsx, y0 = by * G.bsy, z0 = bz * G.bsz;
     const int ox = x0 + wx * 4, oy = y0 + wy * 4, oz = z0 + wz * 4;
-    const int y = oy + (l8 & 3), z = oz + 2 * (l8 >> 2);
+    const int y = oy + (lyz & 3), z = oz + 2 * (lyz >> 2);
     const float fy = float(y);
     const float2 fz2 = f2(float(z), float(z + 1));
     if (tid < 4) srec[tid][kChunk] = make_float4(0.f, 0.f, 0.f, 0.f);
 
-    float2 SWa[4], SWb[4];  // (S, W) of the lane's voxels in its two rows
+    float2 SWa[kX], SWb[kX];  // (S, W) of the lane's voxels in its two rows
 #pragma unroll
-    for (int xi = 0; xi < 4; ++xi) SWa[xi] = SWb[xi] = f2(0.f, 0.f);
+    for (int xi = 0; xi < kX; ++xi) SWa[xi] = SWb[xi] = f2(0.f, 0.f);
     unsigned long long n_eff = 0, n_eval = 0;
     const int start = brick_off[b], end = brick_off[b + 1];
+    // kWide: a thread stages at most one record per round, loaded while the round before is evaluated
+    float4 q[REC_F4];
+    auto fetch = [&](int k, int c0) {
+        const float4* src = rec4 + int64_t(pair_gid[c0 + k]) * REC_F4;
+#pragma unroll
+        for (int part = 0; part < REC_F4; ++part) q[part] = src[part];
+    };
+    auto put = [&](int k) {  // a thread culls and stages one record
+        const Rec R = load_rec(q);
+        const unsigned m = (G.fx == 2 && G.fy == 2 && G.fz == 2) ? foot_mask<2, 2, 2>(R, G, x0, y0, z0)
+                           : (G.fx == 2 && G.fy == 2 && G.fz == 1)
+                               ? foot_mask<2, 2, 1>(R, G, x0, y0, z0)
+                               : foot_mask<0, 0, 0>(R, G, x0, y0, z0);
+        sfoot[k] = static_cast<unsigned char>(m);
+        srec[0][k] = q[0];
+        srec[1][k] = q[1];
+        srec[2][k] = q[2];
+        srec[3][k] = q[4];
+    };
+    if (kWide && start + tid < end && tid < kChunk) fetch(tid, start);
     for (int c0 = start; c0 < end; c0 += kChunk) {
         const int cnt = min(kChunk, end - c0);
         if (c0 != start) __syncthreads();  // the previous chunk's records are no longer read
-        for (int k = tid; k < cnt; k += nthreads) {  // a thread stages and culls one record
-            const float4* src = rec4 + int64_t(pair_gid[c0 + k]) * REC_F4;
-            float4 q[REC_F4];
-#pragma unroll
-            for (int part = 0; part < REC_F4; ++part) q[part] = src[part];
-            const Rec R = load_rec(q);
-            const unsigned m = (G.fx == 2 && G.fy == 2 && G.fz == 2) ? foot_mask<2, 2, 2>(R, G, x0, y0, z0)
-                               : (G.fx == 2 && G.fy == 2 && G.fz == 1)
-                                   ? foot_mask<2, 2, 1>(R, G, x0, y0, z0)
-                                   : foot_mask<0, 0, 0>(R, G, x0, y0, z0);
-            sfoot[k] = static_cast<unsigned char>(m);
-            srec[0][k] = q[0];
-            srec[1][k] = q[1];
-            srec[2][k] = q[2];
-            srec[3][k] = q[4];
+        if (kWide) {
+            if (tid < cnt) put(tid);
+        } else {
+            for (int k = tid; k < cnt; k += nthreads) {
+                fetch(k, c0);
+                put(k);
+            }
         }
         __syncthreads();
-        // each warp lists the hits of its four footprints in ascending Gaussian id
-        int n[4] = {0, 0, 0, 0};
+        if (kWide && c0 + kChunk + tid < end && tid < kChunk) fetch(tid, c0 + kChunk);
+        // each warp lists the hits of its footprints in ascending Gaussian id
+        int n[kFoot] = {};
         for (int k0 = 0; k0 < cnt; k0 += 32) {
             const int k = k0 + lane;
             const unsigned m = (k < cnt ? static_cast<unsigned>(sfoot[k]) : 0u) >> foot0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < kFoot; ++j) {
                 const unsigned bal = __ballot_sync(0xffffffffu, (m >> j) & 1u);
                 if ((m >> j) & 1u)
                     slist[foot0 + j][n[j] + __popc(bal & ((1u << lane) - 1u))] = static_cast<unsigned char>(k);
                 n[j] += __popc(bal);
             }
         }
-        const int myn = (lane & 16) ? ((lane & 8) ? n[3] : n[2]) : ((lane & 8) ? n[1] : n[0]);
-        if (l8 < kFwdHits) slist[foot][myn + l8] = static_cast<unsigned char>(kChunk);
+        int myn = n[0];
+#pragma unroll
+        for (int j = 1; j < kFoot; ++j) myn = foot == foot0 + j ? n[j] : myn;
+        if (lyz < kFwdHits && lx == 0) slist[foot][myn + lyz] = static_cast<unsigned char>(kChunk);
         __syncwarp();
         for (int i = 0; i < myn; i += kFwdHits) {
             const unsigned slots = *reinterpret_cast<const unsigned*>(&slist[foot][i]);
@@ -290,8 +319,10 @@ __global__ void __launch_bounds__(64, 14) k_render_fwd(const int32_t* __restrict
                 const float2 tq0 = mul2(sa2, add2(f2(ux, ux), f2(-dxs.x, -dxs.y)));
                 const float2 vrr = f2(re.x, re.y);
 #pragma unroll
-                for (int xi = 0; xi < 4; ++xi) {
-                    const float2 tq = xi == 0 ? tq0 : fma2(f2(float(xi), float(xi)), sa2, tq0);
+                for (int xi = 0; xi < kX; ++xi) {
+                    // (k = 0 in the packed FMA gives tq0 itself)
+                    const float k = kWide ? float(lx) : float(xi);
+                    const float2 tq = (!kWide && xi == 0) ? tq0 : fma2(f2(k, k), sa2, tq0);
                     const float2 q = fma2(tq, tq, Sr);
                     if (q.x <= G.T) {
                         const float g = ex2_approx(-q.x);
@@ -303,7 +334,7 @@ __global__ void __launch_bounds__(64, 14) k_render_fwd(const int32_t* __restrict
                     }
                     if (kStats) {
                         const bool live = i + u < myn;
-                        const bool in = live && y < G.ny && ox + xi < G.nx;
+                        const bool in = live && y < G.ny && ox + lx + xi < G.nx;
                         n_eff += (in && z < G.nz && q.x <= G.T) ? 1 : 0;
                         n_eff += (in && z + 1 < G.nz && q.y <= G.T) ? 1 : 0;
                         n_eval += live ? 2 : 0;
@@ -315,25 +346,27 @@ __global__ void __launch_bounds__(64, 14) k_render_fwd(const int32_t* __restrict
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (!(foot_ok && y < G.ny && z + h < G.nz)) continue;
-        const int64_t row = (int64_t(z + h) * G.ny + y) * G.nx + ox;
-        float Iv[4], Wv[4];
+        const int64_t row = (int64_t(z + h) * G.ny + y) * G.nx + ox + lx;
+        float Iv[kX], Wv[kX];
 #pragma unroll
-        for (int xi = 0; xi < 4; ++xi) {
+        for (int xi = 0; xi < kX; ++xi) {
             const float S = h ? SWb[xi].x : SWa[xi].x;
             Wv[xi] = h ? SWb[xi].y : SWa[xi].y;
             Iv[xi] = S / (Wv[xi] > G.eps ? Wv[xi] : G.eps);
         }
-        if (ox + 3 < G.nx && (G.nx & 3) == 0) {
-            *reinterpret_cast<float4*>(I + row) = make_float4(Iv[0], Iv[1], Iv[2], Iv[3]);
-            *reinterpret_cast<float4*>(W + row) = make_float4(Wv[0], Wv[1], Wv[2], Wv[3]);
-        } else {
-#pragma unroll
-            for (int xi = 0; xi < 4; ++xi)
-                if (ox + xi < G.nx) {
-                    I[row + xi] = Iv[xi];
-                    W[row + xi] = Wv[xi];
-                }
+        if constexpr (!kWide) {
+            if (ox + 3 < G.nx && (G.nx & 3) == 0) {
+                store4<true>(I + row, Iv);
+                store4<true>(W + row, Wv);
+                continue;
+            }
         }
+#pragma unroll
+        for (int xi = 0; xi < kX; ++xi)
+            if (ox + lx + xi < G.nx) {
+                I[row + xi] = Iv[xi];
+                W[row + xi] = Wv[xi];
+            }
     }
     if (kStats) {
 #pragma unroll
@@ -778,20 +811,29 @@ gs_status render_fwd_impl(const gs_bins* bins, const gs_grid* grid, const gs_con
                           float* I, float* W, unsigned long long* stats, cudaStream_t st) {
     RenderGeo G = make_geo(grid, cfg);
     const int n_foot = G.fx * G.fy * G.fz;
-    const int threads = 32 * ((n_foot + 3) / 4);  // a quarter-warp per footprint
     // records staged per round about in proportion to the footprints (the lists of smaller
     // bricks are shorter), so that smaller bricks keep more blocks resident
     const float4* rec4 = reinterpret_cast<const float4*>(bins->rec);
+    const bool wide = int64_t(bins->n_bricks) * n_foot <= kWideFootprints;
+    // (wide: a thread per record of a round, so two warps also for a single footprint)
+    const int threads = wide ? 32 * (n_foot > 1 ? n_foot : 2) : 32 * ((n_foot + 3) / 4);
     auto go = [&](auto kernel) {
         launch_k(kernel, dim3(bins->n_bricks), dim3(threads), 0, st, bins->brick_off, bins->pair_gid,
             rec4, G, I, W, stats);
     };
+    auto pick = [&](auto chunk) {
+        constexpr int kChunk = decltype(chunk)::value;
+        if (wide)
+            stats ? go(k_render_fwd<true, kChunk, true>) : go(k_render_fwd<false, kChunk, true>);
+        else
+            stats ? go(k_render_fwd<true, kChunk, false>) : go(k_render_fwd<false, kChunk, false>);
+    };
     if (n_foot >= 6)
-        stats ? go(k_render_fwd<true, 8 * kFwdChunkPerFoot>) : go(k_render_fwd<false, 8 * kFwdChunkPerFoot>);
+        pick(std::integral_constant<int, 8 * kFwdChunkPerFoot>{});
     else if (n_foot >= 3)
-        stats ? go(k_render_fwd<true, 4 * kFwdChunkPerFoot>) : go(k_render_fwd<false, 4 * kFwdChunkPerFoot>);
+        pick(std::integral_constant<int, 4 * kFwdChunkPerFoot>{});
     else
-        stats ? go(k_render_fwd<true, 2 * kFwdChunkPerFoot>) : go(k_render_fwd<false, 2 * kFwdChunkPerFoot>);
+        pick(std::integral_constant<int, 2 * kFwdChunkPerFoot>{});
     return last_launch_status();
 }
 
