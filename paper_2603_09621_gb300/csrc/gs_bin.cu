@@ -363,7 +363,8 @@ constexpr long long kBadFlag = 1LL << 62;  // marks a Gaussian tile with an inva
 // sequences, so the extra resident warps pay more than the spills cost.
 // The block also stores its column of the first radix pass's digit counts (hist0[d * stride0 +
 // block]) and its number of pairs (blk[block]), kBadFlag added where a Gaussian was invalid.
-__global__ void __launch_bounds__(kGaussTile, 6) k_preprocess(
+template <int kTile>
+__global__ void __launch_bounds__(kTile, 6 * 256 / kTile) k_preprocess(
     const float* __restrict__ params, int64_t N, GridF G, float trunc_sigma, int signal_mode, int a_act,
     int t_act, float* __restrict__ rec, int32_t* __restrict__ brange, int nd, int32_t* __restrict__ hist0,
     int64_t stride0, long long* __restrict__ blk) {
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(kGaussTile, 6) k_preprocess(
     __shared__ int hcnt[kMaxDigits], hdif[kMaxDigits + 1], sscan[32];
     __shared__ int hall, flags;  // flags: 1 an invalid Gaussian, 2 a box of more than kBoxSerial bricks
     __shared__ unsigned long long btot;
-    for (int d = threadIdx.x; d <= nd; d += kGaussTile) {
+    for (int d = threadIdx.x; d <= nd; d += kTile) {
         if (d < nd) hcnt[d] = 0;
         hdif[d] = 0;
     }
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(kGaussTile, 6) k_preprocess(
         btot = 0;
     }
     __syncthreads();
-    const int64_t g = int64_t(blockIdx.x) * kGaussTile + threadIdx.x;
+    const int64_t g = int64_t(blockIdx.x) * kTile + threadIdx.x;
     BrickBox box;
     box.cnt = 0;
     bool bad = false;
@@ -420,7 +421,7 @@ __global__ void __launch_bounds__(kGaussTile, 6) k_preprocess(
         }
     }
     __syncthreads();
-    const int di = nd > kGaussTile ? nd / kGaussTile : 1;  // thread t stores digits [t di, (t + 1) di)
+    const int di = nd > kTile ? nd / kTile : 1;  // thread t stores digits [t di, (t + 1) di)
     int run = 0;
     if (flags & 2) {
         int v = 0, tot;
@@ -538,6 +539,8 @@ struct Scatter {
     const long long* blk_base;
     int64_t N;
     int nbx, nby;
+    int nb;                    // bricks
+    int32_t* brick_off;        // (a first pass that is the last)
 };
 
 // Stable scatter of one tile of up to kSortTile keys per round. Warp w owns a contiguous part of
@@ -546,7 +549,7 @@ struct Scatter {
 // then gives each digit's run inside the tile and each warp's start in it; the tile is placed in
 // shared memory sorted by digit, ties in tile order, and written out in that order, so consecutive
 // threads store consecutive addresses of a run.
-// kFirst: the tile is emitted by the block itself from its kGaussTile Gaussians' boxes (in rounds
+// kFirst: the tile is emitted by the block itself from its kTile Gaussians' boxes (in rounds
 // of kSortTile pairs; the digits' output positions advance from round to round), else it is one
 // tile of the previous pass's output. kLast: the pass stores the bins' per-pair arrays; every
 // other pass adds each key to the next pass's digit counts at its output position's tile (one
@@ -561,11 +564,11 @@ struct Scatter {
 // values loaded when the tile is placed 90 us and 3.17 ms; copied to shared memory
 // asynchronously during the ranking (here) 90 us and 3.01 ms; 5 (6) blocks per SM with spills 95
 // (97) us.
-template <bool kFirst, bool kLast>
+template <bool kFirst, bool kLast, int kTile>
 __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
     pdl_enter();
     constexpr int kWarps = kSortThreads / 32;
-    static_assert(kSortThreads == kGaussTile, "one thread per Gaussian of a tile");
+    static_assert(kSortThreads >= kTile, "one thread per Gaussian of a tile");
     extern __shared__ int smem[];
     const int nd = 1 << A.bits, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int* wcnt = smem;                 // [kWarps][nd]
@@ -584,7 +587,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
     int loc = 0;                                     // the thread's first pair in the block
     int gpos[kMaxDigits / kSortThreads] = {};        // the thread's digits' next output positions
     if (kFirst) {
-        const int64_t g = int64_t(blockIdx.x) * kGaussTile + tid;
+        const int64_t g = tid < kTile ? int64_t(blockIdx.x) * kTile + tid : A.N;
         if (g < A.N) {
             const int4 lo = reinterpret_cast<const int4*>(A.brange + g * 8)[0];
             const int4 hi = reinterpret_cast<const int4*>(A.brange + g * 8)[1];
@@ -599,6 +602,25 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
                                                   reinterpret_cast<unsigned*>(sscan), &tot);
         if (g < A.N) A.gm_off[g] = static_cast<int32_t>(static_cast<unsigned>(base) + pre);
         if (g == A.N - 1) A.gm_off[A.N] = static_cast<int32_t>(static_cast<unsigned>(base) + pre + box.cnt);
+        if (kLast && blockIdx.x == 0) {
+            // the only pass: a digit is a brick, so the digits' exclusive prefix is brick_off
+            const int di = nd > kSortThreads ? nd / kSortThreads : 1;
+            int row[kMaxDigits / kSortThreads], mine = 0, all;
+#pragma unroll
+            for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
+                const int d = tid * di + e;
+                row[e] = (P > 0 && e < di && d < nd) ? A.rowtot[d] : 0;
+                mine += row[e];
+            }
+            int run = block_exclusive_scan(mine, reinterpret_cast<int*>(sscan), &all);
+#pragma unroll
+            for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
+                const int d = tid * di + e;
+                if (e < di && d <= A.nb) A.brick_off[d] = run;
+                run += row[e];
+            }
+            if (tid == 0 && A.nb == nd) A.brick_off[nd] = all;
+        }
         if (P == 0) return;  // also when the pairs exceed the capacity
         loc = static_cast<int>(pre);
         total = static_cast<int>(tot);
@@ -705,7 +727,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
             const int key = skey[j];
             const int idx = sidx[j];
             const int2 v = kFirst ? make_int2(static_cast<int>(base) + c0 + idx,
-                                              static_cast<int>(blockIdx.x) * kGaussTile + sowner[idx])
+                                              static_cast<int>(blockIdx.x) * kTile + sowner[idx])
                                   : sval[idx];
             const int pos = goff[(key >> A.shift) & (nd - 1)] + j;
             A.keys_out[pos] = key;
@@ -916,8 +938,9 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         return GS_OK;
     }
     const int nd = 1 << ws.radix_bits, passes = ws.radix_passes;
-    const unsigned gb = static_cast<unsigned>((N + kGaussTile - 1) / kGaussTile);
-    launch_k(k_preprocess, dim3(gb), dim3(kGaussTile), 0, st, params, N, G, cfg->trunc_sigma,
+    const int gt = gauss_tile(N);
+    const unsigned gb = static_cast<unsigned>((N + gt - 1) / gt);
+    launch_k(gt == 64 ? k_preprocess<64> : k_preprocess<256>, dim3(gb), dim3(gt), 0, st, params, N, G, cfg->trunc_sigma,
         cfg->signal_mode, cfg->a_act, cfg->t_act, bins->rec, bins->brange, nd, ws.hist0, ws.stride0,
         ws.blk_base);
     gs_status s = last_launch_status();
@@ -966,14 +989,18 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         A.N = N;
         A.nbx = b.nbx;
         A.nby = b.nby;
-        void (*kern)(Scatter) = first ? (last ? k_radix_scatter<true, true> : k_radix_scatter<true, false>)
-                                      : (last ? k_radix_scatter<false, true> : k_radix_scatter<false, false>);
+        A.nb = bins->n_bricks;
+        A.brick_off = bins->brick_off;
+        void (*kern)(Scatter) = !first    ? (last ? k_radix_scatter<false, true, 256> : k_radix_scatter<false, false, 256>)
+                                : gt == 64 ? (last ? k_radix_scatter<true, true, 64> : k_radix_scatter<true, false, 64>)
+                                           : (last ? k_radix_scatter<true, true, 256> : k_radix_scatter<true, false, 256>);
         if (first || tiles > 0) {
             launch_k(kern, dim3(first ? gb : tiles), dim3(kSortThreads), smem, st, A);
             s = last_launch_status();
             if (s != GS_OK) return s;
         }
     }
+    if (passes == 1) return GS_OK;  // (brick_off is written by the pass)
     if (cap == 0)
         return cudaMemsetAsync(bins->brick_off, 0, off_bytes, st) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
     // enough threads for four keys each, at most eight blocks per SM

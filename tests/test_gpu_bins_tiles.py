@@ -1,5 +1,5 @@
 """Brick lists where the binning's tiles can go wrong, bit for bit against the oracle's
-specification: Gaussian tiles of 256, rounds of 2,048 pairs per tile, boxes of more than 64 bricks
+specification: Gaussian tiles of 64 and 256, rounds of 2,048 pairs per tile, boxes of more than 64 bricks
 (counted by rows and emitted by a warp), digit widths from one narrow pass to three passes."""
 import numpy as np
 import pytest
@@ -43,6 +43,19 @@ def test_bins_tiles(dims, brick, n):
     # narrow ones in the same warp
     wide = np.arange(0, n, 97)
     d["log_s"][wide] += np.log(np.linspace(3.0, 12.0, wide.size))[:, None].astype(np.float32)
+    _check(cloud_params(d), og, brick)
+
+
+@pytest.mark.parametrize("n", [38_911, 38_912, 38_913, 39_169])
+@pytest.mark.parametrize("dims,brick", [((13, 11, 10), (8, 8, 8)), ((64, 64, 64), (8, 8, 8)),
+                                        ((72, 64, 64), (8, 8, 8)), ((64, 64, 60), (4, 4, 4))])
+def test_bins_tile_sizes(dims, brick, n):
+    """The largest cloud in tiles of 64 Gaussians and the smallest in tiles of 256, at the edges of their
+    tiles, with one pass (offsets written by it) and two."""
+    import oracle
+    og = oracle.Grid(*dims)
+    d = inputs.gaussian_cloud(n, n, dims[::-1], scale_range=(0.5, 1.2))
+    d["log_s"][::4001] += 2.0
     _check(cloud_params(d), og, brick)
 
 
