@@ -252,13 +252,13 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
     unsigned long long n_eff = 0, n_eval = 0;
     const int start = brick_off[b], end = brick_off[b + 1];
     // kWide: a thread stages at most one record per round, loaded while the round before is evaluated
-    float4 q[REC_F4];
-    auto fetch = [&](int k, int c0) {
-        const float4* src = rec4 + int64_t(pair_gid[c0 + k]) * REC_F4;
+    float4 qw[kWide ? REC_F4 : 1];
+    auto fetch = [&](int gid, float4 (&q)[REC_F4]) {
+        const float4* src = rec4 + int64_t(gid) * REC_F4;
 #pragma unroll
         for (int part = 0; part < REC_F4; ++part) q[part] = src[part];
     };
-    auto put = [&](int k) {  // a thread culls and stages one record
+    auto put = [&](int k, const float4 (&q)[REC_F4]) {
         const Rec R = load_rec(q);
         const unsigned m = (G.fx == 2 && G.fy == 2 && G.fz == 2) ? foot_mask<2, 2, 2>(R, G, x0, y0, z0)
                            : (G.fx == 2 && G.fy == 2 && G.fz == 1)
@@ -270,20 +270,29 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
         srec[2][k] = q[2];
         srec[3][k] = q[4];
     };
-    if (kWide && start + tid < end && tid < kChunk) fetch(tid, start);
+    int gid = start + tid < end ? pair_gid[start + tid] : 0;  // the thread's next record
+    if constexpr (kWide) {
+        if (start + tid < end && tid < kChunk) fetch(gid, qw);
+    }
     for (int c0 = start; c0 < end; c0 += kChunk) {
         const int cnt = min(kChunk, end - c0);
         if (c0 != start) __syncthreads();  // the previous chunk's records are no longer read
-        if (kWide) {
-            if (tid < cnt) put(tid);
+        if constexpr (kWide) {
+            if (tid < cnt) put(tid, qw);
         } else {
             for (int k = tid; k < cnt; k += nthreads) {
-                fetch(k, c0);
-                put(k);
+                float4 q[REC_F4];
+                const int next = k + nthreads < cnt ? pair_gid[c0 + k + nthreads] : 0;
+                fetch(gid, q);
+                put(k, q);
+                gid = next;
             }
         }
         __syncthreads();
-        if (kWide && c0 + kChunk + tid < end && tid < kChunk) fetch(tid, c0 + kChunk);
+        if (c0 + kChunk + tid < end) gid = pair_gid[c0 + kChunk + tid];
+        if constexpr (kWide) {
+            if (c0 + kChunk + tid < end && tid < kChunk) fetch(gid, qw);
+        }
         // each warp lists the hits of its footprints in ascending Gaussian id
         int n[kFoot] = {};
         for (int k0 = 0; k0 < cnt; k0 += 32) {
@@ -298,8 +307,8 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
             }
         }
         int myn = n[0];
-#pragma unroll
-        for (int j = 1; j < kFoot; ++j) myn = foot == foot0 + j ? n[j] : myn;
+        if constexpr (!kWide)
+            myn = (lane & 16) ? ((lane & 8) ? n[3] : n[2]) : ((lane & 8) ? n[1] : n[0]);
         if (lyz < kFwdHits && lx == 0) slist[foot][myn + lyz] = static_cast<unsigned char>(kChunk);
         __syncwarp();
         for (int i = 0; i < myn; i += kFwdHits) {
