@@ -290,6 +290,13 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     return y;
 }
 
+// Approximate reciprocal square root (rsqrt.approx, flush-to-zero); for bounds that carry a margin.
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Four values, as one 16-byte access (kVec) or one by one.
 template <bool kVec>
 __device__ __forceinline__ void load4(const float* src, float (&d)[4]) {
