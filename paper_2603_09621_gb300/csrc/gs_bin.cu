@@ -94,7 +94,13 @@ struct GridF {
     int b[3];
     int nb[3];
     FastDiv db[3];  // division by the brick size along each axis
+    bool pow2[3];   // h is a power of two (and ih finite and exact): x / h and x ih round alike
 };
+
+// x / h_k correctly rounded.
+__device__ __forceinline__ float div_h(float x, const GridF& G, int k) {
+    return G.pow2[k] ? __fmul_rn(x, G.ih[k]) : __fdiv_rn(x, G.h[k]);
+}
 
 // Error-free sum (Knuth): s + e == a + b exactly, s = fl(a + b).
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -221,6 +227,7 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
     R[2][1] = __fmul_rn(2.0f, __fadd_rn(yz, wx));
     R[2][2] = __fsub_rn(1.0f, __fmul_rn(2.0f, __fadd_rn(xx, yy)));
     const float ksig = __fmul_rn(trunc_sigma, 1.0001220703125f);
+    float sd[3];  // standard deviations along the axes
     int lo[3], hi[3];
     bool inside = true;
 #pragma unroll
@@ -230,11 +237,10 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
         float sig = __fmul_rn(m0, m0);
         sig = __fadd_rn(sig, __fmul_rn(m1, m1));
         sig = __fadd_rn(sig, __fmul_rn(m2, m2));
-        float e = __fmul_rn(ksig, __fsqrt_rn(sig));
-        float lo_f = __fsub_rn(__fsub_rn(__fdiv_rn(__fsub_rn(__fsub_rn(p[k], e), G.o[k]), G.h[k]), 0.5f),
-                               0.00390625f);
-        float hi_f = __fadd_rn(__fsub_rn(__fdiv_rn(__fsub_rn(__fadd_rn(p[k], e), G.o[k]), G.h[k]), 0.5f),
-                               0.00390625f);
+        sd[k] = __fsqrt_rn(sig);
+        float e = __fmul_rn(ksig, sd[k]);
+        float lo_f = __fsub_rn(__fsub_rn(div_h(__fsub_rn(__fsub_rn(p[k], e), G.o[k]), G, k), 0.5f), 0.00390625f);
+        float hi_f = __fadd_rn(__fsub_rn(div_h(__fsub_rn(__fadd_rn(p[k], e), G.o[k]), G, k), 0.5f), 0.00390625f);
         float nmax = static_cast<float>(G.n[k] - 1);
         if (!(hi_f >= 0.0f) || !(lo_f <= nmax)) {
             inside = false;
@@ -307,7 +313,7 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
     for (int k = 0; k < 3; ++k) {
         float dh, dl;
         two_sum(p[k], -G.o[k], dh, dl);           // mu - o exactly
-        const float qh = __fdiv_rn(dh, G.h[k]);   // correctly rounded: the remainder is exact
+        const float qh = div_h(dh, G, k);         // correctly rounded: the remainder is exact
         const float rem = fmaf(-qh, G.h[k], dh);
         const float ql = __fmul_rn(__fadd_rn(rem, dl), G.ih[k]);
         float sh, sl;
@@ -339,12 +345,7 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
     // footprint's half-width: a footprint whose centre is farther along an axis is missed
     float ext[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        float sig = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) sig += (R[k][j] * s[j]) * (R[k][j] * s[j]);
-        ext[k] = 1.01f * trunc_sigma * sqrtf(sig) * G.ih[k] + 1.5f + 1e-3f;
-    }
+    for (int k = 0; k < 3; ++k) ext[k] = 1.01f * trunc_sigma * sd[k] * G.ih[k] + 1.5f + 1e-3f;
     r4[3] = make_float4(ext[0], rho4, ext[1], ext[2]);
     // lower bound of q per squared voxel distance from the mean: (log2 e / 2) h_min^2 / s_max^2
     // bounds the smallest eigenvalue of the voxel-space form (less 1e-3 for rounding), so
@@ -360,7 +361,9 @@ constexpr long long kBadFlag = 1LL << 62;  // marks a Gaussian tile with an inva
 
 // Six blocks of 256 per SM (42 registers, a few values spilled to L1) measured faster than
 // four (52 registers, no spills): the kernel is latency-bound on its division and square-root
-// sequences, so the extra resident warps pay more than the spills cost.
+// sequences, so the extra resident warps pay more than the spills cost. Where the voxel size is a
+// power of two (unit spacing above all) nine of its seventeen divisions are exact products: 23.4 -> 22.2
+// us at 500,000 Gaussians.
 // The block also stores its column of the first radix pass's digit counts (hist0[d * stride0 +
 // block]) and its number of pairs (blk[block]), kBadFlag added where a Gaussian was invalid.
 template <int kTile>
@@ -369,6 +372,7 @@ __global__ void __launch_bounds__(kTile, 6 * 256 / kTile) k_preprocess(
     int t_act, float* __restrict__ rec, int32_t* __restrict__ brange, int nd, int32_t* __restrict__ hist0,
     int64_t stride0, long long* __restrict__ blk) {
     pdl_enter();
+    static_assert((kTile & (kTile - 1)) == 0, "the digits (a power of two) divide evenly among the threads");
     __shared__ int hcnt[kMaxDigits], hdif[kMaxDigits + 1], sscan[32];
     __shared__ int hall, flags;  // flags: 1 an invalid Gaussian, 2 a box of more than kBoxSerial bricks
     __shared__ unsigned long long btot;
@@ -923,6 +927,8 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         G.h[k] = grid->h[k];
         G.o[k] = grid->origin[k];
         G.ih[k] = 1.0f / grid->h[k];
+        int e;
+        G.pow2[k] = frexpf(grid->h[k], &e) == 0.5f && e > -100 && e < 100;
     }
     G.b[0] = b.bx; G.b[1] = b.by; G.b[2] = b.bz;
     G.nb[0] = b.nbx; G.nb[1] = b.nby; G.nb[2] = b.nbz;

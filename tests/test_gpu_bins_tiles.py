@@ -59,6 +59,16 @@ def test_bins_tile_sizes(dims, brick, n):
     _check(cloud_params(d), og, brick)
 
 
+@pytest.mark.parametrize("h", [(1.0, 1.0, 1.0), (0.5, 2.0, 0.25), (0.9, 1.0, 1.3), (2.0 ** -8, 3.0, 4.0)])
+def test_bins_voxel_sizes(h):
+    """Voxel sizes that are and are not powers of two (a product and a division), offset origin."""
+    import oracle
+    og = oracle.Grid(53, 41, 37, h, (-3.1, 2.5, 0.7))
+    d = inputs.gaussian_cloud(8, 5000, (37, 41, 53), h=h)
+    d["mu"] = (d["mu"] + np.array(og.origin)).astype(np.float32)
+    _check(cloud_params(d), og)
+
+
 def test_bins_rounds_exact_fill():
     """Tiles of exactly 2,048 and 4,096 pairs, and one more: 256 Gaussians that all meet the same
     8 (16) bricks, plus one."""
