@@ -12,7 +12,7 @@
 //                   shared memory and scatters them by digit: the Gaussian-major pair list never
 //                   goes to memory.
 //   later passes    the same scan and scatter over tiles of 2,048 pairs, whose digit counts the
-//                   scatter before added up. Stability keeps ascending Gaussian ids inside each
+//                   scatter before added up or, for large clouds, k_tile_count counts. Stability keeps ascending Gaussian ids inside each
 //                   brick, so the lists are deterministic. The last pass stores pair_brick (key),
 //                   pair_gmj (Gaussian-major position) and pair_gid directly.
 //   k_brick_off     brick_off from the boundaries of the sorted keys.
@@ -457,8 +457,9 @@ struct RowScan {
     int64_t stride;
     int64_t cols;        // columns in use: fixed (first pass), or from npairs where < 0
     int32_t* rowtot;     // row totals
-    int32_t* zero;       // the next pass's counts, cleared here (nullptr: last pass)
-    int64_t zero_cols;
+    int32_t* zero;       // the next pass's counts, cleared here where the scatter adds them up (else nullptr)
+    int zero_rows;
+    int64_t zero_stride;
     long long* blk;      // first pass: pairs of each Gaussian tile, scanned by the last block,
     int32_t* ticket;     // which also clears the loss kernel's block counter
     int nd;
@@ -467,8 +468,8 @@ struct RowScan {
     int32_t* status;
 };
 
-// Block d scans row d (digit d's counts over the tiles) and clears row d of the next pass's
-// counts; the scatter adds up the row totals before its digits itself, so a pass's scan is one
+// Block d scans row d (digit d's counts over the tiles) and clears the next pass's counts where these are
+// added up by atomics; the scatter adds up the row totals before its digits itself, so a pass's scan is one
 // launch of 3.5 us at 1,954 tiles (a reduction and a down-sweep over all rows took two, 9 us).
 // The first pass's block nd scans the Gaussian tiles' pair counts (64-bit).
 __global__ void __launch_bounds__(kRowThreads) k_row_scan(RowScan A) {
@@ -519,8 +520,53 @@ __global__ void __launch_bounds__(kRowThreads) k_row_scan(RowScan A) {
     }
     if (tid == 0) A.rowtot[row] = static_cast<int>(carry);
     if (A.zero)
-        for (int64_t c = int64_t(tid) * 4; c < A.zero_cols; c += kRowThreads * 4)
-            *reinterpret_cast<int4*>(A.zero + row * A.zero_cols + c) = make_int4(0, 0, 0, 0);
+        for (int r = row; r < A.zero_rows; r += A.nd)
+            for (int64_t c = int64_t(tid) * 4; c < A.zero_stride; c += kRowThreads * 4)
+                *reinterpret_cast<int4*>(A.zero + r * A.zero_stride + c) = make_int4(0, 0, 0, 0);
+}
+
+// Digit counts of a later pass, a column per tile of kSortTile pairs of the pass before: a block counts
+// kCountTiles tiles in shared memory and writes their columns in 16-byte pieces. Bound by the keys' read.
+constexpr int kCountTiles = 4;
+
+__global__ void __launch_bounds__(kSortThreads) k_tile_count(const int32_t* __restrict__ keys,
+                                                             const int64_t* __restrict__ npairs, int64_t capacity,
+                                                             int shift, int nd, int32_t* __restrict__ hist,
+                                                             int64_t stride) {
+    pdl_enter();
+    __shared__ int cnt[kCountTiles][kMaxDigits];
+    const int64_t P = valid_pairs(npairs, capacity);
+    const int64_t tile0 = int64_t(blockIdx.x) * kCountTiles;
+    if (tile0 * kSortTile >= P) return;
+    for (int d = threadIdx.x; d < nd; d += kSortThreads)
+#pragma unroll
+        for (int t = 0; t < kCountTiles; ++t) cnt[t][d] = 0;
+    __syncthreads();
+    constexpr int kPieces = kSortTile / (4 * kSortThreads);  // of 16 bytes per thread and tile
+    int4 k[kCountTiles * kPieces];
+#pragma unroll
+    for (int e = 0; e < kCountTiles * kPieces; ++e) {
+        const int64_t i = tile0 * kSortTile + (e * kSortThreads + threadIdx.x) * 4;
+        k[e] = make_int4(-1, -1, -1, -1);
+        if (i + 3 < P) {
+            k[e] = *reinterpret_cast<const int4*>(keys + i);
+        } else {
+            if (i < P) k[e].x = keys[i];
+            if (i + 1 < P) k[e].y = keys[i + 1];
+            if (i + 2 < P) k[e].z = keys[i + 2];
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < kCountTiles * kPieces; ++e) {
+        int* c = cnt[e / kPieces];
+        if (k[e].x >= 0) atomicAdd(&c[(k[e].x >> shift) & (nd - 1)], 1);
+        if (k[e].y >= 0) atomicAdd(&c[(k[e].y >> shift) & (nd - 1)], 1);
+        if (k[e].z >= 0) atomicAdd(&c[(k[e].z >> shift) & (nd - 1)], 1);
+        if (k[e].w >= 0) atomicAdd(&c[(k[e].w >> shift) & (nd - 1)], 1);
+    }
+    __syncthreads();
+    for (int d = threadIdx.x; d < nd; d += kSortThreads)
+        *reinterpret_cast<int4*>(hist + d * stride + tile0) = make_int4(cnt[0][d], cnt[1][d], cnt[2][d], cnt[3][d]);
 }
 
 struct Scatter {
@@ -533,8 +579,9 @@ struct Scatter {
     const int32_t* hist;       // this pass's scanned counts
     int64_t stride;
     const int32_t* rowtot;
-    int32_t* hist_next;        // the next pass's counts (not the last pass)
+    int32_t* hist_next;        // the next pass's counts where this one adds them up (else nullptr)
     int64_t stride_next;
+    int bits_next;
     int shift, bits;
     const int64_t* npairs;
     int64_t capacity;
@@ -556,17 +603,17 @@ struct Scatter {
 // kFirst: the tile is emitted by the block itself from its kTile Gaussians' boxes (in rounds
 // of kSortTile pairs; the digits' output positions advance from round to round), else it is one
 // tile of the previous pass's output. kLast: the pass stores the bins' per-pair arrays; every
-// other pass adds each key to the next pass's digit counts at its output position's tile (one
-// atomic per group of equal (tile, digit) in a warp).
+// other pass of a small cloud adds each key to the next pass's digit counts at its output
+// position's tile (one atomic per group of equal (tile, digit) in a warp).
 // Bound by latency (barriers, the gathered loads) at 40-65 % issue-active, far from bandwidth: the
 // pair list is cache-resident at the fitting size. Whole binning, L2 flushed, at 3.26M pairs
 // (256 x 256 x 128 grid, 8^3 bricks): 115 us with the pair list emitted to memory, two scan launches
-// per list and the owners gathered in the last pass; 90 us now (preprocess 23, first pass 32, last
-// pass 20, scans 7, offsets 6). 104M pairs (512 x 512 x 256, two 9-bit passes where 8-bit digits took
-// three): 5.86 -> 3.01 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed
+// per list and the owners gathered in the last pass; 88 us now (preprocess 22, first pass 28, last
+// pass 20, count 4, scans 7, offsets 6). 104M pairs (512 x 512 x 256, digits of 9 and 8 bits where 8-bit
+// digits took three passes): 5.86 -> 2.40 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed
 // by a second match per key and the values held in registers (80 registers) 108 us; the
-// values loaded when the tile is placed 90 us and 3.17 ms; copied to shared memory
-// asynchronously during the ranking (here) 90 us and 3.01 ms; 5 (6) blocks per SM with spills 95
+// values loaded when the tile is placed 0.17 ms longer at 104M than copied to shared memory
+// asynchronously during the ranking (here); 5 (6) blocks per SM with spills 95
 // (97) us.
 template <bool kFirst, bool kLast, int kTile>
 __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
@@ -740,10 +787,12 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
                 A.out_gid[pos] = v.y;
             } else {
                 A.vals_out[pos] = v;
-                const int tile = pos / kSortTile, dn = (key >> (A.shift + A.bits)) & (nd - 1);
-                const unsigned peers = __match_any_sync(__activemask(), (tile << A.bits) | dn);
-                if (lane == __ffs(peers) - 1)
-                    atomicAdd(&A.hist_next[dn * A.stride_next + tile], __popc(peers));
+                if (A.hist_next) {
+                    const int tile = pos / kSortTile, dn = (key >> (A.shift + A.bits)) & ((1 << A.bits_next) - 1);
+                    const unsigned peers = __match_any_sync(__activemask(), (tile << kMaxRadixBits) | dn);
+                    if (lane == __ffs(peers) - 1)
+                        atomicAdd(&A.hist_next[dn * A.stride_next + tile], __popc(peers));
+                }
             }
         }
     }
@@ -943,33 +992,44 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
             return GS_ERR_CUDA;
         return GS_OK;
     }
-    const int nd = 1 << ws.radix_bits, passes = ws.radix_passes;
+    const int passes = ws.radix_passes;
+    const int bits0 = pass_bits(ws.key_bits, passes, 0), nd0 = 1 << bits0;
     const int gt = gauss_tile(N);
     const unsigned gb = static_cast<unsigned>((N + gt - 1) / gt);
     launch_k(gt == 64 ? k_preprocess<64> : k_preprocess<256>, dim3(gb), dim3(gt), 0, st, params, N, G, cfg->trunc_sigma,
-        cfg->signal_mode, cfg->a_act, cfg->t_act, bins->rec, bins->brange, nd, ws.hist0, ws.stride0,
+        cfg->signal_mode, cfg->a_act, cfg->t_act, bins->rec, bins->brange, nd0, ws.hist0, ws.stride0,
         ws.blk_base);
     gs_status s = last_launch_status();
     if (s != GS_OK) return s;
-    const size_t smem = sizeof(int) * (kSortThreads / 32 + 1) * nd;
     const unsigned tiles = static_cast<unsigned>((cap + kSortTile - 1) / kSortTile);
-    for (int pass = 0; pass < passes; ++pass) {
+    for (int pass = 0, shift = 0; pass < passes; ++pass) {
+        const int bits = pass_bits(ws.key_bits, passes, pass), nd = 1 << bits;
+        const size_t smem = sizeof(int) * (kSortThreads / 32 + 1) * nd;
         const bool first = pass == 0, last = pass == passes - 1;
         const int cur = (pass + 1) & 1;  // later passes alternate: pass 1 reads buffers 0, pass 2 buffers 1
         const int nxt = pass & 1;
+        const int bits_next = last ? 0 : pass_bits(ws.key_bits, passes, pass + 1);
+        const bool count_next = !last && N < kCountCloud;
         RowScan R = {};
         R.hist = first ? ws.hist0 : ws.hist[cur];
         R.stride = first ? ws.stride0 : ws.stride1;
         R.cols = first ? int64_t(gb) : -1;
         R.rowtot = ws.rowtot;
-        R.zero = last ? nullptr : ws.hist[nxt];
-        R.zero_cols = ws.stride1;
+        R.zero = count_next ? ws.hist[nxt] : nullptr;
+        R.zero_rows = 1 << bits_next;
+        R.zero_stride = ws.stride1;
         R.blk = ws.blk_base;
         R.ticket = ws.ticket;
         R.nd = nd;
         R.npairs = bins->d_npairs;
         R.capacity = cap;
         R.status = bins->d_status;
+        if (!first && tiles > 0 && N >= kCountCloud) {
+            launch_k(k_tile_count, dim3((tiles + kCountTiles - 1) / kCountTiles), dim3(kSortThreads), 0, st, ws.keys[cur],
+                     bins->d_npairs, cap, shift, nd, ws.hist[cur], ws.stride1);
+            s = last_launch_status();
+            if (s != GS_OK) return s;
+        }
         launch_k(k_row_scan, dim3(nd + (first ? 1 : 0)), dim3(kRowThreads), 0, st, R);
         s = last_launch_status();
         if (s != GS_OK) return s;
@@ -985,8 +1045,9 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         A.rowtot = ws.rowtot;
         A.hist_next = R.zero;
         A.stride_next = ws.stride1;
-        A.shift = pass * ws.radix_bits;
-        A.bits = ws.radix_bits;
+        A.bits_next = bits_next;
+        A.shift = shift;
+        A.bits = bits;
         A.npairs = bins->d_npairs;
         A.capacity = cap;
         A.brange = bins->brange;
@@ -1005,6 +1066,7 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
             s = last_launch_status();
             if (s != GS_OK) return s;
         }
+        shift += bits;
     }
     if (passes == 1) return GS_OK;  // (brick_off is written by the pass)
     if (cap == 0)

@@ -26,11 +26,11 @@ def _check(params, og, brick=(8, 8, 8)):
 
 
 # grid (x, y, z) and brick: 1 brick; 2 x 2 x 2; 315 (one 9-bit pass); 512 (one full pass);
-# 513 x 1 x 1 (two passes, rows longer than their 32 digits); 4,096 and 131,072 (two passes of 6 and 9 bits);
-# 266,240 (three passes)
+# 513 x 1 x 1 (two passes, rows longer than their 32 digits); 4,096, 131,072 and 262,144 (two passes of 6, of
+# 9 and 8, of 9 bits); 266,240 (three passes, of 6, 6 and 7 bits)
 GRIDS = [((8, 8, 8), (8, 8, 8)), ((13, 11, 10), (8, 8, 8)), ((50, 33, 71), (8, 8, 8)),
          ((64, 64, 64), (8, 8, 8)), ((4104, 8, 8), (8, 8, 8)), ((64, 64, 64), (4, 4, 4)),
-         ((512, 512, 256), (8, 8, 8)), ((512, 512, 64), (4, 4, 4))]
+         ((512, 512, 256), (8, 8, 8)), ((512, 512, 64), (4, 4, 4)), ((520, 512, 64), (4, 4, 4))]
 
 
 @pytest.mark.parametrize("n", [1, 255, 256, 257, 1500])
@@ -56,6 +56,19 @@ def test_bins_tile_sizes(dims, brick, n):
     og = oracle.Grid(*dims)
     d = inputs.gaussian_cloud(n, n, dims[::-1], scale_range=(0.5, 1.2))
     d["log_s"][::4001] += 2.0
+    _check(cloud_params(d), og, brick)
+
+
+@pytest.mark.parametrize("n", [399_999, 400_000, 401_234])
+@pytest.mark.parametrize("dims,brick", [((64, 64, 60), (4, 4, 4)), ((160, 128, 88), (8, 8, 8)),
+                                        ((512, 512, 256), (8, 8, 8)), ((520, 512, 64), (4, 4, 4))])
+def test_bins_count_kernel(dims, brick, n):
+    """The largest cloud whose later digits are counted by the scatter before and the smallest whose
+    are counted by a kernel: digits of 6 and 6, 6 and 6 of 3,520, 9 and 8, and 6, 6 and 7 bits."""
+    import oracle
+    og = oracle.Grid(*dims)
+    d = inputs.gaussian_cloud(n, n, dims[::-1], scale_range=(0.3, 0.7))
+    d["log_s"][::40_001] += 2.0
     _check(cloud_params(d), og, brick)
 
 
