@@ -5,8 +5,9 @@
  *
  * Conventions shared by every entry point
  *   - Pointers marked "device" are CUDA device memory owned by the caller; "host" pointers
- *     are ordinary host memory. The library allocates no memory: scratch comes from a
- *     caller-provided workspace whose size gs_workspace_bytes() reports.
+ *     are ordinary host memory. The library allocates no device memory: scratch comes from a
+ *     caller-provided workspace whose size gs_workspace_bytes() reports. (What an entry point keeps
+ *     otherwise, a stream, an event or a page-locked word, its comment says.)
  *   - Every compute call is asynchronous on `stream` (a cudaStream_t; NULL = the legacy
  *     default stream) unless its comment says "synchronous". Argument errors are detected on
  *     the host before any launch and returned at once; CUDA launch errors map to
