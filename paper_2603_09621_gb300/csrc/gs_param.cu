@@ -362,7 +362,7 @@ static AdamLr make_adam_lr(const gs_adam* hp) {
     return a;
 }
 
-static bool adam_ok(const gs_adam* hp) {
+bool adam_ok(const gs_adam* hp) {
     return hp->beta1 >= 0.0 && hp->beta1 < 1.0 && hp->beta2 >= 0.0 && hp->beta2 < 1.0 &&
            hp->eps > 0.0;
 }

@@ -338,6 +338,7 @@ gs_status downsample_bwd_impl(const float* dlr, int nz, int ny, int nx, int s, f
 gs_status bind_workspace(void* base, size_t bytes, int64_t n_gauss, int64_t capacity,
                          const gs_grid* grid, const gs_config* cfg, Workspace* ws);
 bool bins_match(const gs_bins* b, const gs_grid* grid, const gs_config* cfg);
+bool adam_ok(const gs_adam* hp);
 gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_config* cfg,
                           gs_bins* bins, const Workspace& ws, cudaStream_t st);
 gs_status render_fwd_impl(const gs_bins* bins, const gs_grid* grid, const gs_config* cfg, float* I,
@@ -483,6 +484,7 @@ extern "C" gs_status gs_fit_step(gs_fit_state* st, gs_stream stream) {
     FitRun run;
     gs_status s = fit_prepare(st, stream, &run);
     if (s != GS_OK) return s;
+    if (!adam_ok(&st->adam)) return GS_ERR_INVALID_ARG;  // before the loss kernel counts the step
     s = fit_front(run, 0, st->d_step);
     if (s != GS_OK) return s;
     s = launch_chain_adam(st->params, st->grad, st->m, st->v, run.w.part, run.w.gacc, &st->bins,
@@ -533,6 +535,7 @@ extern "C" gs_status gs_fit_step_host(gs_fit_state* st, const float* h_params,
     FitRun run;
     gs_status s = fit_prepare(st, stream, &run);
     if (s != GS_OK) return s;
+    if (!adam_ok(&st->adam)) return GS_ERR_INVALID_ARG;
     // The parameters go first, alone on the link, since binning waits for them; the LR target
     // follows on a side stream while the step bins and renders, and the step waits for it
     // only before the LR model. The side stream starts after everything issued on `stream`

@@ -100,3 +100,19 @@ def test_resize_forms_64bit(src, dst):
     u = 2.0 ** -24
     assert (gs.gs_resample_fwd(x, dst).double() - fwd).abs().max() <= 12 * u * x.abs().max()
     assert (gs.gs_resample_bwd(d, src).double() - bwd).abs().max() <= (12 + terms) * terms * u * d.abs().max()
+
+
+def test_refused_step_is_not_counted():
+    """Adam parameters out of range: the step is refused before anything is launched."""
+    import torch
+    from paper_2603_09621_gb300 import gs
+    grid = gs.Grid(16, 12, 8)
+    p = torch.zeros(50, 12, device="cuda")
+    p[:, :3], p[:, 6] = 5.0, 1.0
+    f = gs.FitState(p.clone(), torch.rand(4, 12, 16, device="cuda"), grid, 2, gs.Config(),
+                    adam=gs.Adam(beta1=1.0))
+    for step in (f.step, lambda: f.step_host(torch.ones(50, 12))):
+        with pytest.raises(Exception, match="INVALID_ARG"):
+            step()
+        torch.cuda.synchronize()
+        assert int(f.d_step) == 0 and torch.equal(f.params, p)
