@@ -228,15 +228,17 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ params, const 
 // raw parameters (written to grad), and (kAdam) apply Adam to params, m, v; d_step already counts
 // this step. A step whose binning overflowed rendered nothing: it leaves parameters and moments as
 // they are and zeroes grad (the caller grows the bins and repeats the step).
-// Blocks of 64 threads, a Gaussian's partials loaded three at a time (same order of additions). Bound by
-// HBM and the latency of the scattered partials: 500,000 Gaussians, 3.26M pairs (about 320 MB) 66 us in
-// blocks of 256, 63 us here (unrolled by 1, 2, 4, 8: 69, 66, 64, 64 us), 833,000 97 -> 92 us. kSmall:
-// clouds of at most kSmallCloud Gaussians, whose time is the latency of the longest list, take the registers
-// for four loads: 2,000 Gaussians 8.0 -> 6.6 us, 6,000 with 19 pairs each 17 -> 13 us.
+// Blocks of 64 threads, a Gaussian's partials loaded three or (kFour) four at a time, always added in the same
+// order. Bound by HBM and the latency of the scattered partials: 500,000 Gaussians, 3.26M pairs (about 320 MB)
+// 66 us in blocks of 256, 61.6 us here; 833,000 97 -> 89 us. With Adam four loads without spills (72 registers, 14
+// blocks per SM) beat three with (64, 16 blocks): 61.6 against 63 us, 89 against 91.5, 100,000 Gaussians 15.0
+// against 16.2; five or six loads 66 and 70 us. The gradient alone is shorter with three (188,000 Gaussians, 1.5M
+// pairs 21.9 against 24.3 us) but for clouds of at most kSmallCloud Gaussians, whose time is the latency of the
+// longest list: 6,000 with 19 pairs each 17 -> 13 us.
 constexpr int kChainThreads = 64;
 
-template <bool kDet, bool kAdam, bool kSmall>
-__global__ void __launch_bounds__(kChainThreads, kSmall ? 8 : 16) k_chain_adam(
+template <bool kDet, bool kAdam, bool kFour>
+__global__ void __launch_bounds__(kChainThreads, kFour ? 12 : 16) k_chain_adam(
     float* __restrict__ params, float* __restrict__ grad, float* __restrict__ m,
     float* __restrict__ v, const float* __restrict__ part, const float* __restrict__ gacc,
     const int32_t* __restrict__ gm_off, const int64_t* __restrict__ npairs, int64_t capacity,
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__(kChainThreads, kSmall ? 8 : 16) k_chain_adam(
 #pragma unroll
         for (int k = 0; k < 12; ++k) gv[k] = 0.f;
         const int a = gm_off[g], e = gm_off[g + 1];
-#pragma unroll (kSmall ? 4 : 3)
+#pragma unroll (kFour ? 4 : 3)
         for (int j = a; j < e; ++j) {
             float t[12];
             load12(part + int64_t(j) * GRAD_FLOATS, t);
@@ -378,14 +380,13 @@ gs_status launch_chain_adam(float* params, float* grad, float* m, float* v, cons
     C.a_act = cfg->a_act;
     C.t_act = cfg->t_act;
     const AdamLr a = make_adam_lr(hp);
-    const bool small = n <= kSmallCloud;
     const unsigned gb = static_cast<unsigned>((n + kChainThreads - 1) / kChainThreads);
     if (cfg->deterministic)
-        launch_k(small ? k_chain_adam<true, true, true> : k_chain_adam<true, true, false>, dim3(gb),
+        launch_k(k_chain_adam<true, true, true>, dim3(gb),
             dim3(kChainThreads), 0, st, params, grad, m, v, part,
             gacc, bins->gm_off, bins->d_npairs, bins->capacity, n, C, a, d_step);
     else
-        launch_k(small ? k_chain_adam<false, true, true> : k_chain_adam<false, true, false>, dim3(gb),
+        launch_k(k_chain_adam<false, true, true>, dim3(gb),
             dim3(kChainThreads), 0, st, params, grad, m, v, part,
             gacc, bins->gm_off, bins->d_npairs, bins->capacity, n, C, a, d_step);
     return last_launch_status();
@@ -411,7 +412,7 @@ gs_status launch_chain_grad(const float* params, float* grad, const float* part,
             static_cast<float*>(nullptr), static_cast<float*>(nullptr), part, gacc, bins->gm_off,
             bins->d_npairs, bins->capacity, n, C, a, static_cast<const int32_t*>(nullptr));
     else
-        launch_k(small ? k_chain_adam<false, false, true> : k_chain_adam<false, false, false>, dim3(gb),
+        launch_k(k_chain_adam<false, false, false>, dim3(gb),
             dim3(kChainThreads), 0, st, p, grad,
             static_cast<float*>(nullptr), static_cast<float*>(nullptr), part, gacc, bins->gm_off,
             bins->d_npairs, bins->capacity, n, C, a, static_cast<const int32_t*>(nullptr));
