@@ -21,6 +21,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "gs_common.cuh"
 
 namespace gs {
@@ -594,14 +596,14 @@ struct Scatter {
     int32_t* brick_off;        // (a first pass that is the last)
 };
 
-// Stable scatter of one tile of up to kSortTile keys per round. Warp w owns a contiguous part of
+// Stable scatter of one tile of up to kRound keys per round. Warp w owns a contiguous part of
 // the tile and visits it in rounds of 32 consecutive keys, kept in registers with their ranks
 // among the warp's earlier equal digits (warp match masks). A block-wide prefix over the digits
 // then gives each digit's run inside the tile and each warp's start in it; the tile is placed in
 // shared memory sorted by digit, ties in tile order, and written out in that order, so consecutive
 // threads store consecutive addresses of a run.
 // kFirst: the tile is emitted by the block itself from its kTile Gaussians' boxes (in rounds
-// of kSortTile pairs; the digits' output positions advance from round to round), else it is one
+// of kRound pairs; the digits' output positions advance from round to round), else it is one
 // tile of the previous pass's output. kLast: the pass stores the bins' per-pair arrays; every
 // other pass of a small cloud adds each key to the next pass's digit counts at its output
 // position's tile (one atomic per group of equal (tile, digit) in a warp).
@@ -610,7 +612,7 @@ struct Scatter {
 // (256 x 256 x 128 grid, 8^3 bricks): 115 us with the pair list emitted to memory, two scan launches
 // per list and the owners gathered in the last pass; 88 us now (preprocess 22, first pass 28, last
 // pass 20, count 4, scans 7, offsets 6). 104M pairs (512 x 512 x 256, digits of 9 and 8 bits where 8-bit
-// digits took three passes): 5.86 -> 2.40 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed
+// digits took three passes): 5.86 -> 2.36 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed
 // by a second match per key and the values held in registers (80 registers) 108 us; the
 // values loaded when the tile is placed 0.17 ms longer at 104M than copied to shared memory
 // asynchronously during the ranking (here); 5 (6) blocks per SM with spills 95
@@ -620,13 +622,15 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
     pdl_enter();
     constexpr int kWarps = kSortThreads / 32;
     static_assert(kSortThreads >= kTile, "one thread per Gaussian of a tile");
+    constexpr int kMaxRound = kSortThreads * (kFirst ? kFirstItems : kSortItems);
+    static_assert(kMaxRound < 8192, "runs of a round are packed in 13 bits");
     extern __shared__ int smem[];
     const int nd = 1 << A.bits, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int* wcnt = smem;                 // [kWarps][nd]
     int* goff = wcnt + kWarps * nd;   // output position of tile slot j of digit d: goff[d] + j
-    __shared__ int skey[kSortTile];
-    __shared__ unsigned short sidx[kSortTile];          // sorted: tile index of each key
-    __shared__ unsigned char sowner[kFirst ? kSortTile : 1];  // tile order: Gaussian of the block
+    __shared__ int skey[kMaxRound];
+    __shared__ unsigned short sidx[kMaxRound];             // sorted: tile index of each key
+    __shared__ unsigned char sowner[kFirst ? kMaxRound : 1];  // tile order: Gaussian of the block
     __shared__ int2 sval[kFirst ? 1 : kSortTile];       // tile order: the keys' values
     __shared__ long long sscan[32];
 
@@ -679,123 +683,131 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
         if (base >= P) return;  // past the last pair: nothing to place
         total = static_cast<int>(min(int64_t(kSortTile), P - base));
     }
-    for (int c0 = 0; c0 < total; c0 += kSortTile) {
-        const int n = min(kSortTile, total - c0);
-        if (kFirst) {
-            if (c0 > 0) __syncthreads();  // the previous round has been written out
-            for_box(box, max(0, c0 - loc), min(box.cnt, c0 + n - loc), loc - c0, A.nbx, A.nby,
-                    [&](int src, int o, int key) {
-                        skey[o] = key;
-                        sowner[o] = static_cast<unsigned char>(warp * 32 + src);
-                    });
-        }
-        for (int d = tid; d < kWarps * nd; d += kSortThreads) wcnt[d] = 0;
-        __syncthreads();
-        // each warp's part: the same number of 32-key rounds
-        const int rounds = (n + kSortThreads - 1) / kSortThreads;
-        const int sub0 = warp * rounds * 32;
-        int kr[kSortItems];
-        unsigned short rank[kSortItems];
-#pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            const int idx = sub0 + r * 32 + lane;
-            kr[r] = 0;
-            if (idx < n && r < rounds) {
-                kr[r] = kFirst ? skey[idx] : A.keys_in[base + idx];
-                if (!kFirst)  // read again only when the sorted tile is written out
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                                     static_cast<unsigned>(__cvta_generic_to_shared(&sval[idx]))),
-                                 "l"(A.vals_in + base + idx)
-                                 : "memory");
+    // rounds of kRound pairs, kItems per thread
+    auto rounds_of = [&](auto items) {
+        constexpr int kItems = decltype(items)::value, kRound = kSortThreads * kItems;
+        for (int c0 = 0; c0 < total; c0 += kRound) {
+            const int n = min(kRound, total - c0);
+            if (kFirst) {
+                if (c0 > 0) __syncthreads();  // the previous round has been written out
+                for_box(box, max(0, c0 - loc), min(box.cnt, c0 + n - loc), loc - c0, A.nbx, A.nby,
+                        [&](int src, int o, int key) {
+                            skey[o] = key;
+                            sowner[o] = static_cast<unsigned char>(warp * 32 + src);
+                        });
             }
-        }
+            for (int d = tid; d < kWarps * nd; d += kSortThreads) wcnt[d] = 0;
+            __syncthreads();
+            // each warp's part: the same number of 32-key rounds
+            const int rounds = (n + kSortThreads - 1) / kSortThreads;
+            const int sub0 = warp * rounds * 32;
+            int kr[kItems];
+            unsigned short rank[kItems];
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            if (r < rounds) {
-                const bool valid = sub0 + r * 32 + lane < n;
-                const int d = (kr[r] >> A.shift) & (nd - 1);
-                const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : nd + lane);
-                int* w = &wcnt[warp * nd + d];
-                const int before = valid ? *w : 0;
-                __syncwarp();
-                if (valid && lane == __ffs(peers) - 1) *w = before + __popc(peers);
-                __syncwarp();
-                rank[r] = static_cast<unsigned short>(before + __popc(peers & ((1u << lane) - 1u)));
-            }
-        }
-        __syncthreads();
-        // digit runs: thread t owns digits [t di, (t + 1) di)
-        const int di = nd > kSortThreads ? nd / kSortThreads : 1;
-        long long mine = 0;
-        int runs[kMaxDigits / kSortThreads], rows[kMaxDigits / kSortThreads];
-#pragma unroll
-        for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
-            runs[e] = rows[e] = 0;
-            const int d = tid * di + e;
-            if (e < di && d < nd) {
-                int run = 0;
-#pragma unroll
-                for (int w = 0; w < kWarps; ++w) {
-                    const int c = wcnt[w * nd + d];
-                    wcnt[w * nd + d] = run;
-                    run += c;
-                }
-                runs[e] = run;
-                if (c0 == 0) rows[e] = A.rowtot[d];
-            }
-            mine += (static_cast<long long>(rows[e]) << 13) | runs[e];  // (sums of runs: <= 2,048)
-        }
-        long long all;
-        const long long pre = block_exclusive_scan(mine, sscan, &all);
-        int start = static_cast<int>(pre & 8191);
-        int64_t row0 = pre >> 13;
-#pragma unroll
-        for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
-            const int d = tid * di + e;
-            if (e < di && d < nd) {
-                if (c0 == 0) gpos[e] = static_cast<int>(row0) + A.hist[d * A.stride + blockIdx.x];
-                goff[d] = gpos[e] - start;
-                gpos[e] += runs[e];
-#pragma unroll
-                for (int w = 0; w < kWarps; ++w) wcnt[w * nd + d] += start;
-                row0 += rows[e];
-                start += runs[e];
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            const int idx = sub0 + r * 32 + lane;
-            if (r < rounds && idx < n) {
-                const int lp = wcnt[warp * nd + ((kr[r] >> A.shift) & (nd - 1))] + rank[r];
-                skey[lp] = kr[r];
-                sidx[lp] = static_cast<unsigned short>(idx);
-            }
-        }
-        if (!kFirst) asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();
-        for (int j = tid; j < n; j += kSortThreads) {
-            const int key = skey[j];
-            const int idx = sidx[j];
-            const int2 v = kFirst ? make_int2(static_cast<int>(base) + c0 + idx,
-                                              static_cast<int>(blockIdx.x) * kTile + sowner[idx])
-                                  : sval[idx];
-            const int pos = goff[(key >> A.shift) & (nd - 1)] + j;
-            A.keys_out[pos] = key;
-            if (kLast) {
-                A.out_gmj[pos] = v.x;
-                A.out_gid[pos] = v.y;
-            } else {
-                A.vals_out[pos] = v;
-                if (A.hist_next) {
-                    const int tile = pos / kSortTile, dn = (key >> (A.shift + A.bits)) & ((1 << A.bits_next) - 1);
-                    const unsigned peers = __match_any_sync(__activemask(), (tile << kMaxRadixBits) | dn);
-                    if (lane == __ffs(peers) - 1)
-                        atomicAdd(&A.hist_next[dn * A.stride_next + tile], __popc(peers));
+            for (int r = 0; r < kItems; ++r) {
+                const int idx = sub0 + r * 32 + lane;
+                kr[r] = 0;
+                if (idx < n && r < rounds) {
+                    kr[r] = kFirst ? skey[idx] : A.keys_in[base + idx];
+                    if (!kFirst)  // read again only when the sorted tile is written out
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                                         static_cast<unsigned>(__cvta_generic_to_shared(&sval[idx]))),
+                                     "l"(A.vals_in + base + idx)
+                                     : "memory");
                 }
             }
+#pragma unroll
+            for (int r = 0; r < kItems; ++r) {
+                if (r < rounds) {
+                    const bool valid = sub0 + r * 32 + lane < n;
+                    const int d = (kr[r] >> A.shift) & (nd - 1);
+                    const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : nd + lane);
+                    int* w = &wcnt[warp * nd + d];
+                    const int before = valid ? *w : 0;
+                    __syncwarp();
+                    if (valid && lane == __ffs(peers) - 1) *w = before + __popc(peers);
+                    __syncwarp();
+                    rank[r] = static_cast<unsigned short>(before + __popc(peers & ((1u << lane) - 1u)));
+                }
+            }
+            __syncthreads();
+            // digit runs: thread t owns digits [t di, (t + 1) di)
+            const int di = nd > kSortThreads ? nd / kSortThreads : 1;
+            long long mine = 0;
+            int runs[kMaxDigits / kSortThreads], rows[kMaxDigits / kSortThreads];
+#pragma unroll
+            for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
+                runs[e] = rows[e] = 0;
+                const int d = tid * di + e;
+                if (e < di && d < nd) {
+                    int run = 0;
+#pragma unroll
+                    for (int w = 0; w < kWarps; ++w) {
+                        const int c = wcnt[w * nd + d];
+                        wcnt[w * nd + d] = run;
+                        run += c;
+                    }
+                    runs[e] = run;
+                    if (c0 == 0) rows[e] = A.rowtot[d];
+                }
+                mine += (static_cast<long long>(rows[e]) << 13) | runs[e];  // (sums of runs: <= kRound)
+            }
+            long long all;
+            const long long pre = block_exclusive_scan(mine, sscan, &all);
+            int start = static_cast<int>(pre & 8191);
+            int64_t row0 = pre >> 13;
+#pragma unroll
+            for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
+                const int d = tid * di + e;
+                if (e < di && d < nd) {
+                    if (c0 == 0) gpos[e] = static_cast<int>(row0) + A.hist[d * A.stride + blockIdx.x];
+                    goff[d] = gpos[e] - start;
+                    gpos[e] += runs[e];
+#pragma unroll
+                    for (int w = 0; w < kWarps; ++w) wcnt[w * nd + d] += start;
+                    row0 += rows[e];
+                    start += runs[e];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < kItems; ++r) {
+                const int idx = sub0 + r * 32 + lane;
+                if (r < rounds && idx < n) {
+                    const int lp = wcnt[warp * nd + ((kr[r] >> A.shift) & (nd - 1))] + rank[r];
+                    skey[lp] = kr[r];
+                    sidx[lp] = static_cast<unsigned short>(idx);
+                }
+            }
+            if (!kFirst) asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();
+            for (int j = tid; j < n; j += kSortThreads) {
+                const int key = skey[j];
+                const int idx = sidx[j];
+                const int2 v = kFirst ? make_int2(static_cast<int>(base) + c0 + idx,
+                                                  static_cast<int>(blockIdx.x) * kTile + sowner[idx])
+                                      : sval[idx];
+                const int pos = goff[(key >> A.shift) & (nd - 1)] + j;
+                A.keys_out[pos] = key;
+                if (kLast) {
+                    A.out_gmj[pos] = v.x;
+                    A.out_gid[pos] = v.y;
+                } else {
+                    A.vals_out[pos] = v;
+                    if (A.hist_next) {
+                        const int tile = pos / kSortTile, dn = (key >> (A.shift + A.bits)) & ((1 << A.bits_next) - 1);
+                        const unsigned peers = __match_any_sync(__activemask(), (tile << kMaxRadixBits) | dn);
+                        if (lane == __ffs(peers) - 1)
+                            atomicAdd(&A.hist_next[dn * A.stride_next + tile], __popc(peers));
+                    }
+                }
+            }
         }
-    }
+    };
+    if (kFirst && total > kSortTile)
+        rounds_of(std::integral_constant<int, kFirstItems>());
+    else
+        rounds_of(std::integral_constant<int, kSortItems>());
 }
 
 // brick_off from the boundaries of the sorted keys (brick_off[b] = first pair of brick b, or

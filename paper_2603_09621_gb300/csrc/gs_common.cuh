@@ -72,6 +72,13 @@ enum BrangeField : int { B_LOX = 0, B_LOY, B_LOZ, B_HIX, B_HIY, B_HIZ, B_CNT, B_
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
+// First-pass tiles of more than kSortTile pairs take rounds of 2,304: a round costs 7 us or more whether full or
+// nearly empty, and tiles of 256 Gaussians with 8.2-8.5 pairs each needed a second one (833,333 Gaussians, 6.83M
+// pairs, whole binning 182 -> 171 us; 100,000 with 7.1 pairs 36.7 -> 35.5; 4M with 26 2.40 -> 2.36 ms). Used for all
+// tiles, 0.2 % of a step at 5.6-6.5 pairs, which fill one round either way. 10 and more items spill at 64
+// registers; with the keys read again from shared memory instead, 10 (12) take 171 (171) us and 2.34 (2.28) ms, but
+// 69.3 (69.4) us against 67.5 at 375,000 with 5.6 pairs and 89.9 (89.3) against 88.8 at 500,000.
+constexpr int kFirstItems = 9;
 constexpr int kMaxRadixBits = 9;
 constexpr int kMaxDigits = 1 << kMaxRadixBits;
 // Gaussians per block of the preprocess and emission kernels. A cloud that would fill no more than one

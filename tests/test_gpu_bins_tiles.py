@@ -1,5 +1,5 @@
 """Brick lists where the binning's tiles can go wrong, bit for bit against the oracle's
-specification: Gaussian tiles of 64 and 256, rounds of 2,048 pairs per tile, boxes of more than 64 bricks
+specification: Gaussian tiles of 64 and 256, rounds of 2,304 and 2,048 pairs per tile, boxes of more than 64 bricks
 (counted by rows and emitted by a warp), digit widths from one narrow pass to three passes."""
 import numpy as np
 import pytest
@@ -93,6 +93,21 @@ def test_bins_rounds_exact_fill():
         p[:, 3:6] = np.log(2.0) if z == 8.0 else np.log(np.array([2.0, 2.0, 4.0]))
         p[:, 6], p[:, 10:] = 1.0, 0.5
         _check(p, og)
+
+
+@pytest.mark.parametrize("nz,per", [(8, 9), (16, 18)])
+@pytest.mark.parametrize("n", [38_912, 38_913, 39_167])
+def test_bins_first_pass_rounds(nz, per, n):
+    """First-pass tiles of 256 Gaussians (clouds of more than 38,912) and of 64 that fill rounds of 2,304
+    pairs exactly, once and twice: every Gaussian meets the same 9 (18) bricks; the last tile is ragged."""
+    import oracle
+    p = np.zeros((n, 12), np.float32)
+    p[:, :3] = (12.0, 12.0, nz / 2)
+    p[:, 3:6] = np.log(np.array([2.0, 2.0, nz / 8.0]))
+    p[:, 6], p[:, 10:] = 1.0, 0.5
+    og = oracle.Grid(24, 24, nz)
+    assert oracle.brick_lists(p, og, oracle.Config())["pair_gid"].size == per * n
+    _check(p, og)
 
 
 def test_bins_overflow_with_wide_gaussians():
