@@ -499,6 +499,14 @@ def gs_render_cloud(params: torch.Tensor, grid: Grid, cfg: Config, bins: Bins, w
     return need.value
 
 
+def _foreign_stream(stream, dev):
+    """The stream a call was given, where it is not the current one (whose allocator pool the call's
+    tensors come from); else None."""
+    if stream is None or stream.cuda_stream == torch.cuda.current_stream(dev).cuda_stream:
+        return None
+    return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, dev)
+
+
 def render(params: torch.Tensor, grid: Grid, cfg: Config = Config(), capacity: int | None = None,
            stats: torch.Tensor | None = None, stream=None):
     """Bin and render a cloud. Grows the pair capacity (one host read) if it overflows.
@@ -507,18 +515,21 @@ def render(params: torch.Tensor, grid: Grid, cfg: Config = Config(), capacity: i
     # 16 pairs per Gaussian; small clouds, whose retry costs more than their memory (72 bytes per
     # pair), get up to 64
     cap = capacity if capacity is not None else max(1024, 16 * n, min(64 * n, 1 << 20))
+    side = _foreign_stream(stream, dev)
     I = torch.empty(grid.shape, dtype=torch.float32, device=dev)
     W = torch.empty(grid.shape, dtype=torch.float32, device=dev)
-    spent = None
     while True:
         bins = Bins(n, cap, grid, cfg, dev)
         ws = Workspace(n, cap, grid, cfg, dev)
+        if side is not None:
+            # all four come from the current stream's pool: work queued there may still use the blocks,
+            # and a block given up while the side stream works on it must not go back too early
+            side.wait_stream(torch.cuda.current_stream(dev))
+            for t in (I, W, bins.arena, ws.buf):
+                t.record_stream(side)
         need = gs_render_cloud(params, grid, cfg, bins, ws, I, W, stats, stream)
         if need <= cap:
             return I, W, bins, ws
-        # on a stream that is not the allocator's, kernels may still read the small bins until the
-        # next count is known
-        spent = (bins, ws) if stream is not None else None  # noqa: F841 (kept alive)
         cap = int(need * 1.25) + 1024
 
 
