@@ -436,8 +436,11 @@ __device__ __forceinline__ unsigned long long brick_row_mask(const Rec& R, const
     for (int rz = 0; rz < bsz; ++rz) {
         const float dz = dz0 + float(rz);
         const float hw2 = fmaf(nc3 * dz, dz, h0);
-        const float ish = rsqrt_approx(fmaxf(hw2, 0.0f));
-        const float sh = fmaxf(hw2, 0.0f) * ish;
+        // (bounded away from 0 and infinity, where the product of root and reciprocal root is not a number:
+        // 3e18 voxels, for a Tcull without bound, reach any row)
+        const float hw2b = fminf(fmaxf(hw2, 1e-37f), 1e37f);
+        const float ish = rsqrt_approx(hw2b);
+        const float sh = hw2b * ish;
         const float xc = fmaf(kx, dz, xrel);
         const bool in_x = fabsf(xc) <= fmaf(sh, lam, padx);
         // the section within the brick's nearer x face: at s = (y - yc) / hw its smallest |x| side is
