@@ -130,7 +130,9 @@ gs_status gs_bins_bind(void* arena, size_t arena_bytes, int64_t n_gauss, int64_t
                        const gs_grid* grid, const gs_config* cfg, gs_bins* out);
 
 /* Scratch bytes needed by gs_bin_bricks, gs_render_bwd, gs_l1_loss and gs_fit_step for this
- * problem size (one workspace serves all of them; calls sharing it must not overlap). */
+ * problem size (one workspace serves all of them; calls sharing it must not overlap). The size
+ * never falls as Gaussians, capacity, bricks or voxels grow, so a workspace sized for the largest
+ * problem serves every smaller one of the same mode (cfg->deterministic). */
 size_t gs_workspace_bytes(int64_t n_gauss, int64_t capacity, const gs_grid* grid,
                           const gs_config* cfg);
 

@@ -157,7 +157,12 @@ inline bool carve_workspace(void* base, int64_t n_gauss, int64_t capacity, int32
     const int64_t cap = capacity > 0 ? capacity : 1;
     const int64_t n = n_gauss > 0 ? n_gauss : 1;
     radix_plan(n_bricks, &ws->radix_passes, &ws->key_bits);
-    const int64_t nd = int64_t(1) << (ws->key_bits + ws->radix_passes - 1) / ws->radix_passes;  // (the widest)
+    // Counts and tiles are sized for the largest table of any smaller problem (fewer Gaussians in smaller
+    // tiles; fewer bricks in fewer, wider digits), so that a workspace serves every smaller problem too.
+    const int64_t nd0 = int64_t(1) << (ws->key_bits < kMaxRadixBits ? ws->key_bits : kMaxRadixBits);
+    const int64_t nd1 = ws->radix_passes > 2 ? kMaxDigits : int64_t(1) << (ws->key_bits + 1) / 2;
+    const int64_t small_tiles = ((n < kSmallCloud ? n : kSmallCloud) + 63) / 64, large_tiles = (n + 255) / 256;
+    const int64_t max_tiles = small_tiles > large_tiles ? small_tiles : large_tiles;
     const int64_t g_tiles = (n + gauss_tile(n) - 1) / gauss_tile(n);
     ws->stride0 = (g_tiles + 3) / 4 * 4;  // rows are scanned in 16-byte pieces
     ws->stride1 = ((cap + kSortTile - 1) / kSortTile + 3) / 4 * 4;
@@ -165,11 +170,11 @@ inline bool carve_workspace(void* base, int64_t n_gauss, int64_t capacity, int32
         const bool used = k == 0 ? ws->radix_passes > 1 : ws->radix_passes > 2;
         ws->keys[k] = reinterpret_cast<int32_t*>(take(used ? sizeof(int32_t) * cap : 256));
         ws->vals[k] = reinterpret_cast<int2*>(take(used ? sizeof(int2) * cap : 256));
-        ws->hist[k] = reinterpret_cast<int32_t*>(take(used ? sizeof(int32_t) * nd * ws->stride1 : 256));
+        ws->hist[k] = reinterpret_cast<int32_t*>(take(used ? sizeof(int32_t) * nd1 * ws->stride1 : 256));
     }
-    ws->hist0 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * nd * ws->stride0));
+    ws->hist0 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * nd0 * ((max_tiles + 3) / 4 * 4)));
     ws->rowtot = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * kMaxDigits));
-    ws->blk_base = reinterpret_cast<long long*>(take(sizeof(long long) * (g_tiles + 1)));
+    ws->blk_base = reinterpret_cast<long long*>(take(sizeof(long long) * (max_tiles + 1)));
     ws->part = reinterpret_cast<float*>(
         take(deterministic ? sizeof(float) * GRAD_FLOATS * cap : 256));
     ws->gacc = reinterpret_cast<float*>(take(sizeof(float) * GRAD_FLOATS * n));
