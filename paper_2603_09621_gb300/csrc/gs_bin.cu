@@ -10,7 +10,7 @@
 //                   status word (GS_STATUS_NONFINITE, GS_STATUS_CAPACITY).
 //   k_radix_scatter (first pass) a block writes gm_off of its Gaussians, emits their pairs into
 //                   shared memory and scatters them by digit: the Gaussian-major pair list never
-//                   goes to memory.
+//                   goes to memory. Tiles of very many pairs are shared out in parts (first_part).
 //   later passes    the same scan and scatter over tiles of 2,048 pairs, whose digit counts the
 //                   scatter before added up or, for large clouds, k_tile_count counts. Stability keeps ascending Gaussian ids inside each
 //                   brick, so the lists are deterministic. The last pass stores pair_brick (key),
@@ -359,6 +359,23 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
     return true;
 }
 
+// Digit counts of `len` pairs of consecutive keys from `key` on (a row of a box): a constant on all digits, added
+// to hall, and 1 on an interval of digits, as differences in hdif.
+__device__ __forceinline__ void count_row(int key, int len, int nd, int* hdif, int* hall) {
+    const int a = key & (nd - 1);
+    const int rem = len & (nd - 1), e = a + rem;
+    if (len >= nd) atomicAdd(hall, len / nd);
+    if (rem) {
+        atomicAdd(&hdif[a], 1);
+        if (e <= nd) {
+            atomicAdd(&hdif[e], -1);
+        } else {
+            atomicAdd(&hdif[0], 1);
+            atomicAdd(&hdif[e - nd], -1);
+        }
+    }
+}
+
 constexpr long long kBadFlag = 1LL << 62;  // marks a Gaussian tile with an invalid Gaussian
 
 // Six blocks of 256 per SM (42 registers, a few values spilled to L1) measured faster than
@@ -412,18 +429,7 @@ __global__ void __launch_bounds__(kTile, 6 * 256 / kTile) k_preprocess(
         const BrickBox o = box_of_lane(box, src);
         for (int r = lane; r < o.n[1] * o.n[2]; r += 32) {
             const int z = r / o.n[1], y = r - z * o.n[1];
-            const int a = (((o.lo[2] + z) * G.nb[1] + o.lo[1] + y) * G.nb[0] + o.lo[0]) & (nd - 1);
-            const int rem = o.n[0] & (nd - 1), e = a + rem;
-            if (o.n[0] >= nd) atomicAdd(&hall, o.n[0] / nd);
-            if (rem) {
-                atomicAdd(&hdif[a], 1);
-                if (e <= nd) {
-                    atomicAdd(&hdif[e], -1);
-                } else {
-                    atomicAdd(&hdif[0], 1);
-                    atomicAdd(&hdif[e - nd], -1);
-                }
-            }
+            count_row(((o.lo[2] + z) * G.nb[1] + o.lo[1] + y) * G.nb[0] + o.lo[0], o.n[0], nd, hdif, &hall);
         }
     }
     __syncthreads();
@@ -481,8 +487,13 @@ __global__ void __launch_bounds__(kRowThreads) k_row_scan(RowScan A) {
     long long carry = 0;
     if (row == A.nd) {
         __shared__ int bad;
-        if (tid == 0) bad = 0;
+        __shared__ long long heaviest;
+        if (tid == 0) {
+            bad = 0;
+            heaviest = 0;
+        }
         __syncthreads();
+        long long most = 0;
         for (int64_t c0 = 0; c0 < A.cols; c0 += kRowThreads) {
             const int64_t c = c0 + tid;
             long long v = c < A.cols ? A.blk[c] : 0;
@@ -490,14 +501,17 @@ __global__ void __launch_bounds__(kRowThreads) k_row_scan(RowScan A) {
                 v -= kBadFlag;
                 bad = 1;
             }
+            most = v > most ? v : most;
             long long tot;
             const long long pre = block_exclusive_scan(v, sm, &tot);
             if (c < A.cols) A.blk[c] = carry + pre;
             carry += tot;
         }
+        if (most > kFirstMinPart) atomicMax(&heaviest, most);
         __syncthreads();
         if (tid == 0) {
             A.blk[A.cols] = carry;
+            A.blk[A.cols + 1] = heaviest;
             *A.ticket = 0;
             *A.npairs = carry;
             *A.status = (bad ? GS_STATUS_NONFINITE : 0) | (carry > A.capacity ? GS_STATUS_CAPACITY : 0);
@@ -594,6 +608,8 @@ struct Scatter {
     int nbx, nby;
     int nb;                    // bricks
     int32_t* brick_off;        // (a first pass that is the last)
+    unsigned tiles;            // first pass: blocks from this one on take parts of the heavy tiles
+    unsigned block0;           // and the grid's first block
 };
 
 // Stable scatter of one tile of up to kRound keys per round. Warp w owns a contiguous part of
@@ -603,7 +619,9 @@ struct Scatter {
 // shared memory sorted by digit, ties in tile order, and written out in that order, so consecutive
 // threads store consecutive addresses of a run.
 // kFirst: the tile is emitted by the block itself from its kTile Gaussians' boxes (in rounds
-// of kRound pairs; the digits' output positions advance from round to round), else it is one
+// of kRound pairs; the digits' output positions advance from round to round; what a tile has beyond first_part
+// pairs is left to blocks for parts, whose rounds start further on: 64 Gaussians on 16,384 bricks, 1.05M pairs in one
+// tile, 6.35 -> 0.16 ms, on 131,072 bricks 51.4 -> 0.8 ms), else it is one
 // tile of the previous pass's output. kLast: the pass stores the bins' per-pair arrays; every
 // other pass of a small cloud adds each key to the next pass's digit counts at its output
 // position's tile (one atomic per group of equal (tile, digit) in a warp).
@@ -624,11 +642,11 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
     static_assert(kSortThreads >= kTile, "one thread per Gaussian of a tile");
     constexpr int kMaxRound = kSortThreads * (kFirst ? kFirstItems : kSortItems);
     static_assert(kMaxRound < 8192, "runs of a round are packed in 13 bits");
-    extern __shared__ int smem[];
     const int nd = 1 << A.bits, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    extern __shared__ int smem[];
     int* wcnt = smem;                 // [kWarps][nd]
     int* goff = wcnt + kWarps * nd;   // output position of tile slot j of digit d: goff[d] + j
-    __shared__ int skey[kMaxRound];
+    __shared__ __align__(16) int skey[kMaxRound];
     __shared__ unsigned short sidx[kMaxRound];             // sorted: tile index of each key
     __shared__ unsigned char sowner[kFirst ? kMaxRound : 1];  // tile order: Gaussian of the block
     __shared__ int2 sval[kFirst ? 1 : kSortTile];       // tile order: the keys' values
@@ -636,13 +654,35 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
 
     const int64_t P = valid_pairs(A.npairs, A.capacity);
     int64_t base = int64_t(blockIdx.x) * kSortTile;  // first pair (Gaussian-major in the first pass)
-    int total;                                       // pairs of this block
+    int tile = kFirst ? blockIdx.x + A.block0 : blockIdx.x;
+    int begin = 0, end;                              // pairs of the tile that this block places
     BrickBox box;
     box.cnt = 0;
     int loc = 0;                                     // the thread's first pair in the block
-    int gpos[kMaxDigits / kSortThreads] = {};        // the thread's digits' next output positions
+    int gpos[kMaxDigits / kSortThreads] = {};        // the thread's digits' next output positions (first: what
+                                                     // the tile places before `begin`)
     if (kFirst) {
-        const int64_t g = tid < kTile ? int64_t(blockIdx.x) * kTile + tid : A.N;
+        const int64_t part = first_part(P);
+        const bool own = static_cast<unsigned>(tile) < A.tiles;
+        if (!own) {
+            // the part [p0, p0 + part) of the pair list, as far as it lies behind the first `part` pairs of the tile
+            // that p0 falls in (any later tile's share of it is its own block's)
+            const int64_t p0 = int64_t(tile - A.tiles) * part;
+            if (A.blk_base[A.tiles + 1] <= part || p0 >= P) return;
+            int hi = static_cast<int>(A.tiles) - 1;
+            for (tile = 0; tile < hi;) {
+                const int mid = (tile + hi + 1) >> 1;
+                if (A.blk_base[mid] <= p0)
+                    tile = mid;
+                else
+                    hi = mid - 1;
+            }
+            const int64_t b = A.blk_base[tile], n = A.blk_base[tile + 1] - b;
+            begin = static_cast<int>(max(p0 - b, part));
+            end = static_cast<int>(min(p0 + part - b, n));
+            if (begin >= end) return;
+        }
+        const int64_t g = tid < kTile ? int64_t(tile) * kTile + tid : A.N;
         if (g < A.N) {
             const int4 lo = reinterpret_cast<const int4*>(A.brange + g * 8)[0];
             const int4 hi = reinterpret_cast<const int4*>(A.brange + g * 8)[1];
@@ -650,14 +690,16 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
             box.n[0] = lo.w - lo.x + 1; box.n[1] = hi.x - lo.y + 1; box.n[2] = hi.y - lo.z + 1;
             box.cnt = hi.z;
         }
-        base = A.blk_base[blockIdx.x];
+        base = A.blk_base[tile];
         // (offsets modulo 2^32: exact where the pairs fit the capacity, which is below 2^31)
         unsigned tot;
         const unsigned pre = block_exclusive_scan(static_cast<unsigned>(box.cnt),
                                                   reinterpret_cast<unsigned*>(sscan), &tot);
-        if (g < A.N) A.gm_off[g] = static_cast<int32_t>(static_cast<unsigned>(base) + pre);
-        if (g == A.N - 1) A.gm_off[A.N] = static_cast<int32_t>(static_cast<unsigned>(base) + pre + box.cnt);
-        if (kLast && blockIdx.x == 0) {
+        if (own && g < A.N) {
+            A.gm_off[g] = static_cast<int32_t>(static_cast<unsigned>(base) + pre);
+            if (g == A.N - 1) A.gm_off[A.N] = static_cast<int32_t>(static_cast<unsigned>(base) + pre + box.cnt);
+        }
+        if (kLast && blockIdx.x + A.block0 == 0) {
             // the only pass: a digit is a brick, so the digits' exclusive prefix is brick_off
             const int di = nd > kSortThreads ? nd / kSortThreads : 1;
             int row[kMaxDigits / kSortThreads], mine = 0, all;
@@ -678,18 +720,48 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
         }
         if (P == 0) return;  // also when the pairs exceed the capacity
         loc = static_cast<int>(pre);
-        total = static_cast<int>(tot);
+        if (own) {
+            end = static_cast<int>(min(int64_t(tot), part));
+        } else {
+            // digit counts of the tile's pairs before `begin`: its boxes staged in skey (first pair, size along x
+            // and y, first key), their rows shared by all warps
+            static_assert(kMaxRound >= 4 * kTile, "a tile's boxes fit the key buffer");
+            int4* sbox = reinterpret_cast<int4*>(skey);
+            int* hdif = wcnt;
+            if (tid < kTile)
+                sbox[tid] = make_int4(min(max(begin - loc, 0), box.cnt), box.n[0], box.n[1],
+                                      (box.lo[2] * A.nby + box.lo[1]) * A.nbx + box.lo[0]);
+            for (int d = tid; d <= nd + 1; d += kSortThreads) hdif[d] = 0;
+            __syncthreads();
+            for (int t = warp; t < kTile; t += kWarps) {
+                const int4 b = sbox[t];  // (pairs before `begin`, row length, rows per plane, first key)
+                if (b.x == 0) continue;
+                for (int r = lane; r <= (b.x - 1) / b.y; r += 32) {
+                    const int z = r / b.z, y = r - z * b.z;
+                    count_row(b.w + (z * A.nby + y) * A.nbx, min(b.y, b.x - r * b.y), nd, hdif, &hdif[nd + 1]);
+                }
+            }
+            __syncthreads();
+            const int di = nd > kSortThreads ? nd / kSortThreads : 1;
+            int v = 0, sum;
+            for (int e = 0; e < di; ++e) v += tid * di + e < nd ? hdif[tid * di + e] : 0;
+            int run = block_exclusive_scan(v, reinterpret_cast<int*>(sscan), &sum) + hdif[nd + 1];
+#pragma unroll
+            for (int e = 0; e < kMaxDigits / kSortThreads; ++e)
+                if (e < di && tid * di + e < nd) gpos[e] = run += hdif[tid * di + e];
+            __syncthreads();
+        }
     } else {
         if (base >= P) return;  // past the last pair: nothing to place
-        total = static_cast<int>(min(int64_t(kSortTile), P - base));
+        end = static_cast<int>(min(int64_t(kSortTile), P - base));
     }
     // rounds of kRound pairs, kItems per thread
     auto rounds_of = [&](auto items) {
         constexpr int kItems = decltype(items)::value, kRound = kSortThreads * kItems;
-        for (int c0 = 0; c0 < total; c0 += kRound) {
-            const int n = min(kRound, total - c0);
+        for (int c0 = begin; c0 < end; c0 += kRound) {
+            const int n = min(kRound, end - c0);
             if (kFirst) {
-                if (c0 > 0) __syncthreads();  // the previous round has been written out
+                if (c0 > begin) __syncthreads();  // the previous round has been written out
                 for_box(box, max(0, c0 - loc), min(box.cnt, c0 + n - loc), loc - c0, A.nbx, A.nby,
                         [&](int src, int o, int key) {
                             skey[o] = key;
@@ -748,7 +820,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
                         run += c;
                     }
                     runs[e] = run;
-                    if (c0 == 0) rows[e] = A.rowtot[d];
+                    if (c0 == begin) rows[e] = A.rowtot[d];
                 }
                 mine += (static_cast<long long>(rows[e]) << 13) | runs[e];  // (sums of runs: <= kRound)
             }
@@ -760,7 +832,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
             for (int e = 0; e < kMaxDigits / kSortThreads; ++e) {
                 const int d = tid * di + e;
                 if (e < di && d < nd) {
-                    if (c0 == 0) gpos[e] = static_cast<int>(row0) + A.hist[d * A.stride + blockIdx.x];
+                    if (c0 == begin) gpos[e] += static_cast<int>(row0) + A.hist[d * A.stride + tile];
                     goff[d] = gpos[e] - start;
                     gpos[e] += runs[e];
 #pragma unroll
@@ -785,7 +857,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
                 const int key = skey[j];
                 const int idx = sidx[j];
                 const int2 v = kFirst ? make_int2(static_cast<int>(base) + c0 + idx,
-                                                  static_cast<int>(blockIdx.x) * kTile + sowner[idx])
+                                                  tile * kTile + sowner[idx])
                                       : sval[idx];
                 const int pos = goff[(key >> A.shift) & (nd - 1)] + j;
                 A.keys_out[pos] = key;
@@ -804,7 +876,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
             }
         }
     };
-    if (kFirst && total > kSortTile)
+    if (kFirst && end - begin > kSortTile)
         rounds_of(std::integral_constant<int, kFirstItems>());
     else
         rounds_of(std::integral_constant<int, kSortItems>());
@@ -1014,6 +1086,14 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
     gs_status s = last_launch_status();
     if (s != GS_OK) return s;
     const unsigned tiles = static_cast<unsigned>((cap + kSortTile - 1) / kSortTile);
+    // Blocks for the parts of heavy tiles (no tile is heavy where its Gaussians on all bricks, or the capacity, are no
+    // more than a part). They follow the tiles' blocks, or, where the tiles are more than two per SM but fewer than
+    // the resident blocks and may take several rounds, in a launch of their own: more blocks than tiles there put a
+    // fourth tile on a few SMs (391 tiles of three rounds 101 -> 110 us; the launch costs 2 us).
+    const int64_t max_tile = int64_t(gt) * bins->n_bricks < cap ? int64_t(gt) * bins->n_bricks : cap;
+    const int64_t max_parts = max_tile > kFirstMinPart ? (cap + kFirstMinPart - 1) / kFirstMinPart : 0;
+    const unsigned parts = static_cast<unsigned>(max_parts < kFirstParts ? max_parts : kFirstParts);
+    const bool parts_apart = gb > kScatterWave / 2 && gb < kScatterWave && cap > int64_t(gb) * 2 * kFirstRound;
     for (int pass = 0, shift = 0; pass < passes; ++pass) {
         const int bits = pass_bits(ws.key_bits, passes, pass), nd = 1 << bits;
         const size_t smem = sizeof(int) * (kSortThreads / 32 + 1) * nd;
@@ -1066,6 +1146,7 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         A.gm_off = bins->gm_off;
         A.blk_base = ws.blk_base;
         A.N = N;
+        A.tiles = gb;
         A.nbx = b.nbx;
         A.nby = b.nby;
         A.nb = bins->n_bricks;
@@ -1074,7 +1155,13 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
                                 : gt == 64 ? (last ? k_radix_scatter<true, true, 64> : k_radix_scatter<true, false, 64>)
                                            : (last ? k_radix_scatter<true, true, 256> : k_radix_scatter<true, false, 256>);
         if (first || tiles > 0) {
-            launch_k(kern, dim3(first ? gb : tiles), dim3(kSortThreads), smem, st, A);
+            launch_k(kern, dim3(first ? gb + (parts_apart ? 0 : parts) : tiles), dim3(kSortThreads), smem, st, A);
+            s = last_launch_status();
+            if (s != GS_OK) return s;
+        }
+        if (first && parts_apart && parts > 0) {
+            A.block0 = gb;
+            launch_k(kern, dim3(parts), dim3(kSortThreads), smem, st, A);
             s = last_launch_status();
             if (s != GS_OK) return s;
         }

@@ -79,6 +79,19 @@ constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
 // registers; with the keys read again from shared memory instead, 10 (12) take 171 (171) us and 2.34 (2.28) ms, but
 // 69.3 (69.4) us against 67.5 at 375,000 with 5.6 pairs and 89.9 (89.3) against 88.8 at 500,000.
 constexpr int kFirstItems = 9;
+// A tile's own block places at most first_part(P) of its pairs; what is left of a heavier tile is taken in parts
+// of that size by further blocks, each of which first counts the digits of the tile's pairs before its part (by
+// rows of the boxes). So a block's serial work follows the pairs in all, not the widest Gaussians: four
+// rounds at least, and no less than twice an even share of the pairs among the resident blocks, so that clouds whose
+// tiles are all alike are not cut up (with one share 12.3M pairs in 391 tiles 490 -> 525 us).
+constexpr int kFirstRound = kSortThreads * kFirstItems;
+constexpr int kFirstMinPart = 4 * kFirstRound;
+constexpr int kScatterWave = 152 * 4;  // resident scatter blocks
+constexpr int kFirstParts = kScatterWave / 2;
+__host__ __device__ inline int64_t first_part(int64_t pairs) {
+    const int64_t share = (pairs / kFirstParts / kFirstRound + 1) * kFirstRound;  // > pairs / kFirstParts
+    return share > kFirstMinPart ? share : kFirstMinPart;
+}
 constexpr int kMaxRadixBits = 9;
 constexpr int kMaxDigits = 1 << kMaxRadixBits;
 // Gaussians per block of the preprocess and emission kernels. A cloud that would fill no more than one
@@ -100,7 +113,8 @@ struct Workspace {
                              // Gaussian tile (row stride stride0)
     int32_t* hist[2];        // later passes': a column per kSortTile pairs (row stride stride1)
     int32_t* rowtot;         // [kMaxDigits] totals of the digits of the pass being scanned
-    long long* blk_base;     // [Gaussian tiles + 1] pairs of each tile, then their exclusive sums
+    long long* blk_base;     // [Gaussian tiles + 2] pairs of each tile, then their exclusive sums (one more
+                             // entry than tiles) and the heaviest tile's pairs
     int64_t stride0, stride1;
     int32_t key_bits, radix_passes;
     float* part;             // [capacity, 12] per-pair partial gradients (deterministic mode)
@@ -174,7 +188,7 @@ inline bool carve_workspace(void* base, int64_t n_gauss, int64_t capacity, int32
     }
     ws->hist0 = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * nd0 * ((max_tiles + 3) / 4 * 4)));
     ws->rowtot = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * kMaxDigits));
-    ws->blk_base = reinterpret_cast<long long*>(take(sizeof(long long) * (max_tiles + 1)));
+    ws->blk_base = reinterpret_cast<long long*>(take(sizeof(long long) * (max_tiles + 2)));
     ws->part = reinterpret_cast<float*>(
         take(deterministic ? sizeof(float) * GRAD_FLOATS * cap : 256));
     ws->gacc = reinterpret_cast<float*>(take(sizeof(float) * GRAD_FLOATS * n));
