@@ -7,6 +7,7 @@ is missing (there is no fallback path). Function names follow the C ABI.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 from dataclasses import dataclass, field
 
@@ -326,9 +327,17 @@ class Bins:
 
 class Workspace:
     def __init__(self, n_gauss: int, capacity: int, grid: Grid, cfg: Config, device="cuda"):
-        lib = load()
-        g, c = grid.c(), cfg.c()
-        self.nbytes = lib.gs_workspace_bytes(n_gauss, capacity, ctypes.byref(g), ctypes.byref(c))
+        self._allocate(n_gauss, capacity, grid.c(), cfg.c(), device)
+
+    @classmethod
+    def for_bins(cls, bins: Bins) -> "Workspace":
+        """Scratch for the problem that `bins` was made for."""
+        ws = cls.__new__(cls)
+        ws._allocate(bins.n_gauss, bins.capacity, bins._g, bins._c, bins.arena.device)
+        return ws
+
+    def _allocate(self, n_gauss, capacity, g, c, device):
+        self.nbytes = load().gs_workspace_bytes(n_gauss, capacity, ctypes.byref(g), ctypes.byref(c))
         if self.nbytes == 0:
             raise GsError("gs_workspace_bytes: invalid arguments")
         self.buf = _empty_bytes(self.nbytes, device)
@@ -363,8 +372,11 @@ def gs_render_fwd(bins: Bins, grid: Grid, cfg: Config, I=None, W=None, stats=Non
 
 def gs_render_bwd(params, bins: Bins, grid: Grid, cfg: Config, I, W, dI, ws: Workspace,
                   dparams=None, stream=None):
+    return _render_bwd(params, bins, grid.c(), cfg.c(), I, W, dI, ws, dparams, stream)
+
+
+def _render_bwd(params, bins, g, c, I, W, dI, ws, dparams=None, stream=None):
     dparams = torch.empty_like(params) if dparams is None else dparams
-    g, c = grid.c(), cfg.c()
     _check(load().gs_render_bwd(_ptr(params), ctypes.byref(bins.c), ctypes.byref(g),
                                 ctypes.byref(c), _ptr(I), _ptr(W), _ptr(dI), _ptr(dparams),
                                 _ptr(ws.buf), ws.nbytes, _stream(stream)), "gs_render_bwd")
@@ -488,8 +500,11 @@ def gs_render_cloud(params: torch.Tensor, grid: Grid, cfg: Config, bins: Bins, w
                     stats=None, stream=None) -> int:
     """Bin and render; returns the pairs needed once they are known (the render may still run).
     More than bins.capacity: nothing was rendered."""
+    return _render_cloud(params, grid.c(), cfg.c(), bins, ws, I, W, stats, stream)
+
+
+def _render_cloud(params, g, c, bins, ws, I, W, stats, stream):
     assert params.is_contiguous() and params.dtype == torch.float32
-    g, c = grid.c(), cfg.c()
     need = ctypes.c_int64(0)
     rc = load().gs_render_cloud(_ptr(params), ctypes.byref(g), ctypes.byref(c), ctypes.byref(bins.c),
                                 _ptr(ws.buf), ws.nbytes, _ptr(I), _ptr(W), _ptr(stats),
@@ -513,21 +528,24 @@ def render(params: torch.Tensor, grid: Grid, cfg: Config = Config(), capacity: i
     Returns (I, W, bins, workspace)."""
     n, dev = params.shape[0], params.device
     # 16 pairs per Gaussian; small clouds, whose retry costs more than their memory (72 bytes per
-    # pair), get up to 64
-    cap = capacity if capacity is not None else max(1024, 16 * n, min(64 * n, 1 << 20))
+    # pair), get up to 64; no cloud has more than all bricks for each Gaussian
+    cap = capacity
+    if cap is None:
+        bricks = math.prod(-(-d // max(b, 1)) for d, b in zip((grid.nx, grid.ny, grid.nz), cfg.brick))
+        cap = max(1024, min(max(16 * n, min(64 * n, 1 << 20)), n * bricks))
     side = _foreign_stream(stream, dev)
     I = torch.empty(grid.shape, dtype=torch.float32, device=dev)
     W = torch.empty(grid.shape, dtype=torch.float32, device=dev)
     while True:
         bins = Bins(n, cap, grid, cfg, dev)
-        ws = Workspace(n, cap, grid, cfg, dev)
+        ws = Workspace.for_bins(bins)
         if side is not None:
             # all four come from the current stream's pool: work queued there may still use the blocks,
             # and a block given up while the side stream works on it must not go back too early
             side.wait_stream(torch.cuda.current_stream(dev))
             for t in (I, W, bins.arena, ws.buf):
                 t.record_stream(side)
-        need = gs_render_cloud(params, grid, cfg, bins, ws, I, W, stats, stream)
+        need = _render_cloud(params, bins._g, bins._c, bins, ws, I, W, stats, stream)
         if need <= cap:
             return I, W, bins, ws
         cap = int(need * 1.25) + 1024
@@ -541,13 +559,14 @@ class GaussianRender(torch.autograd.Function):
         params = params.contiguous()
         I, W, bins, ws = render(params, grid, cfg)
         ctx.save_for_backward(params, I, W)
-        ctx.bins, ctx.ws, ctx.grid, ctx.cfg = bins, ws, grid, cfg
+        ctx.bins = bins  # (the scratch, most of what render() returns, is not kept until the backward pass)
         return I
 
     @staticmethod
     def backward(ctx, dI):
         params, I, W = ctx.saved_tensors
-        dparams = gs_render_bwd(params, ctx.bins, ctx.grid, ctx.cfg, I, W, dI.contiguous(), ctx.ws)
+        ws = Workspace.for_bins(ctx.bins)
+        dparams = _render_bwd(params, ctx.bins, ctx.bins._g, ctx.bins._c, I, W, dI.contiguous(), ws)
         return dparams, None, None
 
 
