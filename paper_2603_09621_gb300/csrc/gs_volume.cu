@@ -15,7 +15,7 @@ namespace gs {
 static std::atomic<unsigned long long> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
-// Slice profile and its adjoint over a 2D grid: blockIdx.y strides over the LR slices, a thread
+// Slice profile and its adjoint over a 2D grid of 2D blocks: y strides over the LR slices, a thread
 // owns kV consecutive voxels of a plane (4: 16-byte accesses, for aligned volumes whose planes
 // are a multiple of 4 voxels; else 1), so no voxel needs an index division. Bound by HBM. The
 // adjoint reads each LR value once for its s HR slices and took 33 us with one HR voxel and two
@@ -43,19 +43,29 @@ __device__ __forceinline__ void store_voxels(float* dst, const Voxels<kV>& r) {
         *dst = r.v[0];
 }
 
-template <int kV>
-__global__ void __launch_bounds__(256) k_downsample_fwd(const float* __restrict__ hr, int64_t plane, int nzl,
-                                                        int s, float inv_s, float* __restrict__ lr) {
+// kS: slices per LR slice at compile time, their loads in flight together (0: any number s_, four or six at a
+// time). With the loop left to the compiler two slices took 23 us where 18 are enough (300 x 256 x 256).
+template <int kV, int kS>
+__global__ void __launch_bounds__(256) k_downsample_fwd(const float* __restrict__ hr, unsigned plane,
+                                                        unsigned nzl, int s_, float inv_s,
+                                                        float* __restrict__ lr) {
     pdl_enter();
-    for (int k = blockIdx.y; k < nzl; k += gridDim.y) {
+    constexpr int kBatch = kS > 0 ? kS : (kV == 4 ? 4 : 6);
+    const int s = kS > 0 ? kS : s_;
+    for (unsigned k = blockIdx.y * blockDim.y + threadIdx.y; k < nzl; k += gridDim.y * blockDim.y) {
         const float* src = hr + int64_t(k) * s * plane;
-        for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) * kV; r < plane;
-             r += int64_t(gridDim.x) * blockDim.x * kV) {
+        for (unsigned r = (blockIdx.x * blockDim.x + threadIdx.x) * kV; r < plane; r += gridDim.x * blockDim.x * kV) {
             Voxels<kV> acc = {};
-            for (int j = 0; j < s; ++j) {
-                const Voxels<kV> x = load_voxels<kV>(src + int64_t(j) * plane + r);
+            for (int j0 = 0; j0 < s; j0 += kBatch) {
+                Voxels<kV> x[kBatch];
 #pragma unroll
-                for (int e = 0; e < kV; ++e) acc.v[e] += x.v[e];
+                for (int j = 0; j < kBatch; ++j)
+                    if (kS > 0 || j0 + j < s) x[j] = load_voxels<kV>(src + int64_t(j0 + j) * plane + r);
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j)
+                    if (kS > 0 || j0 + j < s)
+#pragma unroll
+                        for (int e = 0; e < kV; ++e) acc.v[e] += x[j].v[e];
             }
 #pragma unroll
             for (int e = 0; e < kV; ++e) acc.v[e] *= inv_s;
@@ -66,15 +76,14 @@ __global__ void __launch_bounds__(256) k_downsample_fwd(const float* __restrict_
 
 // (slice nzl stands for the trailing HR slices, whose gradient is zero)
 template <int kV>
-__global__ void __launch_bounds__(256) k_downsample_bwd(const float* __restrict__ dlr, int nz, int64_t plane,
-                                                        int nzl, int s, float inv_s,
+__global__ void __launch_bounds__(256) k_downsample_bwd(const float* __restrict__ dlr, int nz, unsigned plane,
+                                                        unsigned nzl, int s, float inv_s,
                                                         float* __restrict__ dhr) {
     pdl_enter();
-    for (int k = blockIdx.y; k <= nzl; k += gridDim.y) {
-        const int j1 = k < nzl ? s : nz - nzl * s;
+    for (unsigned k = blockIdx.y * blockDim.y + threadIdx.y; k <= nzl; k += gridDim.y * blockDim.y) {
+        const int j1 = k < nzl ? s : nz - static_cast<int>(nzl) * s;
         float* dst = dhr + int64_t(k) * s * plane;
-        for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) * kV; r < plane;
-             r += int64_t(gridDim.x) * blockDim.x * kV) {
+        for (unsigned r = (blockIdx.x * blockDim.x + threadIdx.x) * kV; r < plane; r += gridDim.x * blockDim.x * kV) {
             Voxels<kV> x = {};
             if (k < nzl) {
                 x = load_voxels<kV>(dlr + int64_t(k) * plane + r);
@@ -260,9 +269,24 @@ __global__ void __launch_bounds__(kL1Threads, 7) k_profile_loss(
     l1_finish(acc, inv_n, partials, ticket, loss);
 }
 
-static dim3 grid2d(int64_t per_plane, int64_t slices) {
-    const int64_t bx = (per_plane + 255) / 256;
-    return dim3(static_cast<unsigned>(bx < 64 ? bx : 64), static_cast<unsigned>(slices < 65535 ? slices : 65535));
+// Blocks of up to 256 threads over a plane's pieces (whole warps where there are 32 or more), the rest over the
+// slices; about 32 blocks per SM, so few large planes and many small ones fill the chip too: a grid of at most 64
+// blocks per slice with all threads along the plane took 185 us where 27 are enough (4 planes of 2,047 x 2,047, s =
+// 4) and 52 in place of 7 (100,000 planes of one voxel).
+struct Grid2d {
+    dim3 grid, block;
+};
+
+static Grid2d grid2d(int64_t per_plane, int64_t slices) {
+    unsigned tx = 1;
+    if (per_plane < 32)
+        while (tx < per_plane) tx *= 2;
+    else
+        tx = per_plane < 256 ? static_cast<unsigned>((per_plane + 31) / 32 * 32) : 256;
+    const unsigned ty = 256 / tx;
+    const int64_t by = slices < 1 ? 1 : (slices + ty - 1) / ty, gy = by < 65535 ? by : 65535;
+    const int64_t bx = (per_plane + tx - 1) / tx, most = 152 * 32 / gy > 64 ? 152 * 32 / gy : 64;
+    return {dim3(static_cast<unsigned>(bx < most ? bx : most), static_cast<unsigned>(gy)), dim3(tx, ty)};
 }
 
 static bool vec_ok(const void* a, const void* b, int64_t plane) {
@@ -312,12 +336,23 @@ gs_status downsample_fwd_impl(const float* hr, int nz, int ny, int nx, int s, fl
     const int nzl = nz / s;
     const int64_t plane = int64_t(ny) * nx;
     if (nzl == 0) return GS_OK;
-    if (vec_ok(hr, lr, plane))
-        launch_k(k_downsample_fwd<4>, grid2d(plane / 4, nzl), dim3(256), 0, st, hr, plane, nzl, s,
+    const bool vec = vec_ok(hr, lr, plane);
+    const Grid2d g = grid2d(vec ? plane / 4 : plane, nzl);
+    auto go = [&](auto kernel) {
+        launch_k(kernel, g.grid, g.block, 0, st, hr, static_cast<unsigned>(plane), static_cast<unsigned>(nzl), s,
             1.0f / float(s), lr);
-    else
-        launch_k(k_downsample_fwd<1>, grid2d(plane, nzl), dim3(256), 0, st, hr, plane, nzl, s,
-            1.0f / float(s), lr);
+    };
+    switch (s) {
+        case 1: vec ? go(k_downsample_fwd<4, 1>) : go(k_downsample_fwd<1, 1>); break;
+        case 2: vec ? go(k_downsample_fwd<4, 2>) : go(k_downsample_fwd<1, 2>); break;
+        case 3: vec ? go(k_downsample_fwd<4, 3>) : go(k_downsample_fwd<1, 3>); break;
+        case 4: vec ? go(k_downsample_fwd<4, 4>) : go(k_downsample_fwd<1, 4>); break;
+        case 5: vec ? go(k_downsample_fwd<4, 5>) : go(k_downsample_fwd<1, 5>); break;
+        case 6: vec ? go(k_downsample_fwd<4, 6>) : go(k_downsample_fwd<1, 6>); break;
+        case 7: vec ? go(k_downsample_fwd<4, 7>) : go(k_downsample_fwd<1, 7>); break;
+        case 8: vec ? go(k_downsample_fwd<4, 8>) : go(k_downsample_fwd<1, 8>); break;
+        default: vec ? go(k_downsample_fwd<4, 0>) : go(k_downsample_fwd<1, 0>);
+    }
     return last_launch_status();
 }
 
@@ -325,12 +360,10 @@ gs_status downsample_bwd_impl(const float* dlr, int nz, int ny, int nx, int s, f
                               cudaStream_t st) {
     const int nzl = nz / s;
     const int64_t plane = int64_t(ny) * nx;
-    if (vec_ok(dlr, dhr, plane))
-        launch_k(k_downsample_bwd<4>, grid2d(plane / 4, nzl + 1), dim3(256), 0, st, dlr, nz, plane, nzl, s,
-            1.0f / float(s), dhr);
-    else
-        launch_k(k_downsample_bwd<1>, grid2d(plane, nzl + 1), dim3(256), 0, st, dlr, nz, plane, nzl, s,
-            1.0f / float(s), dhr);
+    const bool vec = vec_ok(dlr, dhr, plane);
+    const Grid2d g = grid2d(vec ? plane / 4 : plane, nzl + (nz > nzl * s ? 1 : 0));
+    launch_k(vec ? k_downsample_bwd<4> : k_downsample_bwd<1>, g.grid, g.block, 0, st, dlr, nz,
+        static_cast<unsigned>(plane), static_cast<unsigned>(nzl), s, 1.0f / float(s), dhr);
     return last_launch_status();
 }
 
