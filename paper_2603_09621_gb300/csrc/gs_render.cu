@@ -8,10 +8,10 @@
 // in both kernels from the voxel's global index and the Gaussian alone, so forward and
 // adjoint agree on every inclusion decision and no result depends on the brick shape.
 //
-// Forward: the brick is split into 4 x 4 x 4 footprints, a quarter-warp each; a lane owns the two
-// x-rows of four voxels at z and z + 1. The block stages the brick's list in rounds of 20 records
+// Forward: the brick is split into 4 x 4 x 4 footprints, a quarter-warp each (a half or a whole warp in bricks of
+// two or one); a lane owns the two x-rows of four (two, one) voxels at z and z + 1. The block stages the brick's list in rounds of 20 records
 // per footprint (160 for an 8^3 brick); smaller bricks, with shorter lists, take shorter rounds
-// and keep more blocks resident. The thread that stages a record tests it against every footprint
+// (64 records for one or two footprints) and keep more blocks resident. The thread that stages a record tests it against every footprint
 // (three conservative tests, see foot_mask: the triangle inequality in whitened space
 // |M (p - mu)| >= |M (c - mu)| - rho4, with rho4 the whitened radius of the footprint around its
 // centre c; the truncated ellipsoid's bounding box widened by 3/2 along each axis; and q's lower
@@ -45,8 +45,8 @@
 
 namespace gs {
 
-constexpr int kFwdChunkPerFoot = 20;  // Gaussians staged per forward round and 4^3 footprint
-                                      // (in steps of a factor 2: 40, 80 or 160 records)
+constexpr int kFwdChunkPerFoot = 20;  // Gaussians staged per forward round and 4^3 footprint (80 or 160 records)
+constexpr int kFwdChunkSmall = 64;    // and for bricks of one or two footprints (see k_render_fwd)
 constexpr int kBwdThreads = 128;
 constexpr int kBwdPairs = 256;        // pairs per adjoint block, taken by warps 32 at a time
 constexpr int kBwdStage = 4;          // bricks of per-voxel factors staged per adjoint block
@@ -180,7 +180,7 @@ __device__ __forceinline__ unsigned foot_mask(const Rec& R, const RenderGeo& G, 
 
 // ------------------------------------------------------------------------ forward
 
-// One block of 32 or 64 threads per brick (kWide: a warp per footprint, below). What bounds it is instruction issue (72 % active) and
+// One block of 32 or 64 threads per brick (more with kFew, below). What bounds it is instruction issue (72 % active) and
 // the latency of the gathered records, so work per instruction decides:
 //   - A quarter-warp per 4^3 footprint, a lane owning the x-rows at z and z + 1: the row terms,
 //     offsets and exponents of the two rows run as FP32x2 pairs (element by element the scalar
@@ -201,19 +201,24 @@ __device__ __forceinline__ unsigned foot_mask(const Rec& R, const RenderGeo& G, 
 //     records 212 us and 5.20 ms; 24 records 207 us but 5.50 ms; 64 registers (spills) 216 us;
 //     96 registers 217 us. Rounds double-buffered with cp.async measured slower (242 against
 //     241 us, 7.06 against 6.13 ms).
+// kLanes: lanes per footprint, 8 as above; 16 in bricks of two footprints and 32 in bricks of one, which would leave half or
+// three quarters of the only warp idle. Rounds of 64 records there fill the staging passes of 32. Random clouds
+// on 128^3, against a quarter-warp and rounds of 40: 8 x 4 x 4 bricks 193 -> 142 us, 4^3 314 -> 202 (a half-warp per
+// footprint throughout took 146 and 221; rounds of 32 or 96: 148 and 205, 151 and 209).
 // A grid of few bricks leaves most schedulers with one warp or none, and a brick's time is the latency
-// of its lists. There (kWide) a footprint gets a whole warp, each lane the two voxels at z and z + 1,
+// of its lists. There (kFew) a footprint gets a whole warp, each lane the two voxels at z and z + 1,
 // and a thread fetches its record of the next round while the present one is evaluated. Forward us,
-// narrow -> wide: 8 bricks of 8^3 25 -> 21, 64 bricks 33-38 -> 26-28 (random and clustered clouds), 216
+// narrow -> whole warps: 8 bricks of 8^3 25 -> 21, 64 bricks 33-38 -> 26-28 (random and clustered clouds), 216
 // bricks 35-46 -> 34-36, but 512 bricks 41-53 -> 51-56 and 4,096 bricks 146 -> 270: a lane with one
 // voxel per row repeats the row terms four times as often. 8 x 8 x 4 bricks: 128 of them 36-42 ->
-// 24-26, 1,024 43-64 -> 48-54. So wide where all footprints' warps are resident at once (152 SMs of 2
-// blocks of 8 warps: 304 bricks of 8^3, 608 of 8 x 8 x 4). Eight hits per iteration 1-2 us slower.
-constexpr int64_t kWideFootprints = 152 * 16;
+// 24-26, 1,024 43-64 -> 48-54. So where all footprints' warps are resident at once (152 SMs of 2
+// blocks of 8 warps: 304 bricks of 8^3, 608 of 8 x 8 x 4; bricks of one footprint have two warps, for staging). Eight
+// hits per iteration 1-2 us slower.
+constexpr int64_t kFewFootprints = 152 * 16;
 constexpr int kFwdHits = 4;  // hits per iteration of the evaluation loop (one 32-bit list word)
 
-template <bool kStats, int kChunk, bool kWide>
-__global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd(const int32_t* __restrict__ brick_off,
+template <bool kStats, int kChunk, int kLanes, bool kFew>
+__global__ void __launch_bounds__(kFew ? 256 : 64, kFew ? 2 : 14) k_render_fwd(const int32_t* __restrict__ brick_off,
                                                        const int32_t* __restrict__ pair_gid,
                                                        const float4* __restrict__ rec4, RenderGeo G,
                                                        float* __restrict__ I, float* __restrict__ W,
@@ -229,12 +234,12 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
     const int b = blockIdx.x;
     int bx, by, bz;
     brick_xyz(b, G, bx, by, bz);
-    // quarter-warp per 4^3 footprint, a lane owns two x-rows of 4 voxels, at z and z + 1; kWide: a
-    // warp per footprint, a lane owns voxel lx of the two rows
-    constexpr int kFoot = kWide ? 1 : 4;  // footprints per warp
-    constexpr int kX = kWide ? 1 : 4;     // voxels of a row per lane
-    const int foot = tid / (32 / kFoot), foot0 = (tid >> 5) * kFoot;
-    const int lx = kWide ? lane & 3 : 0, lyz = kWide ? lane >> 2 : lane & 7;
+    // kLanes lanes per 4^3 footprint, a lane owns kX voxels from lx on of two x-rows, at z and z + 1
+    static_assert(kLanes == 8 || kLanes == 16 || kLanes == 32, "a lane owns 4, 2 or 1 voxels of a row");
+    constexpr int kFoot = 32 / kLanes;  // footprints per warp
+    constexpr int kX = 32 / kLanes;
+    const int foot = tid / kLanes, foot0 = (tid >> 5) * kFoot;
+    const int lx = (lane % (kLanes / 8)) * kX, lyz = (lane % kLanes) / (kLanes / 8);
     const int n_foot = G.fx * G.fy * G.fz;
     const bool foot_ok = foot < n_foot;
     const int f = foot_ok ? foot : 0;
@@ -251,8 +256,8 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
     for (int xi = 0; xi < kX; ++xi) SWa[xi] = SWb[xi] = f2(0.f, 0.f);
     unsigned long long n_eff = 0, n_eval = 0;
     const int start = brick_off[b], end = brick_off[b + 1];
-    // kWide: a thread stages at most one record per round, loaded while the round before is evaluated
-    float4 qw[kWide ? REC_F4 : 1];
+    // kFew: a thread stages at most one record per round, loaded while the round before is evaluated
+    float4 qw[kFew ? REC_F4 : 1];
     auto fetch = [&](int gid, float4 (&q)[REC_F4]) {
         const float4* src = rec4 + int64_t(gid) * REC_F4;
 #pragma unroll
@@ -271,13 +276,13 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
         srec[3][k] = q[4];
     };
     int gid = start + tid < end ? pair_gid[start + tid] : 0;  // the thread's next record
-    if constexpr (kWide) {
+    if constexpr (kFew) {
         if (start + tid < end && tid < kChunk) fetch(gid, qw);
     }
     for (int c0 = start; c0 < end; c0 += kChunk) {
         const int cnt = min(kChunk, end - c0);
         if (c0 != start) __syncthreads();  // the previous chunk's records are no longer read
-        if constexpr (kWide) {
+        if constexpr (kFew) {
             if (tid < cnt) put(tid, qw);
         } else {
             for (int k = tid; k < cnt; k += nthreads) {
@@ -290,7 +295,7 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
         }
         __syncthreads();
         if (c0 + kChunk + tid < end) gid = pair_gid[c0 + kChunk + tid];
-        if constexpr (kWide) {
+        if constexpr (kFew) {
             if (c0 + kChunk + tid < end && tid < kChunk) fetch(gid, qw);
         }
         // each warp lists the hits of its footprints in ascending Gaussian id
@@ -307,8 +312,10 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
             }
         }
         int myn = n[0];
-        if constexpr (!kWide)
+        if constexpr (kFoot == 4)
             myn = (lane & 16) ? ((lane & 8) ? n[3] : n[2]) : ((lane & 8) ? n[1] : n[0]);
+        else if constexpr (kFoot == 2)
+            myn = (lane & 16) ? n[1] : n[0];
         if (lyz < kFwdHits && lx == 0) slist[foot][myn + lyz] = static_cast<unsigned char>(kChunk);
         __syncwarp();
         for (int i = 0; i < myn; i += kFwdHits) {
@@ -330,8 +337,8 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
 #pragma unroll
                 for (int xi = 0; xi < kX; ++xi) {
                     // (k = 0 in the packed FMA gives tq0 itself)
-                    const float k = kWide ? float(lx) : float(xi);
-                    const float2 tq = (!kWide && xi == 0) ? tq0 : fma2(f2(k, k), sa2, tq0);
+                    const float k = float(lx + xi);
+                    const float2 tq = (kX == 4 && xi == 0) ? tq0 : fma2(f2(k, k), sa2, tq0);
                     const float2 q = fma2(tq, tq, Sr);
                     if (q.x <= G.T) {
                         const float g = ex2_approx(-q.x);
@@ -363,7 +370,7 @@ __global__ void __launch_bounds__(kWide ? 256 : 64, kWide ? 2 : 14) k_render_fwd
             Wv[xi] = h ? SWb[xi].y : SWa[xi].y;
             Iv[xi] = S / (Wv[xi] > G.eps ? Wv[xi] : G.eps);
         }
-        if constexpr (!kWide) {
+        if constexpr (kX == 4) {
             if (ox + 3 < G.nx && (G.nx & 3) == 0) {
                 store4<true>(I + row, Iv);
                 store4<true>(W + row, Wv);
@@ -845,26 +852,33 @@ gs_status render_fwd_impl(const gs_bins* bins, const gs_grid* grid, const gs_con
     // records staged per round about in proportion to the footprints (the lists of smaller
     // bricks are shorter), so that smaller bricks keep more blocks resident
     const float4* rec4 = reinterpret_cast<const float4*>(bins->rec);
-    const bool wide = int64_t(bins->n_bricks) * n_foot <= kWideFootprints;
-    // (wide: a thread per record of a round, so two warps also for a single footprint)
-    const int threads = wide ? 32 * (n_foot > 1 ? n_foot : 2) : 32 * ((n_foot + 3) / 4);
+    const bool few = int64_t(bins->n_bricks) * (n_foot > 1 ? n_foot : 2) <= kFewFootprints;
+    const int lanes = few || n_foot == 1 ? 32 : (n_foot == 2 ? 16 : 8);
+    // (few: a thread per record of a round, so two warps also for a single footprint)
+    const int threads = few && n_foot == 1 ? 64 : 32 * ((n_foot * lanes + 31) / 32);
     auto go = [&](auto kernel) {
         launch_k(kernel, dim3(bins->n_bricks), dim3(threads), 0, st, bins->brick_off, bins->pair_gid,
             rec4, G, I, W, stats);
     };
     auto pick = [&](auto chunk) {
         constexpr int kChunk = decltype(chunk)::value;
-        if (wide)
-            stats ? go(k_render_fwd<true, kChunk, true>) : go(k_render_fwd<false, kChunk, true>);
-        else
-            stats ? go(k_render_fwd<true, kChunk, false>) : go(k_render_fwd<false, kChunk, false>);
+        if (few)
+            stats ? go(k_render_fwd<true, kChunk, 32, true>) : go(k_render_fwd<false, kChunk, 32, true>);
+        else if (n_foot > 2)
+            stats ? go(k_render_fwd<true, kChunk, 8, false>) : go(k_render_fwd<false, kChunk, 8, false>);
+        else if constexpr (kChunk == kFwdChunkSmall) {
+            if (n_foot == 2)
+                stats ? go(k_render_fwd<true, kChunk, 16, false>) : go(k_render_fwd<false, kChunk, 16, false>);
+            else
+                stats ? go(k_render_fwd<true, kChunk, 32, false>) : go(k_render_fwd<false, kChunk, 32, false>);
+        }
     };
     if (n_foot >= 6)
         pick(std::integral_constant<int, 8 * kFwdChunkPerFoot>{});
     else if (n_foot >= 3)
         pick(std::integral_constant<int, 4 * kFwdChunkPerFoot>{});
     else
-        pick(std::integral_constant<int, 2 * kFwdChunkPerFoot>{});
+        pick(std::integral_constant<int, kFwdChunkSmall>{});
     return last_launch_status();
 }
 
