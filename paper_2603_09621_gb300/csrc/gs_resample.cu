@@ -48,6 +48,14 @@ __device__ __forceinline__ void res_range(const ResAxis& A, int i, int& jlo, int
     jhi = min(A.n_dst - 1, static_cast<int>(ceilf((float(i) + 1.5f) * A.inv - 0.5f)) + 1);
 }
 
+// Threads along a row of n pieces: up to 256 in whole warps, or the power of two that covers a short row.
+__host__ __device__ inline int row_threads(int n) {
+    if (n >= 32) return n >= 256 ? 256 : (n + 31) / 32 * 32;
+    int t = 1;
+    while (t < n) t *= 2;
+    return t;
+}
+
 // A thread owns one destination column x of a plane z and walks kRows rows y: its x and z taps are
 // formed once, and an element offset (T: 32 bits where the source allows) is a sum of precomputed
 // parts. Bound by instruction issue: one voxel per thread with three index remainders and 64-bit
@@ -68,7 +76,7 @@ __global__ void __launch_bounds__(256) k_resample_fwd(const float* __restrict__ 
     res_map(AX, x, x0, x1, wx);
     const float ux = 1.0f - wx;
     const T sx = T(AX.n_src), sxy = sx * T(AY.n_src);
-    for (int z = blockIdx.z; z < AZ.n_dst; z += gridDim.z) {
+    for (int z = blockIdx.z * blockDim.z + threadIdx.z; z < AZ.n_dst; z += gridDim.z * blockDim.z) {
         int z0, z1;
         float wz;
         res_map(AZ, z, z0, z1, wz);
@@ -307,17 +315,52 @@ static unsigned res_blocks(int64_t n) {
 gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t snx, float* dst,
                             int32_t dnz, int32_t dny, int32_t dnx, cudaStream_t st) {
     const ResGeo G = make_res(snz, sny, snx, dnz, dny, dnx);
-    // columns in whole warps, the rest of the block's threads over rows
     const bool narrow = int64_t(snz) * sny * snx <= (int64_t(1) << 31) - 1;
     const bool rows4 = int64_t(dnz) * dny * dnx >= kFwdRowsMin;
-    const int tx = dnx >= 256 ? 256 : (dnx + 31) / 32 * 32, ty = 256 / tx, per = ty * (rows4 ? 4 : 1);
-    const int64_t gx = (int64_t(dnx) + tx - 1) / tx, gy = (int64_t(dny) + per - 1) / per;
+    // a block's threads over columns (whole warps, or a power of two of a narrow volume's), then rows, then planes:
+    // with whole warps along any row 1,024 x 1,024 samples of one column took 146 us, 15 now
+    const int tx = row_threads(dnx), rows = rows4 ? 4 : 1;
+    int ty = 1, tz = 1;
+    while (2 * ty * tx <= 256 && ty * rows < dny) ty *= 2;
+    while (2 * tz * ty * tx <= 256 && tz < dnz && tz < 64) tz *= 2;
+    const int64_t gx = (int64_t(dnx) + tx - 1) / tx, gy = (int64_t(dny) + ty * rows - 1) / (ty * rows);
+    const int64_t gz = (int64_t(dnz) + tz - 1) / tz;
     const dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy < 65535 ? gy : 65535),
-                    static_cast<unsigned>(dnz < 65535 ? dnz : 65535));
+                    static_cast<unsigned>(gz < 65535 ? gz : 65535));
     launch_k(narrow ? (rows4 ? k_resample_fwd<unsigned, 4> : k_resample_fwd<unsigned, 1>)
                     : (rows4 ? k_resample_fwd<int64_t, 4> : k_resample_fwd<int64_t, 1>),
-        grid, dim3(tx, ty), 0, st, src, G, dst);
+        grid, dim3(tx, ty, tz), 0, st, src, G, dst);
     return last_launch_status();
+}
+
+// The adjoint of kV consecutive voxels from v on: as it is, or (kPrep) as the adjoint render's factors.
+template <bool kPrep, int kV>
+__device__ __forceinline__ void emit_voxels(int64_t v, const float (&acc)[kV], const float* __restrict__ Iv,
+                                            const float* __restrict__ Wv, float eps, float* __restrict__ dsrc,
+                                            float2* __restrict__ aip) {
+    if constexpr (kPrep) {
+        float w[kV], iv[kV];
+        float2 a[kV];
+        if constexpr (kV == 4) {
+            load4<true>(Wv + v, w);
+            load4<true>(Iv + v, iv);
+        } else {
+            w[0] = Wv[v];
+            iv[0] = Iv[v];
+        }
+#pragma unroll
+        for (int e = 0; e < kV; ++e) a[e] = adj_factor(acc[e], w[e], iv[e], eps);
+        if constexpr (kV == 4) {
+            reinterpret_cast<float4*>(aip + v)[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+            reinterpret_cast<float4*>(aip + v)[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
+        } else {
+            aip[v] = a[0];
+        }
+    } else if constexpr (kV == 4) {
+        store4<true>(dsrc + v, acc);
+    } else {
+        dsrc[v] = acc[0];
+    }
 }
 
 // Separable form of the adjoint for a tile of kRows source rows on each of up to kPlanes source planes
@@ -372,6 +415,13 @@ __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restr
     const int step = 256 / per_row, ty = tid / per_row;
     for (int z = zb; z < zb + planes; ++z) {
         const ResRun<K> zr = zt[z - zb];
+        if (zr.n == 0) {
+            // no LR sample reads the plane (two in three where z is resized by 3): zero over one run of voxels
+            const float none[kV] = {};
+            for (int e = tid; e < rows * groups; e += 256)
+                emit_voxels<kPrep, kV>((int64_t(z) * ny + y0) * nx + int64_t(e) * kV, none, Iv, Wv, eps, dsrc, aip);
+            continue;
+        }
         // LR rows of the tile: runs start in ascending order, so rows jf .. jf + nv - 1 (v_rows bounds them)
         const int jf = min(yt[0].j0, lny - 1);
         const int nv = min(min(yt[rows - 1].j0 + K, lny) - jf, v_rows);
@@ -411,35 +461,106 @@ __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restr
                         if (c < rx[e].n) acc[e] = fmaf(rx[e].w[c], u[rx[e].j0 + c], acc[e]);
                 }
                 const int64_t v = (int64_t(z) * ny + (y0 + r)) * nx + gx * kV;
-                if constexpr (kPrep) {
-                    float w[kV], iv[kV];
-                    float2 a[kV];
-                    if constexpr (kV == 4) {
-                        load4<true>(Wv + v, w);
-                        load4<true>(Iv + v, iv);
-                    } else {
-                        w[0] = Wv[v];
-                        iv[0] = Iv[v];
-                    }
-#pragma unroll
-                    for (int e = 0; e < kV; ++e) a[e] = adj_factor(acc[e], w[e], iv[e], eps);
-                    if constexpr (kV == 4) {
-                        reinterpret_cast<float4*>(aip + v)[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
-                        reinterpret_cast<float4*>(aip + v)[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
-                    } else {
-                        aip[v] = a[0];
-                    }
-                } else if constexpr (kV == 4) {
-                    store4<true>(dsrc + v, acc);
-                } else {
-                    dsrc[v] = acc[0];
-                }
+                emit_voxels<kPrep, kV>(v, acc, Iv, Wv, eps, dsrc, aip);
             }
         }
     }
 }
 
-constexpr int kPlaneSmem = 48 * 1024 - 512;  // (the kernel also holds the z run)
+// The same sums for narrow volumes, of up to kThinRow columns. Their tiles are small, and the latency of the phases and
+// the lanes without a sample count: U is formed from the LR values in memory, without V and its barrier, and
+// the threads run over a tile's samples and voxels without regard to rows. 512 x 300 planes of 20 columns, from as
+// many (from a third of the planes): 37 (37) us by the plane kernel, 27 (17) here; of 48 columns 49 (46) and 52 (27), of
+// 60 45 (25 with the empty planes left out) and 58 (31).
+// Tiles of 128 rows up to 20 columns, else of 32 (one column of 2,048 x 2,048 from 1,024 x 1,024: 186 us with 32, 60 here).
+constexpr int kThinRow = 56;
+constexpr int kThinTile = 128;
+
+template <bool kPrep, int K, int kV>
+__global__ void __launch_bounds__(256) k_resample_adj_thin(const float* __restrict__ ddst, ResGeo G, int tile,
+                                                           int per, FastDiv by_lnx, FastDiv by_groups,
+                                                           const float* __restrict__ Iv,
+                                                           const float* __restrict__ Wv, float eps,
+                                                           float* __restrict__ dsrc, float2* __restrict__ aip) {
+    pdl_enter();
+    const ResAxis &AX = G.a[0], &AY = G.a[1], &AZ = G.a[2];
+    const int nx = AX.n_src, ny = AY.n_src, lnx = AX.n_dst, lny = AY.n_dst;
+    __shared__ ResRun<K> xt[kThinRow], yt[kThinTile], zt[kPlanes];
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    float* U = reinterpret_cast<float*>(res_smem);  // [rows][lnx]
+    const int tid = threadIdx.x;
+    const int y0 = blockIdx.y * tile, rows = min(tile, ny - y0);  // tile <= kThinTile
+    const int zb = blockIdx.x * per, planes = min(per, AZ.n_src - zb);  // per <= kPlanes
+    for (int e = tid; e < nx + rows + planes; e += 256) {
+        ResRun<K> rr;
+        if (e < nx) {
+            res_list<K>(AX, e, rr.j0, rr.n, rr.w);
+            xt[e] = rr;
+        } else if (e < nx + rows) {
+            res_list<K>(AY, y0 + (e - nx), rr.j0, rr.n, rr.w);
+            yt[e - nx] = rr;
+        } else {
+            res_list<K>(AZ, zb + (e - nx - rows), rr.j0, rr.n, rr.w);
+            zt[e - nx - rows] = rr;
+        }
+    }
+    __syncthreads();
+    const int groups = nx / kV;  // kV divides nx
+    for (int z = zb; z < zb + planes; ++z) {
+        const ResRun<K> zr = zt[z - zb];
+        const int64_t v0 = (int64_t(z) * ny + y0) * nx;
+        if (zr.n == 0) {
+            const float none[kV] = {};
+            for (int e = tid; e < rows * groups; e += 256)
+                emit_voxels<kPrep, kV>(v0 + int64_t(e) * kV, none, Iv, Wv, eps, dsrc, aip);
+            continue;
+        }
+        if (z > zb) __syncthreads();  // U is no longer read
+        for (int e = tid; e < rows * lnx; e += 256) {
+            const int r = static_cast<int>(fast_div(static_cast<unsigned>(e), by_lnx)), jx = e - r * lnx;
+            const ResRun<K> ry = yt[r];
+            float acc = 0.0f;
+#pragma unroll
+            for (int b = 0; b < K; ++b) {
+                if (b >= ry.n) break;
+                float v = 0.0f;
+#pragma unroll
+                for (int a = 0; a < K; ++a)
+                    if (a < zr.n) v = fmaf(zr.w[a], ddst[(int64_t(zr.j0 + a) * lny + ry.j0 + b) * lnx + jx], v);
+                acc = fmaf(ry.w[b], v, acc);
+            }
+            U[e] = acc;
+        }
+        __syncthreads();
+        for (int e = tid; e < rows * groups; e += 256) {
+            const int r = static_cast<int>(fast_div(static_cast<unsigned>(e), by_groups)), gx = e - r * groups;
+            const float* u = U + r * lnx;
+            float acc[kV];
+#pragma unroll
+            for (int k = 0; k < kV; ++k) {
+                const ResRun<K> rx = xt[gx * kV + k];
+                acc[k] = 0.0f;
+#pragma unroll
+                for (int c = 0; c < K; ++c)
+                    if (c < rx.n) acc[k] = fmaf(rx.w[c], u[rx.j0 + c], acc[k]);
+            }
+            emit_voxels<kPrep, kV>(v0 + int64_t(e) * kV, acc, Iv, Wv, eps, dsrc, aip);
+        }
+    }
+}
+
+// Shared memory of a tile (the kernel also holds the z run): 32 rows as long as five blocks fit an SM, else 8 rows as long
+// as two do, which takes volumes of up to about 1,000 columns (512 x 512 x 256 from 512 x 512 x 64, 54 KB: 271 us by
+// the run tables, 177 by the plane kernel).
+constexpr int kPlaneSmem = 48 * 1024 - 512;
+constexpr int kPlaneSmemMax = 112 * 1024;
+
+static int planes_per_block(int64_t nz, int64_t tiles) { return nz * tiles >= 152 * 6 ? kPlanes : 1; }
+
+template <bool kPrep>
+static bool vec_volume(const ResGeo& G, const float* I, const float* W, const float* dsrc, const float2* aip) {
+    return G.a[0].n_src % 4 == 0 && (kPrep ? aligned16(I) && aligned16(W) && aligned16(aip) : aligned16(dsrc));
+}
 
 // Rows per tile: the more, the fewer LR values are read again, but the fewer blocks there are and the
 // more shared memory each takes.
@@ -452,19 +573,40 @@ static bool launch_adj_plane_rows(const float* dd, const ResGeo& G, const float*
     const int v_rows = static_cast<int>((kRows - 1) * G.a[1].inv) + 5 + K;
     const size_t smem = sizeof(ResRun<K>) * (size_t(nx) + kRows) + sizeof(float) * lnx * (size_t(kRows) + v_rows);
     const int64_t tiles = (ny + kRows - 1) / kRows;
-    if (smem > size_t(kPlaneSmem) || tiles > 65535) return false;
-    const int per = nz * tiles >= 152 * 6 ? kPlanes : 1;
-    const bool vec = nx % 4 == 0 && (kPrep ? aligned16(I) && aligned16(W) && aligned16(aip) : aligned16(dsrc));
-    launch_k(vec ? k_resample_adj_plane<kPrep, K, kRows, 4> : k_resample_adj_plane<kPrep, K, kRows, 1>,
-        dim3(static_cast<unsigned>((nz + per - 1) / per), static_cast<unsigned>(tiles)), dim3(256), smem, st, dd,
-        G, v_rows, per, I, W, eps, dsrc, aip);
+    if (smem > size_t(kRows > 8 ? kPlaneSmem : kPlaneSmemMax) || tiles > 65535) return false;
+    const int per = planes_per_block(nz, tiles);
+    const auto kernel = vec_volume<kPrep>(G, I, W, dsrc, aip) ? k_resample_adj_plane<kPrep, K, kRows, 4>
+                                                             : k_resample_adj_plane<kPrep, K, kRows, 1>;
+    // (an attribute of the kernel on the current device; beyond 48 KB only)
+    if (smem > size_t(kPlaneSmem) &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+        return false;
+    launch_k(kernel, dim3(static_cast<unsigned>((nz + per - 1) / per), static_cast<unsigned>(tiles)), dim3(256), smem,
+        st, dd, G, v_rows, per, I, W, eps, dsrc, aip);
+    return true;
+}
+
+template <bool kPrep, int K>
+static bool launch_adj_thin(const float* dd, const ResGeo& G, const float* I, const float* W, float eps, float* dsrc,
+                            float2* aip, cudaStream_t st) {
+    const int nx = G.a[0].n_src, ny = G.a[1].n_src, nz = G.a[2].n_src, lnx = G.a[0].n_dst;
+    const int tile = nx <= 20 ? kThinTile : 32;
+    const int64_t tiles = (ny + tile - 1) / tile;
+    if (nx > kThinRow || tiles > 65535) return false;
+    const int per = planes_per_block(nz, tiles);
+    const bool vec = vec_volume<kPrep>(G, I, W, dsrc, aip);
+    launch_k(vec ? k_resample_adj_thin<kPrep, K, 4> : k_resample_adj_thin<kPrep, K, 1>,
+        dim3(static_cast<unsigned>((nz + per - 1) / per), static_cast<unsigned>(tiles)), dim3(256),
+        sizeof(float) * tile * lnx, st, dd, G, tile, per, make_fastdiv(static_cast<unsigned>(lnx)),
+        make_fastdiv(static_cast<unsigned>(vec ? nx / 4 : nx)), I, W, eps, dsrc, aip);
     return true;
 }
 
 template <bool kPrep, int K>
 static bool launch_adj_plane_k(const float* dd, const ResGeo& G, const float* I, const float* W,
                                float eps, float* dsrc, float2* aip, cudaStream_t st) {
-    return launch_adj_plane_rows<kPrep, K, 32>(dd, G, I, W, eps, dsrc, aip, st) ||
+    return launch_adj_thin<kPrep, K>(dd, G, I, W, eps, dsrc, aip, st) ||
+           launch_adj_plane_rows<kPrep, K, 32>(dd, G, I, W, eps, dsrc, aip, st) ||
            launch_adj_plane_rows<kPrep, K, 8>(dd, G, I, W, eps, dsrc, aip, st);
 }
 
