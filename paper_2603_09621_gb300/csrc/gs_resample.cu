@@ -333,36 +333,6 @@ gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t 
     return last_launch_status();
 }
 
-// The adjoint of kV consecutive voxels from v on: as it is, or (kPrep) as the adjoint render's factors.
-template <bool kPrep, int kV>
-__device__ __forceinline__ void emit_voxels(int64_t v, const float (&acc)[kV], const float* __restrict__ Iv,
-                                            const float* __restrict__ Wv, float eps, float* __restrict__ dsrc,
-                                            float2* __restrict__ aip) {
-    if constexpr (kPrep) {
-        float w[kV], iv[kV];
-        float2 a[kV];
-        if constexpr (kV == 4) {
-            load4<true>(Wv + v, w);
-            load4<true>(Iv + v, iv);
-        } else {
-            w[0] = Wv[v];
-            iv[0] = Iv[v];
-        }
-#pragma unroll
-        for (int e = 0; e < kV; ++e) a[e] = adj_factor(acc[e], w[e], iv[e], eps);
-        if constexpr (kV == 4) {
-            reinterpret_cast<float4*>(aip + v)[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
-            reinterpret_cast<float4*>(aip + v)[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
-        } else {
-            aip[v] = a[0];
-        }
-    } else if constexpr (kV == 4) {
-        store4<true>(dsrc + v, acc);
-    } else {
-        dsrc[v] = acc[0];
-    }
-}
-
 // Separable form of the adjoint for a tile of kRows source rows on each of up to kPlanes source planes
 // z, in shared memory: V[j][jx] = sum over the z run of w_z dL/dLR[jz][jy][jx] for the LR rows jy that the tile's
 // rows read (each LR value is loaded once per tile), U[y][jx] = sum over the y run of w_y V, then

@@ -95,6 +95,28 @@ __global__ void __launch_bounds__(256) k_downsample_bwd(const float* __restrict_
     }
 }
 
+// The adjoint render's factors with the profile's adjoint, one HR slice after the other (the LR values are cached).
+template <int kV>
+__global__ void __launch_bounds__(256) k_profile_factors(const float* __restrict__ dlr, unsigned nz, unsigned plane,
+                                                         unsigned nzl, unsigned s, float inv_s,
+                                                         const float* __restrict__ Iv,
+                                                         const float* __restrict__ Wv, float eps,
+                                                         float2* __restrict__ aip) {
+    pdl_enter();
+    for (unsigned z = blockIdx.y * blockDim.y + threadIdx.y; z < nz; z += gridDim.y * blockDim.y) {
+        const unsigned k = z / s;
+        for (unsigned r = (blockIdx.x * blockDim.x + threadIdx.x) * kV; r < plane; r += gridDim.x * blockDim.x * kV) {
+            Voxels<kV> x = {};
+            if (k < nzl) {
+                x = load_voxels<kV>(dlr + int64_t(k) * plane + r);
+#pragma unroll
+                for (int e = 0; e < kV; ++e) x.v[e] *= inv_s;
+            }
+            emit_voxels<true, kV>(int64_t(z) * plane + r, x.v, Iv, Wv, eps, nullptr, aip);
+        }
+    }
+}
+
 // L1 sums: a fixed grid of kL1Blocks blocks of kL1Threads; thread t sums |pred - target| over the
 // quads of consecutive values t, t + 131,072, ..., then a fixed-shape tree over the block (partials)
 // and over the blocks, so the loss does not depend on which kernel forms it or on alignment. The
@@ -216,14 +238,25 @@ __global__ void __launch_bounds__(kL1Threads) k_l1_final(const float* partials, 
 // The fitting step's z box model in one pass: slice profile, L1 and its sign gradient (to lr_pred),
 // profile adjoint and the adjoint render's factors (alpha, alpha I') of the s HR voxels below each
 // LR voxel, with dL/dI = dL/dLR / s (0 in the trailing slices, which no LR slice covers). Bound by
-// HBM: I, W, target read once, dL/dLR and the factors written once. kS: slices per LR slice at
-// compile time (their I values stay in registers), 0: read again from the cache. A thread owns a
+// HBM: I, W, target read once, dL/dLR and the factors written once. kS: slices per LR slice, whose I values stay in
+// registers. A thread owns a
 // quad of LR voxels as in k_l1_partial, so loss and gradient equal the separate entry points' bit for
 // bit; kVec: planes of a multiple of 4 voxels and aligned volumes, by 16-byte accesses.
 // As four kernels (profile, L1, its tree, factors) 16 us at 128^3, s = 2, and 33 us at
 // 256 x 256 x 128, s = 4; here 9 and 27 us (151 MB). All 1,024 blocks of 128 threads are resident at
 // once; with 256 threads and 3 (4) blocks per SM 12 and 32 (28) us; one LR voxel per thread with
 // 4-byte accesses 9 and 48 us.
+// (kS = 0: any number s_, I read again from the cache.) With more than four slices a thread's column is too long a
+// chain where there are few LR voxels or no 16-byte accesses (61 x 45 x 37, s = 16: 22 us; 33 x 33 x 256, s = 8: 14;
+// 255 x 255 x 128, s = 8: 65); the step then takes profile, L1 and factors as three kernels (11, 12 and 39 us). 256 x
+// 256 x 128: s = 5 37 in one, 35 in three; s = 8 30 and 33 (with the columns in registers 35).
+constexpr int kFusedSlices = 4, kFusedSlicesVec = 8;
+constexpr int64_t kFusedVoxels = 1 << 17;
+
+static bool fused_profile(int s, int64_t n_lr, bool vec) {
+    return s <= kFusedSlices || (vec && s >= kFusedSlicesVec && n_lr >= kFusedVoxels);
+}
+
 template <int kS, bool kVec>
 __global__ void __launch_bounds__(kL1Threads, 7) k_profile_loss(
     const float* __restrict__ Iv, const float* __restrict__ Wv, const float* __restrict__ target, unsigned plane,
@@ -339,7 +372,8 @@ static gs_status launch_profile_loss(const float* I, const float* W, const float
         case 2: go(k_profile_loss<2, kVec>); break;
         case 3: go(k_profile_loss<3, kVec>); break;
         case 4: go(k_profile_loss<4, kVec>); break;
-        default: go(k_profile_loss<0, kVec>);
+        default:
+            if constexpr (kVec) go(k_profile_loss<0, true>);  // (fused_profile)
     }
     return last_launch_status();
 }
@@ -377,6 +411,17 @@ gs_status downsample_bwd_impl(const float* dlr, int nz, int ny, int nx, int s, f
     const Grid2d g = grid2d(vec ? plane / 4 : plane, nzl + (nz > nzl * s ? 1 : 0));
     launch_k(vec ? k_downsample_bwd<4> : k_downsample_bwd<1>, g.grid, g.block, 0, st, dlr, nz,
         static_cast<unsigned>(plane), static_cast<unsigned>(nzl), s, 1.0f / float(s), dhr);
+    return last_launch_status();
+}
+
+static gs_status launch_profile_factors(const float* dlr, int nz, int ny, int nx, int s, const float* I, const float* W,
+                                        float eps, float2* aip, cudaStream_t st) {
+    const int64_t plane = int64_t(ny) * nx;
+    const bool vec = vec_ok(I, W, plane) && aligned16(dlr);
+    const Grid2d g = grid2d(vec ? plane / 4 : plane, nz);
+    launch_k(vec ? k_profile_factors<4> : k_profile_factors<1>, g.grid, g.block, 0, st, dlr, static_cast<unsigned>(nz),
+        static_cast<unsigned>(plane), static_cast<unsigned>(nz / s), static_cast<unsigned>(s), 1.0f / float(s), I, W,
+        eps, aip);
     return last_launch_status();
 }
 
@@ -510,11 +555,21 @@ gs_status fit_front(const FitRun& run, int64_t n_norm, int32_t* d_step) {
         s = resample_adj_prep_impl(st->lr_pred, st->lr_nz, st->lr_ny, st->lr_nx, st->I, st->W, g.nz,
                                    g.ny, g.nx, st->cfg.eps, w.aip, cs);
     } else {
+        const int64_t n_lr = int64_t(g.nz / st->s) * g.ny * g.nx;
         const bool vec = vec_ok(st->I, st->W, int64_t(g.ny) * g.nx) && aligned16(st->lr_target) &&
                          aligned16(st->lr_pred);
-        s = (vec ? launch_profile_loss<true> : launch_profile_loss<false>)(
-            st->I, st->W, st->lr_target, g.nz, g.ny, g.nx, st->s, st->cfg.eps, st->lr_pred, st->d_loss, n_norm, w,
-            count, cs);
+        if (fused_profile(st->s, n_lr, vec)) {
+            s = (vec ? launch_profile_loss<true> : launch_profile_loss<false>)(
+                st->I, st->W, st->lr_target, g.nz, g.ny, g.nx, st->s, st->cfg.eps, st->lr_pred, st->d_loss, n_norm,
+                w, count, cs);
+        } else {
+            s = downsample_fwd_impl(st->I, g.nz, g.ny, g.nx, st->s, st->lr_pred, cs);
+            if (s != GS_OK) return s;
+            s = launch_l1(st->lr_pred, st->lr_target, n_lr, st->d_loss, st->lr_pred, w.l1_part, cs, n_norm, w.ticket,
+                          count);
+            if (s != GS_OK) return s;
+            s = launch_profile_factors(st->lr_pred, g.nz, g.ny, g.nx, st->s, st->I, st->W, st->cfg.eps, w.aip, cs);
+        }
     }
     if (s != GS_OK) return s;
     if (!run.mark(3)) return GS_ERR_CUDA;
