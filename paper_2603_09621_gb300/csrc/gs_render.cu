@@ -420,7 +420,7 @@ __device__ __forceinline__ unsigned long long brick_row_mask(const Rec& R, const
     const float ipyy = __fdividef(1.0f, R.pyc1.x);
     const float k1 = -0.5f * (R.pc2.x * ipyy);
     const float nc3 = -(R.pzz - 0.25f * R.pc2.x * (R.pc2.x * ipyy)) * ipyy;
-    const float h0 = G.Tcull * ipyy;
+    const float h0 = fminf(G.Tcull * ipyy, 1e37f);  // (finite: 3e18 voxels, for a Tcull without bound, reach any row)
     const float mu_y = -(R.nmh_yz.x + R.nml_yz.x);
     const float mu_x = -(R.nmhx + R.nmlx);
     const float pad = 1e-3f + 1e-5f * fabsf(mu_y);
@@ -443,9 +443,8 @@ __device__ __forceinline__ unsigned long long brick_row_mask(const Rec& R, const
     for (int rz = 0; rz < bsz; ++rz) {
         const float dz = dz0 + float(rz);
         const float hw2 = fmaf(nc3 * dz, dz, h0);
-        // (bounded away from 0 and infinity, where the product of root and reciprocal root is not a number:
-        // 3e18 voxels, for a Tcull without bound, reach any row)
-        const float hw2b = fminf(fmaxf(hw2, 1e-37f), 1e37f);
+        // (1e-37: at 0 the product of root and reciprocal root is not a number)
+        const float hw2b = fmaxf(hw2, 1e-37f);
         const float ish = rsqrt_approx(hw2b);
         const float sh = hw2b * ish;
         const float xc = fmaf(kx, dz, xrel);
