@@ -4,7 +4,7 @@
 // Pipeline of gs_bin_bricks (all asynchronous on one stream):
 //   k_preprocess    one thread per Gaussian: validity, FP32 brick range (fixed operation order,
 //                   bit-exact against the oracle's binning specification), render record. A block
-//                   also counts its 256 Gaussians' pairs and their first radix digits.
+//                   also counts the pairs of its tile of 64 or 256 Gaussians and their first digits.
 //   k_row_scan      one block per digit: exclusive scan of the digit's counts over the Gaussian
 //                   tiles; one more block scans the tiles' pair counts, stores d_npairs and the
 //                   status word (GS_STATUS_NONFINITE, GS_STATUS_CAPACITY).
@@ -12,9 +12,10 @@
 //                   shared memory and scatters them by digit: the Gaussian-major pair list never
 //                   goes to memory. Tiles of very many pairs are shared out in parts (first_part).
 //   later passes    the same scan and scatter over tiles of 2,048 pairs, whose digit counts the
-//                   scatter before added up or, for large clouds, k_tile_count counts. Stability keeps ascending Gaussian ids inside each
-//                   brick, so the lists are deterministic. The last pass stores pair_brick (key),
-//                   pair_gmj (Gaussian-major position) and pair_gid directly.
+//                   scatter before added up or, for large clouds, k_tile_count counts. Stability
+//                   keeps ascending Gaussian ids inside each brick, so the lists are deterministic.
+//                   The last pass stores pair_brick (key), pair_gmj (Gaussian-major position) and
+//                   pair_gid directly.
 //   k_brick_off     brick_off from the boundaries of the sorted keys.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -293,7 +294,6 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
 #pragma unroll
     for (int j = 0; j < 3; ++j)
         nrm[j] = sqrtf(col[j][0] * col[j][0] + col[j][1] * col[j][1] + col[j][2] * col[j][2]);
-    // n1, n2: m1, m2 with their components along m0 removed
     // n1, n2: m1, m2 with their components along m0 removed; c_j = -(m_j . m0) / a
     float n1[3], n2[3];
     const float d1 = (col[1][0] * col[0][0] + col[1][1] * col[0][1] + col[1][2] * col[0][2]) * inv_a;
@@ -359,8 +359,8 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ params,
     return true;
 }
 
-// Digit counts of `len` pairs of consecutive keys from `key` on (a row of a box): a constant on all digits, added
-// to hall, and 1 on an interval of digits, as differences in hdif.
+// Digit counts of `len` pairs of consecutive keys from `key` on (a row of a box): a constant on all
+// digits, added to hall, and 1 on an interval of digits, as differences in hdif.
 __device__ __forceinline__ void count_row(int key, int len, int nd, int* hdif, int* hall) {
     const int a = key & (nd - 1);
     const int rem = len & (nd - 1), e = a + rem;
@@ -612,29 +612,28 @@ struct Scatter {
     unsigned block0;           // and the grid's first block
 };
 
-// Stable scatter of one tile of up to kRound keys per round. Warp w owns a contiguous part of
-// the tile and visits it in rounds of 32 consecutive keys, kept in registers with their ranks
-// among the warp's earlier equal digits (warp match masks). A block-wide prefix over the digits
-// then gives each digit's run inside the tile and each warp's start in it; the tile is placed in
-// shared memory sorted by digit, ties in tile order, and written out in that order, so consecutive
-// threads store consecutive addresses of a run.
-// kFirst: the tile is emitted by the block itself from its kTile Gaussians' boxes (in rounds
-// of kRound pairs; the digits' output positions advance from round to round; what a tile has beyond first_part
-// pairs is left to blocks for parts, whose rounds start further on: 64 Gaussians on 16,384 bricks, 1.05M pairs in one
-// tile, 6.35 -> 0.16 ms, on 131,072 bricks 51.4 -> 0.8 ms), else it is one
-// tile of the previous pass's output. kLast: the pass stores the bins' per-pair arrays; every
-// other pass of a small cloud adds each key to the next pass's digit counts at its output
-// position's tile (one atomic per group of equal (tile, digit) in a warp).
-// Bound by latency (barriers, the gathered loads) at 40-65 % issue-active, far from bandwidth: the
-// pair list is cache-resident at the fitting size. Whole binning, L2 flushed, at 3.26M pairs
-// (256 x 256 x 128 grid, 8^3 bricks): 115 us with the pair list emitted to memory, two scan launches
-// per list and the owners gathered in the last pass; 88 us now (preprocess 22, first pass 28, last
-// pass 20, count 4, scans 7, offsets 6). 104M pairs (512 x 512 x 256, digits of 9 and 8 bits where 8-bit
-// digits took three passes): 5.86 -> 2.36 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed
-// by a second match per key and the values held in registers (80 registers) 108 us; the
-// values loaded when the tile is placed 0.17 ms longer at 104M than copied to shared memory
-// asynchronously during the ranking (here); 5 (6) blocks per SM with spills 95
-// (97) us.
+// Stable scatter of one tile of up to kRound keys per round. Warp w owns a contiguous part of the tile
+// and visits it in rounds of 32 consecutive keys, kept in registers with their ranks among the warp's
+// earlier equal digits (warp match masks). A block-wide prefix over the digits then gives each digit's
+// run inside the tile and each warp's start in it; the tile is placed in shared memory sorted by digit,
+// ties in tile order, and written out in that order, so consecutive threads store consecutive addresses
+// of a run.
+// kFirst: the tile is emitted by the block itself from its kTile Gaussians' boxes (in rounds of kRound
+// pairs; the digits' output positions advance from round to round; what a tile has beyond first_part
+// pairs is left to blocks for parts, whose rounds start further on: 64 Gaussians on 16,384 bricks, 1.05M
+// pairs in one tile, 6.35 -> 0.17 ms, on 131,072 bricks 51.4 -> 0.7 ms), else it is one tile of the
+// previous pass's output. kLast: the pass stores the bins' per-pair arrays; every other pass of a small
+// cloud adds each key to the next pass's digit counts at its output position's tile (one atomic per group
+// of equal (tile, digit) in a warp).
+// Bound by latency (barriers, the gathered loads) at 40-65 % issue-active, far from bandwidth: the pair
+// list is cache-resident at the fitting size. Whole binning, L2 flushed, at 3.26M pairs (256 x 256 x 128
+// grid, 8^3 bricks): 115 us with the pair list emitted to memory, two scan launches per list and the
+// owners gathered in the last pass; 88 us now (preprocess 22, first pass 28, last pass 20, count 4, scans
+// 7, offsets 6). 104M pairs (512 x 512 x 256, digits of 9 and 8 bits where 8-bit digits took three
+// passes): 5.86 -> 2.36 ms. 21,828 pairs (32^3): 30 -> 17 us. At 3.26M pairs: ranks recomputed by a
+// second match per key and the values held in registers (80 registers) 108 us; the values loaded when the
+// tile is placed 0.17 ms longer at 104M than copied to shared memory asynchronously during the ranking
+// (here); 5 (6) blocks per SM with spills 95 (97) us.
 template <bool kFirst, bool kLast, int kTile>
 __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
     pdl_enter();
@@ -665,8 +664,8 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
         const int64_t part = first_part(P);
         const bool own = static_cast<unsigned>(tile) < A.tiles;
         if (!own) {
-            // the part [p0, p0 + part) of the pair list, as far as it lies behind the first `part` pairs of the tile
-            // that p0 falls in (any later tile's share of it is its own block's)
+            // the part [p0, p0 + part) of the pair list, as far as it lies behind the first `part` pairs
+            // of the tile that p0 falls in (any later tile's share of it is its own block's)
             const int64_t p0 = int64_t(tile - A.tiles) * part;
             if (A.blk_base[A.tiles + 1] <= part || p0 >= P) return;
             int hi = static_cast<int>(A.tiles) - 1;
@@ -723,8 +722,8 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(Scatter A) {
         if (own) {
             end = static_cast<int>(min(int64_t(tot), part));
         } else {
-            // digit counts of the tile's pairs before `begin`: its boxes staged in skey (first pair, size along x
-            // and y, first key), their rows shared by all warps
+            // digit counts of the tile's pairs before `begin`: its boxes staged in skey (first pair, size
+            // along x and y, first key), their rows shared by all warps
             static_assert(kMaxRound >= 4 * kTile, "a tile's boxes fit the key buffer");
             int4* sbox = reinterpret_cast<int4*>(skey);
             int* hdif = wcnt;
@@ -1086,10 +1085,11 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
     gs_status s = last_launch_status();
     if (s != GS_OK) return s;
     const unsigned tiles = static_cast<unsigned>((cap + kSortTile - 1) / kSortTile);
-    // Blocks for the parts of heavy tiles (no tile is heavy where its Gaussians on all bricks, or the capacity, are no
-    // more than a part). They follow the tiles' blocks, or, where the tiles are more than two per SM but fewer than
-    // the resident blocks and may take several rounds, in a launch of their own: more blocks than tiles there put a
-    // fourth tile on a few SMs (391 tiles of three rounds 101 -> 110 us; the launch costs 2 us).
+    // Blocks for the parts of heavy tiles (no tile is heavy where its Gaussians on all bricks, or the
+    // capacity, are no more than a part). They follow the tiles' blocks, or, where the tiles are more
+    // than two per SM but fewer than the resident blocks and may take several rounds, in a launch of
+    // their own: more blocks than tiles there put a fourth tile on a few SMs (391 tiles of three rounds
+    // 101 -> 110 us; the launch costs 2 us).
     const int64_t max_tile = int64_t(gt) * bins->n_bricks < cap ? int64_t(gt) * bins->n_bricks : cap;
     const int64_t max_parts = max_tile > kFirstMinPart ? (cap + kFirstMinPart - 1) / kFirstMinPart : 0;
     const unsigned parts = static_cast<unsigned>(max_parts < kFirstParts ? max_parts : kFirstParts);
@@ -1172,7 +1172,7 @@ gs_status bin_bricks_impl(const float* params, const gs_grid* grid, const gs_con
         return cudaMemsetAsync(bins->brick_off, 0, off_bytes, st) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
     // enough threads for four keys each, at most eight blocks per SM
     const int64_t ob = (cap / 4 + 256) / 256;
-    launch_k(k_brick_off, dim3(static_cast<unsigned>(ob < 152 * 8 ? ob : 152 * 8)), dim3(256), 0, st,
+    launch_k(k_brick_off, dim3(static_cast<unsigned>(ob < kSms * 8 ? ob : kSms * 8)), dim3(256), 0, st,
         bins->pair_brick, bins->d_npairs, cap, bins->n_bricks, bins->brick_off);
     return last_launch_status();
 }

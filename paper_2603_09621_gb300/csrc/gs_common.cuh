@@ -68,25 +68,30 @@ constexpr float kHalfLog2e = 0.7213475204444817f;  // (1/2) log2(e)
 // Brick-range brange layout [N, 8].
 enum BrangeField : int { B_LOX = 0, B_LOY, B_LOZ, B_HIX, B_HIY, B_HIZ, B_CNT, B_VALID };
 
+// Streaming multiprocessors of the GPU that the grids and the sizes of the dispatch rules are made for.
+constexpr int kSms = 152;
+
 // ------------------------------------------------------------------ sort constants
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per tile
-// First-pass tiles of more than kSortTile pairs take rounds of 2,304: a round costs 7 us or more whether full or
-// nearly empty, and tiles of 256 Gaussians with 8.2-8.5 pairs each needed a second one (833,333 Gaussians, 6.83M
-// pairs, whole binning 182 -> 171 us; 100,000 with 7.1 pairs 36.7 -> 35.5; 4M with 26 2.40 -> 2.36 ms). Used for all
-// tiles, 0.2 % of a step at 5.6-6.5 pairs, which fill one round either way. 10 and more items spill at 64
-// registers; with the keys read again from shared memory instead, 10 (12) take 171 (171) us and 2.34 (2.28) ms, but
-// 69.3 (69.4) us against 67.5 at 375,000 with 5.6 pairs and 89.9 (89.3) against 88.8 at 500,000.
+// First-pass tiles of more than kSortTile pairs take rounds of 2,304: a round costs 7 us or more whether
+// full or nearly empty, and tiles of 256 Gaussians with 8.2-8.5 pairs each needed a second one (833,333
+// Gaussians, 6.83M pairs, whole binning 182 -> 171 us; 100,000 with 7.1 pairs 36.7 -> 35.5; 4M with 26
+// 2.40 -> 2.36 ms). Used for all tiles, 0.2 % of a step at 5.6-6.5 pairs, which fill one round either
+// way. 10 and more items spill at 64 registers; with the keys read again from shared memory instead, 10
+// (12) take 171 (171) us and 2.34 (2.28) ms, but 69.3 (69.4) us against 67.5 at 375,000 with 5.6 pairs
+// and 89.9 (89.3) against 88.8 at 500,000.
 constexpr int kFirstItems = 9;
-// A tile's own block places at most first_part(P) of its pairs; what is left of a heavier tile is taken in parts
-// of that size by further blocks, each of which first counts the digits of the tile's pairs before its part (by
-// rows of the boxes). So a block's serial work follows the pairs in all, not the widest Gaussians: four
-// rounds at least, and no less than twice an even share of the pairs among the resident blocks, so that clouds whose
-// tiles are all alike are not cut up (with one share 12.3M pairs in 391 tiles 490 -> 525 us).
+// A tile's own block places at most first_part(P) of its pairs; what is left of a heavier tile is taken
+// in parts of that size by further blocks, each of which first counts the digits of the tile's pairs
+// before its part (by rows of the boxes). So a block's serial work follows the pairs in all, not the
+// widest Gaussians: four rounds at least, and no less than twice an even share of the pairs among the
+// resident blocks, so that clouds whose tiles are all alike are not cut up (with one share 12.3M pairs in
+// 391 tiles 490 -> 525 us).
 constexpr int kFirstRound = kSortThreads * kFirstItems;
 constexpr int kFirstMinPart = 4 * kFirstRound;
-constexpr int kScatterWave = 152 * 4;  // resident scatter blocks
+constexpr int kScatterWave = kSms * 4;  // resident scatter blocks
 constexpr int kFirstParts = kScatterWave / 2;
 __host__ __device__ inline int64_t first_part(int64_t pairs) {
     const int64_t share = (pairs / kFirstParts / kFirstRound + 1) * kFirstRound;  // > pairs / kFirstParts
@@ -98,7 +103,7 @@ constexpr int kMaxDigits = 1 << kMaxRadixBits;
 // block of 256 per SM is spread over more SMs in tiles of 64: 6,000 clustered Gaussians, 119,000 pairs,
 // one radix pass 18.2 -> 7.8 us, preprocess 6.9 -> 6.3; 30,000 lattice Gaussians 8.1 -> 6.5 us; the
 // largest such cloud gains least.
-constexpr int64_t kSmallCloud = 152 * 256;
+constexpr int64_t kSmallCloud = kSms * 256;
 inline int gauss_tile(int64_t n_gauss) { return n_gauss <= kSmallCloud ? 64 : 256; }
 
 constexpr int kL1Blocks = 1024;  // fixed block count of the L1 reduction (deterministic)
@@ -147,12 +152,14 @@ inline int pass_bits(int key_bits, int passes, int pass) {
     return narrow + (is_wide ? 1 : 0);
 }
 
-// Who counts a later pass's digits: from this many Gaussians on a kernel of its own, over the output of the
-// pass before; below, the scatter before itself, with an atomic per group of equal (tile, digit) in a warp.
-// The launch costs 2 us; the atomics nothing where neighbours in the list are neighbours in space (lattice clouds,
-// whose groups are large: 131,072 Gaussians, 0.71M pairs 36.4 us with them, 39.1 without; 500,000: 88.6, 89.0; 1M:
-// 130.4, 130.5) and 4 us per million pairs where they are not (1M random Gaussians, 6.83M pairs 184.3 us with
-// them, 182.1 without; 4M clustered ones, 104M pairs 2.81 ms and 2.40 ms).
+// Who counts a later pass's digits: from this many Gaussians on a kernel of its own, over the output of
+// the pass before; below, the scatter before itself, with an atomic per group of equal (tile, digit) in a
+// warp.
+// The launch costs 2 us; the atomics nothing where neighbours in the list are neighbours in space
+// (lattice clouds, whose groups are large: 131,072 Gaussians, 0.71M pairs 36.4 us with them, 39.1
+// without; 500,000: 88.6, 89.0; 1M: 130.4, 130.5) and 4 us per million pairs where they are not (1M
+// random Gaussians, 6.83M pairs 184.3 us with them, 182.1 without; 4M clustered ones, 104M pairs 2.81 ms
+// and 2.40 ms).
 constexpr int64_t kCountCloud = 400000;
 
 inline bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }

@@ -223,18 +223,19 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ params, const 
     }
 }
 
-// Fitting step tail, one thread per Gaussian: sum the per-brick partials in Gaussian-major
-// order (deterministic mode) or take the atomically accumulated gradient, chain it to the
-// raw parameters (written to grad), and (kAdam) apply Adam to params, m, v; d_step already counts
-// this step. A step whose binning overflowed rendered nothing: it leaves parameters and moments as
-// they are and zeroes grad (the caller grows the bins and repeats the step).
-// Blocks of 64 threads, a Gaussian's partials loaded three or (kFour) four at a time, always added in the same
-// order. Bound by HBM and the latency of the scattered partials: 500,000 Gaussians, 3.26M pairs (about 320 MB)
-// 66 us in blocks of 256, 61.6 us here; 833,000 97 -> 89 us. With Adam four loads without spills (72 registers, 14
-// blocks per SM) beat three with (64, 16 blocks): 61.6 against 63 us, 89 against 91.5, 100,000 Gaussians 15.0
-// against 16.2; five or six loads 66 and 70 us. The gradient alone is shorter with three (188,000 Gaussians, 1.5M
-// pairs 21.9 against 24.3 us) but for clouds of at most kSmallCloud Gaussians, whose time is the latency of the
-// longest list: 6,000 with 19 pairs each 17 -> 13 us.
+// Fitting step tail, one thread per Gaussian: sum the per-brick partials in Gaussian-major order
+// (deterministic mode) or take the atomically accumulated gradient, chain it to the raw parameters
+// (written to grad), and (kAdam) apply Adam to params, m, v; d_step already counts this step. A step
+// whose binning overflowed rendered nothing: it leaves parameters and moments as they are and zeroes grad
+// (the caller grows the bins and repeats the step).
+// Blocks of 64 threads, a Gaussian's partials loaded three or (kFour) four at a time, always added in the
+// same order. Bound by HBM and the latency of the scattered partials: 500,000 Gaussians, 3.26M pairs
+// (about 320 MB) 66 us in blocks of 256, 61.6 us here; 833,000 97 -> 89 us. With Adam four loads without
+// spills (72 registers, 14 blocks per SM) beat three with (64, 16 blocks): 61.6 against 63 us, 89 against
+// 91.5, 100,000 Gaussians 15.0 against 16.2; five or six loads 66 and 70 us. The gradient alone is
+// shorter with three (188,000 Gaussians, 1.5M pairs 21.9 against 24.3 us) but for clouds of at most
+// kSmallCloud Gaussians, whose time is the latency of the longest list: 6,000 with 19 pairs each 17 -> 13
+// us.
 constexpr int kChainThreads = 64;
 
 template <bool kDet, bool kAdam, bool kFour>
@@ -429,7 +430,7 @@ gs_status launch_adam(float* params, const float* grad, float* m, float* v, int6
         const AdamLr a = make_adam_lr(hp);
         const int64_t n4 = n_gauss * 3;
         const int64_t blocks64 = (n4 + 255) / 256;
-        const unsigned blocks = static_cast<unsigned>(blocks64 < 152 * 32 ? blocks64 : 152 * 32);
+        const unsigned blocks = static_cast<unsigned>(blocks64 < kSms * 32 ? blocks64 : kSms * 32);
         const bool vec = aligned16(params) && aligned16(grad) && aligned16(m) && aligned16(v);
         launch_k(vec ? k_adam<true> : k_adam<false>, dim3(blocks), dim3(256), 0, st, params, grad, m, v, n4,
             a, d_step, d_skip);

@@ -1,41 +1,39 @@
-// gs_render.cu -- Eq. 3-4 forward render and its Eq. 5-6 adjoint, one CTA per brick
-// (Sec. 3.3: "each handled by one CUDA thread block"; the brick's Gaussians are staged into
-// shared memory and no depth order is needed).
+// gs_render.cu -- Eq. 3-4 forward render and its Eq. 5-6 adjoint, one CTA per brick (Sec. 3.3: "each
+// handled by one CUDA thread block"; the brick's Gaussians are staged into shared memory and no depth
+// order is needed).
 //
-// Exponent of a pair (voxel p, Gaussian i) in voxel units: q = S(dy, dz) + (sa (dx - dx*))^2
-// (record layout in gs_common.cuh), the Gaussian kernel is 2^-q and the pair contributes
-// only where q <= T = (log2 e / 2) trunc_sigma^2. q is computed by the same operation sequence
-// in both kernels from the voxel's global index and the Gaussian alone, so forward and
-// adjoint agree on every inclusion decision and no result depends on the brick shape.
+// Exponent of a pair (voxel p, Gaussian i) in voxel units: q = S(dy, dz) + (sa (dx - dx*))^2 (record
+// layout in gs_common.cuh), the Gaussian kernel is 2^-q and the pair contributes only where q <= T =
+// (log2 e / 2) trunc_sigma^2. q is computed by the same operation sequence in both kernels from the
+// voxel's global index and the Gaussian alone, so forward and adjoint agree on every inclusion decision
+// and no result depends on the brick shape.
 //
-// Forward: the brick is split into 4 x 4 x 4 footprints, a quarter-warp each (a half or a whole warp in bricks of
-// two or one); a lane owns the two x-rows of four (two, one) voxels at z and z + 1. The block stages the brick's list in rounds of 20 records
-// per footprint (160 for an 8^3 brick); smaller bricks, with shorter lists, take shorter rounds
-// (64 records for one or two footprints) and keep more blocks resident. The thread that stages a record tests it against every footprint
-// (three conservative tests, see foot_mask: the triangle inequality in whitened space
-// |M (p - mu)| >= |M (c - mu)| - rho4, with rho4 the whitened radius of the footprint around its
-// centre c; the truncated ellipsoid's bounding box widened by 3/2 along each axis; and q's lower
-// bound from the smallest eigenvalue at the footprint's nearest point; a margin absorbs FP32
-// rounding). Each warp lists the hits of its footprints and evaluates them in ascending Gaussian
-// id, accumulating S and W in registers (deterministic; one packed FFMA2 updates a voxel's (S, W)
-// with (v r, r) g).
-// Adjoint: one thread per (brick, Gaussian) pair evaluates the brick rows the Gaussian
-// reaches (the row shadow, per z-row a quadratic in dy; z-planes whose section of the
-// ellipsoid misses the brick's x range are skipped), each row as bx predicated voxel slots in
-// packed FP32x2 pairs, so lanes never diverge inside a row. A block takes 256 consecutive
-// brick-major pairs (one to three bricks), computes their row masks and counting-sorts them
-// by number of rows in shared memory; its four warps then take 32-pair chunks of the sorted
-// list, longest first, from a shared counter, so the lanes of a warp run pairs of equal length
-// and a warp that drew short pairs moves on to the next chunk (64 registers without spills,
-// 8 blocks per SM, 7 for 16-voxel-wide bricks; the y and z cross moments are summed over both
-// FP32x2 elements per row to keep the accumulators that small). The per-voxel factors (alpha, alpha I'), alpha = dL/dI / max(W, eps), are
-// precomputed into one float2 volume; a block copies those of its first four bricks into
-// shared memory (zero outside the grid), so rows read them without range tests; a 16-byte pad
-// after every 128 bytes and a 32-byte offset between staged bricks spread the rows that the
-// lanes of a warp read at once over the shared-memory banks. Each pair's partial is summed by
-// one thread in a fixed voxel order (the processing order does not change results) and goes
-// to a per-pair slot (deterministic mode, reduced later in Gaussian-major order) or to three
-// vector atomics of four floats (fast mode).
+// Forward: the brick is split into 4 x 4 x 4 footprints, a quarter-warp each (a half or a whole warp in
+// bricks of two or one); a lane owns the two x-rows of four (two, one) voxels at z and z + 1. The block
+// stages the brick's list in rounds of 20 records per footprint (160 for an 8^3 brick); smaller bricks,
+// with shorter lists, take shorter rounds (64 records for one or two footprints) and keep more blocks
+// resident. The thread that stages a record tests it against every footprint (three conservative tests,
+// see foot_mask: the triangle inequality in whitened space |M (p - mu)| >= |M (c - mu)| - rho4, with rho4
+// the whitened radius of the footprint around its centre c; the truncated ellipsoid's bounding box
+// widened by 3/2 along each axis; and q's lower bound from the smallest eigenvalue at the footprint's
+// nearest point; a margin absorbs FP32 rounding). Each warp lists the hits of its footprints and
+// evaluates them in ascending Gaussian id, accumulating S and W in registers (deterministic; one packed
+// FFMA2 updates a voxel's (S, W) with (v r, r) g).
+// Adjoint: one thread per (brick, Gaussian) pair evaluates the brick rows the Gaussian reaches (the row
+// shadow, per z-row a quadratic in dy; z-planes whose section of the ellipsoid misses the brick's x range
+// are skipped), each row as bx predicated voxel slots in packed FP32x2 pairs, so lanes never diverge
+// inside a row. A block takes 256 consecutive brick-major pairs (one to three bricks), computes their row
+// masks and counting-sorts them by number of rows in shared memory; its four warps then take 32-pair
+// chunks of the sorted list, longest first, from a shared counter, so the lanes of a warp run pairs of
+// equal length and a warp that drew short pairs moves on to the next chunk (64 registers without spills,
+// 8 blocks per SM, 7 for 16-voxel-wide bricks; the y and z cross moments are summed over both FP32x2
+// elements per row to keep the accumulators that small). The per-voxel factors (alpha, alpha I'), alpha =
+// dL/dI / max(W, eps), are precomputed into one float2 volume; a block copies those of its first four
+// bricks into shared memory (zero outside the grid), so rows read them without range tests; a 16-byte pad
+// after every 128 bytes and a 32-byte offset between staged bricks spread the rows that the lanes of a
+// warp read at once over the shared-memory banks. Each pair's partial is summed by one thread in a fixed
+// voxel order (the processing order does not change results) and goes to a per-pair slot (deterministic
+// mode, reduced later in Gaussian-major order) or to three vector atomics of four floats (fast mode).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -180,41 +178,41 @@ __device__ __forceinline__ unsigned foot_mask(const Rec& R, const RenderGeo& G, 
 
 // ------------------------------------------------------------------------ forward
 
-// One block of 32 or 64 threads per brick (more with kFew, below). What bounds it is instruction issue (72 % active) and
-// the latency of the gathered records, so work per instruction decides:
-//   - A quarter-warp per 4^3 footprint, a lane owning the x-rows at z and z + 1: the row terms,
-//     offsets and exponents of the two rows run as FP32x2 pairs (element by element the scalar
-//     operations, so results are bit-identical to one row per lane). Against a half-warp per
-//     footprint and one row per lane: 277 -> 241 us (256 x 256 x 128 grid, 500k Gaussians of a fit
-//     in progress, 132M effective pairs, L2 flushed), 6.97 -> 6.13 ms (512 x 512 x 256 grid, 4M
-//     clustered Gaussians).
-//   - The thread that stages a record also culls it against all the brick's footprints from
-//     registers (row terms shared along x). With one lane per (record, footprint) reading the
-//     staged copy, the cull's shared-memory loads were half of all its wavefronts, and staging
-//     and culling took 110 us of the 241. Each warp then lists its footprints' hits of the whole
-//     round, so quarters of unequal hit counts wait for one another once per round instead of
-//     once per 32 records: 241 -> 215 us, 6.13 -> 5.28 ms.
-//   - Four hits per iteration (the lists are padded with a null record): 215 -> 212 us,
-//     5.28 -> 5.17 ms, and 35 -> 27 us where few bricks leave one warp per scheduler (32^3 grid,
-//     4,096 Gaussians). Two hits 217 us, eight 215 us.
-//   - 72 registers, 14 blocks per SM, 20 records per round and footprint: 209 us and 5.23 ms. 16
-//     records 212 us and 5.20 ms; 24 records 207 us but 5.50 ms; 64 registers (spills) 216 us;
-//     96 registers 217 us. Rounds double-buffered with cp.async measured slower (242 against
-//     241 us, 7.06 against 6.13 ms).
-// kLanes: lanes per footprint, 8 as above; 16 in bricks of two footprints and 32 in bricks of one, which would leave half or
-// three quarters of the only warp idle. Rounds of 64 records there fill the staging passes of 32. Random clouds
-// on 128^3, against a quarter-warp and rounds of 40: 8 x 4 x 4 bricks 193 -> 142 us, 4^3 314 -> 202 (a half-warp per
-// footprint throughout took 146 and 221; rounds of 32 or 96: 148 and 205, 151 and 209).
-// A grid of few bricks leaves most schedulers with one warp or none, and a brick's time is the latency
-// of its lists. There (kFew) a footprint gets a whole warp, each lane the two voxels at z and z + 1,
-// and a thread fetches its record of the next round while the present one is evaluated. Forward us,
-// narrow -> whole warps: 8 bricks of 8^3 25 -> 21, 64 bricks 33-38 -> 26-28 (random and clustered clouds), 216
-// bricks 35-46 -> 34-36, but 512 bricks 41-53 -> 51-56 and 4,096 bricks 146 -> 270: a lane with one
-// voxel per row repeats the row terms four times as often. 8 x 8 x 4 bricks: 128 of them 36-42 ->
-// 24-26, 1,024 43-64 -> 48-54. So where all footprints' warps are resident at once (152 SMs of 2
-// blocks of 8 warps: 304 bricks of 8^3, 608 of 8 x 8 x 4; bricks of one footprint have two warps, for staging). Eight
-// hits per iteration 1-2 us slower.
-constexpr int64_t kFewFootprints = 152 * 16;
+// One block of 32 or 64 threads per brick (more with kFew, below). What bounds it is instruction issue
+// (72 % active) and the latency of the gathered records, so work per instruction decides:
+//   - A quarter-warp per 4^3 footprint, a lane owning the x-rows at z and z + 1: the row terms, offsets
+//     and exponents of the two rows run as FP32x2 pairs (element by element the scalar operations, so
+//     results are bit-identical to one row per lane). Against a half-warp per footprint and one row per
+//     lane: 277 -> 241 us (256 x 256 x 128 grid, 500k Gaussians of a fit in progress, 132M effective
+//     pairs, L2 flushed), 6.97 -> 6.13 ms (512 x 512 x 256 grid, 4M clustered Gaussians).
+//   - The thread that stages a record also culls it against all the brick's footprints from registers
+//     (row terms shared along x). With one lane per (record, footprint) reading the staged copy, the
+//     cull's shared-memory loads were half of all its wavefronts, and staging and culling took 110 us of
+//     the 241. Each warp then lists its footprints' hits of the whole round, so quarters of unequal hit
+//     counts wait for one another once per round instead of once per 32 records: 241 -> 215 us, 6.13 ->
+//     5.28 ms.
+//   - Four hits per iteration (the lists are padded with a null record): 215 -> 212 us, 5.28 -> 5.17 ms,
+//     and 35 -> 27 us where few bricks leave one warp per scheduler (32^3 grid, 4,096 Gaussians). Two
+//     hits 217 us, eight 215 us.
+//   - 72 registers, 14 blocks per SM, 20 records per round and footprint: 209 us and 5.23 ms. 16 records
+//     212 us and 5.20 ms; 24 records 207 us but 5.50 ms; 64 registers (spills) 216 us; 96 registers 217
+//     us. Rounds double-buffered with cp.async measured slower (242 against 241 us, 7.06 against 6.13
+//     ms).
+// kLanes: lanes per footprint, 8 as above; 16 in bricks of two footprints and 32 in bricks of one, which
+// would leave half or three quarters of the only warp idle. Rounds of 64 records there fill the staging
+// passes of 32. Random clouds on 128^3, against a quarter-warp and rounds of 40: 8 x 4 x 4 bricks 193 ->
+// 142 us, 4^3 314 -> 202 (a half-warp per footprint throughout took 146 and 221; rounds of 32 or 96: 148
+// and 205, 151 and 209).
+// A grid of few bricks leaves most schedulers with one warp or none, and a brick's time is the latency of
+// its lists. There (kFew) a footprint gets a whole warp, each lane the two voxels at z and z + 1, and a
+// thread fetches its record of the next round while the present one is evaluated. Forward us, narrow ->
+// whole warps: 8 bricks of 8^3 25 -> 21, 64 bricks 33-38 -> 26-28 (random and clustered clouds), 216
+// bricks 35-46 -> 34-36, but 512 bricks 41-53 -> 51-56 and 4,096 bricks 146 -> 270: a lane with one voxel
+// per row repeats the row terms four times as often. 8 x 8 x 4 bricks: 128 of them 36-42 -> 24-26, 1,024
+// 43-64 -> 48-54. So where all footprints' warps are resident at once (152 SMs of 2 blocks of 8 warps:
+// 304 bricks of 8^3, 608 of 8 x 8 x 4; bricks of one footprint have two warps, for staging). Eight hits
+// per iteration 1-2 us slower.
+constexpr int64_t kFewFootprints = kSms * 16;
 constexpr int kFwdHits = 4;  // hits per iteration of the evaluation loop (one 32-bit list word)
 
 template <bool kStats, int kChunk, int kLanes, bool kFew>

@@ -309,7 +309,7 @@ static ResGeo make_res(int32_t snz, int32_t sny, int32_t snx, int32_t dnz, int32
 
 static unsigned res_blocks(int64_t n) {
     const int64_t b = (n + 255) / 256;
-    return static_cast<unsigned>(b < 152 * 64 ? b : 152 * 64);
+    return static_cast<unsigned>(b < kSms * 64 ? b : kSms * 64);
 }
 
 gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t snx, float* dst,
@@ -317,8 +317,8 @@ gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t 
     const ResGeo G = make_res(snz, sny, snx, dnz, dny, dnx);
     const bool narrow = int64_t(snz) * sny * snx <= (int64_t(1) << 31) - 1;
     const bool rows4 = int64_t(dnz) * dny * dnx >= kFwdRowsMin;
-    // a block's threads over columns (whole warps, or a power of two of a narrow volume's), then rows, then planes:
-    // with whole warps along any row 1,024 x 1,024 samples of one column took 146 us, 15 now
+    // a block's threads over columns (whole warps, or a power of two of a narrow volume's), then rows,
+    // then planes: with whole warps along any row 1,024 x 1,024 samples of one column took 146 us, 15 now
     const int tx = row_threads(dnx), rows = rows4 ? 4 : 1;
     int ty = 1, tz = 1;
     while (2 * ty * tx <= 256 && ty * rows < dny) ty *= 2;
@@ -333,17 +333,17 @@ gs_status resample_fwd_impl(const float* src, int32_t snz, int32_t sny, int32_t 
     return last_launch_status();
 }
 
-// Separable form of the adjoint for a tile of kRows source rows on each of up to kPlanes source planes
-// z, in shared memory: V[j][jx] = sum over the z run of w_z dL/dLR[jz][jy][jx] for the LR rows jy that the tile's
-// rows read (each LR value is loaded once per tile), U[y][jx] = sum over the y run of w_y V, then
-// each voxel sums its x run over U[y]. Fixed order: z, then y, then x. A thread owns kV consecutive x
-// of every (256 / threads per row)-th row: its x runs stay in registers, and with kV = 4 (rows of
-// whole, aligned quads) I, W and the factors move by 16-byte accesses. Bound by HBM where it forms
-// the adjoint render's factors (143 MB at 240 x 240 x 155 from 100^3: 21 us at the copy bandwidth).
-// With z and y taps gathered per (y, jx) from global memory, one voxel per thread, an index
-// division per voxel and 1,240 blocks for 1,216 resident ones it took 62 us (26 us without the
-// factors); 36 (16) us now. Tiles of 16 (24, 48) rows took 41 (43, 44) us; one plane per block,
-// which forms the x runs twice as often, 38 us; kept where two would leave SMs idle.
+// Separable form of the adjoint for a tile of kRows source rows on each of up to kPlanes source planes z,
+// in shared memory: V[j][jx] = sum over the z run of w_z dL/dLR[jz][jy][jx] for the LR rows jy that the
+// tile's rows read (each LR value is loaded once per tile), U[y][jx] = sum over the y run of w_y V, then
+// each voxel sums its x run over U[y]. Fixed order: z, then y, then x. A thread owns kV consecutive x of
+// every (256 / threads per row)-th row: its x runs stay in registers, and with kV = 4 (rows of whole,
+// aligned quads) I, W and the factors move by 16-byte accesses. Bound by HBM where it forms the adjoint
+// render's factors (143 MB at 240 x 240 x 155 from 100^3: 21 us at the copy bandwidth).
+// With z and y taps gathered per (y, jx) from global memory, one voxel per thread, an index division per
+// voxel and 1,240 blocks for 1,216 resident ones it took 62 us (26 us without the factors); 36 (16) us
+// now. Tiles of 16 (24, 48) rows took 41 (43, 44) us; one plane per block, which forms the x runs twice
+// as often, 38 us; kept where two would leave SMs idle.
 constexpr int kPlanes = 2;
 
 template <bool kPrep, int K, int kRows, int kV>
@@ -386,7 +386,8 @@ __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restr
     for (int z = zb; z < zb + planes; ++z) {
         const ResRun<K> zr = zt[z - zb];
         if (zr.n == 0) {
-            // no LR sample reads the plane (two in three where z is resized by 3): zero over one run of voxels
+            // no LR sample reads the plane (two in three where z is resized by 3): zero over one run of
+            // voxels
             const float none[kV] = {};
             for (int e = tid; e < rows * groups; e += 256)
                 emit_voxels<kPrep, kV>((int64_t(z) * ny + y0) * nx + int64_t(e) * kV, none, Iv, Wv, eps, dsrc, aip);
@@ -437,12 +438,13 @@ __global__ void __launch_bounds__(256) k_resample_adj_plane(const float* __restr
     }
 }
 
-// The same sums for narrow volumes, of up to kThinRow columns. Their tiles are small, and the latency of the phases and
-// the lanes without a sample count: U is formed from the LR values in memory, without V and its barrier, and
-// the threads run over a tile's samples and voxels without regard to rows. 512 x 300 planes of 20 columns, from as
-// many (from a third of the planes): 37 (37) us by the plane kernel, 27 (17) here; of 48 columns 49 (46) and 52 (27), of
-// 60 45 (25 with the empty planes left out) and 58 (31).
-// Tiles of 128 rows up to 20 columns, else of 32 (one column of 2,048 x 2,048 from 1,024 x 1,024: 186 us with 32, 60 here).
+// The same sums for narrow volumes, of up to kThinRow columns. Their tiles are small, and the latency of
+// the phases and the lanes without a sample count: U is formed from the LR values in memory, without V
+// and its barrier, and the threads run over a tile's samples and voxels without regard to rows. 512 x 300
+// planes of 20 columns, from as many (from a third of the planes): 37 (37) us by the plane kernel, 27
+// (17) here; of 48 columns 49 (46) and 52 (27), of 60 45 (25 with the empty planes left out) and 58 (31).
+// Tiles of 128 rows up to 20 columns, else of 32 (one column of 2,048 x 2,048 from 1,024 x 1,024: 186 us
+// with 32, 60 here).
 constexpr int kThinRow = 56;
 constexpr int kThinTile = 128;
 
@@ -519,13 +521,13 @@ __global__ void __launch_bounds__(256) k_resample_adj_thin(const float* __restri
     }
 }
 
-// Shared memory of a tile (the kernel also holds the z run): 32 rows as long as five blocks fit an SM, else 8 rows as long
-// as two do, which takes volumes of up to about 1,000 columns (512 x 512 x 256 from 512 x 512 x 64, 54 KB: 271 us by
-// the run tables, 177 by the plane kernel).
+// Shared memory of a tile (the kernel also holds the z run): 32 rows as long as five blocks fit an SM,
+// else 8 rows as long as two do, which takes volumes of up to about 1,000 columns (512 x 512 x 256 from
+// 512 x 512 x 64, 54 KB: 271 us by the run tables, 177 by the plane kernel).
 constexpr int kPlaneSmem = 48 * 1024 - 512;
 constexpr int kPlaneSmemMax = 112 * 1024;
 
-static int planes_per_block(int64_t nz, int64_t tiles) { return nz * tiles >= 152 * 6 ? kPlanes : 1; }
+static int planes_per_block(int64_t nz, int64_t tiles) { return nz * tiles >= kSms * 6 ? kPlanes : 1; }
 
 template <bool kPrep>
 static bool vec_volume(const ResGeo& G, const float* I, const float* W, const float* dsrc, const float2* aip) {
@@ -594,7 +596,7 @@ static bool launch_adj_tab(const float* dd, const ResGeo& G, const float* I, con
     const int n_tab = G.a[0].n_src + G.a[1].n_src + G.a[2].n_src;
     if (!res_list_ok(G) || n_tab > kResTabMax) return false;
     const int64_t rows = int64_t(G.a[2].n_src) * G.a[1].n_src;
-    const unsigned nb = static_cast<unsigned>(rows < 152 * 8 ? rows : 152 * 8);
+    const unsigned nb = static_cast<unsigned>(rows < kSms * 8 ? rows : kSms * 8);
     if (res_two_taps(G))
         launch_k(k_resample_adj_tab<kPrep, 2>, dim3(nb), dim3(256), sizeof(ResRun<2>) * n_tab, st,
             dd, G, I, W, eps, dsrc, aip);

@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(256) k_downsample_bwd(const float* __restrict_
     }
 }
 
-// The adjoint render's factors with the profile's adjoint, one HR slice after the other (the LR values are cached).
+// The adjoint render's factors with the profile's adjoint, one HR slice after the other (the LR values
+// are cached).
 template <int kV>
 __global__ void __launch_bounds__(256) k_profile_factors(const float* __restrict__ dlr, unsigned nz, unsigned plane,
                                                          unsigned nzl, unsigned s, float inv_s,
@@ -184,9 +185,9 @@ __device__ __forceinline__ void count_step(const StepCount& c) {
     }
 }
 
-// Optionally writes sign(pred - target) / n. kVec: 16-byte accesses of aligned arrays. Bound by HBM: two quads of a
-// thread are in flight together, added in their order (67M values with the gradient: 118 us; one quad at a time
-// 136, four 125, twice the threads with 4-byte accesses 123).
+// Optionally writes sign(pred - target) / n. kVec: 16-byte accesses of aligned arrays. Bound by HBM: two
+// quads of a thread are in flight together, added in their order (67M values with the gradient: 118 us;
+// one quad at a time 136, four 125, twice the threads with 4-byte accesses 123).
 constexpr int kL1Ahead = 2;
 
 template <bool kVec>
@@ -236,20 +237,20 @@ __global__ void __launch_bounds__(kL1Threads) k_l1_final(const float* partials, 
 }
 
 // The fitting step's z box model in one pass: slice profile, L1 and its sign gradient (to lr_pred),
-// profile adjoint and the adjoint render's factors (alpha, alpha I') of the s HR voxels below each
-// LR voxel, with dL/dI = dL/dLR / s (0 in the trailing slices, which no LR slice covers). Bound by
-// HBM: I, W, target read once, dL/dLR and the factors written once. kS: slices per LR slice, whose I values stay in
-// registers. A thread owns a
-// quad of LR voxels as in k_l1_partial, so loss and gradient equal the separate entry points' bit for
-// bit; kVec: planes of a multiple of 4 voxels and aligned volumes, by 16-byte accesses.
-// As four kernels (profile, L1, its tree, factors) 16 us at 128^3, s = 2, and 33 us at
-// 256 x 256 x 128, s = 4; here 9 and 27 us (151 MB). All 1,024 blocks of 128 threads are resident at
-// once; with 256 threads and 3 (4) blocks per SM 12 and 32 (28) us; one LR voxel per thread with
-// 4-byte accesses 9 and 48 us.
-// (kS = 0: any number s_, I read again from the cache.) With more than four slices a thread's column is too long a
-// chain where there are few LR voxels or no 16-byte accesses (61 x 45 x 37, s = 16: 22 us; 33 x 33 x 256, s = 8: 14;
-// 255 x 255 x 128, s = 8: 65); the step then takes profile, L1 and factors as three kernels (11, 12 and 39 us). 256 x
-// 256 x 128: s = 5 37 in one, 35 in three; s = 8 30 and 33 (with the columns in registers 35).
+// profile adjoint and the adjoint render's factors (alpha, alpha I') of the s HR voxels below each LR
+// voxel, with dL/dI = dL/dLR / s (0 in the trailing slices, which no LR slice covers). Bound by HBM: I,
+// W, target read once, dL/dLR and the factors written once. kS: slices per LR slice, whose I values stay
+// in registers. A thread owns a quad of LR voxels as in k_l1_partial, so loss and gradient equal the
+// separate entry points' bit for bit; kVec: planes of a multiple of 4 voxels and aligned volumes, by
+// 16-byte accesses.
+// As four kernels (profile, L1, its tree, factors) 16 us at 128^3, s = 2, and 33 us at 256 x 256 x 128, s
+// = 4; here 9 and 27 us (151 MB). All 1,024 blocks of 128 threads are resident at once; with 256 threads
+// and 3 (4) blocks per SM 12 and 32 (28) us; one LR voxel per thread with 4-byte accesses 9 and 48 us.
+// (kS = 0: any number s_, I read again from the cache.) With more than four slices a thread's column is
+// too long a chain where there are few LR voxels or no 16-byte accesses (61 x 45 x 37, s = 16: 22 us; 33
+// x 33 x 256, s = 8: 14; 255 x 255 x 128, s = 8: 65); the step then takes profile, L1 and factors as
+// three kernels (11, 12 and 39 us). 256 x 256 x 128: s = 5 37 in one, 35 in three; s = 8 30 and 33 (with
+// the columns in registers 35).
 constexpr int kFusedSlices = 4, kFusedSlicesVec = 8;
 constexpr int64_t kFusedVoxels = 1 << 17;
 
@@ -315,10 +316,10 @@ __global__ void __launch_bounds__(kL1Threads, 7) k_profile_loss(
     l1_finish(acc, inv_n, partials, ticket, loss);
 }
 
-// Blocks of up to 256 threads over a plane's pieces (whole warps where there are 32 or more), the rest over the
-// slices; about 32 blocks per SM, so few large planes and many small ones fill the chip too: a grid of at most 64
-// blocks per slice with all threads along the plane took 185 us where 27 are enough (4 planes of 2,047 x 2,047, s =
-// 4) and 52 in place of 7 (100,000 planes of one voxel).
+// Blocks of up to 256 threads over a plane's pieces (whole warps where there are 32 or more), the rest
+// over the slices; about 32 blocks per SM, so few large planes and many small ones fill the chip too: a
+// grid of at most 64 blocks per slice with all threads along the plane took 185 us where 27 are enough (4
+// planes of 2,047 x 2,047, s = 4) and 52 in place of 7 (100,000 planes of one voxel).
 struct Grid2d {
     dim3 grid, block;
 };
@@ -331,7 +332,7 @@ static Grid2d grid2d(int64_t per_plane, int64_t slices) {
         tx = per_plane < 256 ? static_cast<unsigned>((per_plane + 31) / 32 * 32) : 256;
     const unsigned ty = 256 / tx;
     const int64_t by = slices < 1 ? 1 : (slices + ty - 1) / ty, gy = by < 65535 ? by : 65535;
-    const int64_t bx = (per_plane + tx - 1) / tx, most = 152 * 32 / gy > 64 ? 152 * 32 / gy : 64;
+    const int64_t bx = (per_plane + tx - 1) / tx, most = kSms * 32 / gy > 64 ? kSms * 32 / gy : 64;
     return {dim3(static_cast<unsigned>(bx < most ? bx : most), static_cast<unsigned>(gy)), dim3(tx, ty)};
 }
 

@@ -30,7 +30,8 @@ def test_bins_all_wide(dims, brick, n):
     _check(_cover(n, dims), oracle.Grid(*dims), brick)
 
 
-@pytest.mark.parametrize("dims,brick", [((64, 64, 64), (8, 8, 8)), ((64, 64, 60), (4, 4, 4)), ((520, 16, 4104), (8, 8, 8))])
+@pytest.mark.parametrize("dims,brick", [((64, 64, 64), (8, 8, 8)), ((64, 64, 60), (4, 4, 4)),
+                                        ((520, 16, 4104), (8, 8, 8))])
 @pytest.mark.parametrize("n", [300, 38_912, 38_913])
 def test_bins_wide_among_narrow(dims, brick, n):
     """Wide Gaussians of many sizes, clipped by the grid, alone and in a row, in tiles of 64 and of 256."""

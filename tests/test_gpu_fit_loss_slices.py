@@ -5,9 +5,10 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dims,s", [((61, 45, 37), 16), ((61, 45, 37), 8), ((33, 33, 64), 5), ((16, 12, 37), 37), ((5, 3, 40), 9),
-                                    ((16, 16, 33), 6), ((256, 256, 19), 9), ((256, 256, 17), 8), ((256, 256, 16), 16),
-                                    ((255, 257, 17), 8), ((256, 254, 12), 5), ((258, 128, 32), 8), ((512, 256, 9), 8)])
+@pytest.mark.parametrize("dims,s", [((61, 45, 37), 16), ((61, 45, 37), 8), ((33, 33, 64), 5), ((16, 12, 37), 37),
+                                    ((5, 3, 40), 9), ((16, 16, 33), 6), ((256, 256, 19), 9), ((256, 256, 17), 8),
+                                    ((256, 256, 16), 16), ((255, 257, 17), 8), ((256, 254, 12), 5),
+                                    ((258, 128, 32), 8), ((512, 256, 9), 8)])
 def test_loss_stage_equals_entry_points(dims, s):
     import torch
     from paper_2603_09621_gb300 import gs

@@ -7,8 +7,8 @@ pytestmark = pytest.mark.gpu
 STRIDE = 4 * 1024 * 128
 
 
-@pytest.mark.parametrize("n", [1, 3, 4, 5, 511, STRIDE - 1, STRIDE, STRIDE + 1, STRIDE + 6, 2 * STRIDE - 3, 2 * STRIDE,
-                               2 * STRIDE + 4, 3 * STRIDE - 1, 3 * STRIDE + 2, 5 * STRIDE + 7])
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 511, STRIDE - 1, STRIDE, STRIDE + 1, STRIDE + 6,
+                               2 * STRIDE - 3, 2 * STRIDE, 2 * STRIDE + 4, 3 * STRIDE - 1, 3 * STRIDE + 2, 5 * STRIDE + 7])
 def test_l1_sizes(n):
     import torch
     from paper_2603_09621_gb300 import gs

@@ -70,8 +70,9 @@ def test_resize_shapes_64bit(src, dst):
     assert torch.equal(off[1:].view(src), got) and off[0] == -7.0
 
 
-@pytest.mark.parametrize("dims,lr_shape", [((20, 24, 30), (10, 24, 20)), ((5, 33, 31), (5, 33, 31)), ((56, 34, 9), (56, 17, 3)),
-                                           ((57, 34, 9), (57, 17, 3)), ((512, 8, 12), (512, 8, 4))])
+@pytest.mark.parametrize("dims,lr_shape", [((20, 24, 30), (10, 24, 20)), ((5, 33, 31), (5, 33, 31)),
+                                           ((56, 34, 9), (56, 17, 3)), ((57, 34, 9), (57, 17, 3)),
+                                           ((512, 8, 12), (512, 8, 4))])
 def test_fused_adjoint_equals_entry_points(dims, lr_shape):
     """The fitting step's fused adjoint at these shapes, against the separate calls bit for bit."""
     from test_gpu_fit_loss import test_trilinear_step_equals_entry_points as check

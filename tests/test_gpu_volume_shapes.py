@@ -5,9 +5,11 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nz,ny,nx,s", [(1, 1, 1, 1), (1000, 1, 1, 3), (70_001, 1, 1, 1), (70_001, 1, 2, 2), (1001, 4, 4, 4),
-                                        (300, 5, 25, 7), (300, 4, 32, 5), (130, 16, 64, 3), (3, 1030, 1028, 2),
-                                        (2, 2047, 2047, 1), (4, 1031, 1033, 4), (5, 33, 31, 5), (19, 33, 31, 6), (19, 12, 31, 8), (40, 33, 31, 13), (40, 32, 31, 19)])
+@pytest.mark.parametrize("nz,ny,nx,s", [(1, 1, 1, 1), (1000, 1, 1, 3), (70_001, 1, 1, 1), (70_001, 1, 2, 2),
+                                        (1001, 4, 4, 4), (300, 5, 25, 7), (300, 4, 32, 5), (130, 16, 64, 3),
+                                        (3, 1030, 1028, 2), (2, 2047, 2047, 1), (4, 1031, 1033, 4),
+                                        (5, 33, 31, 5), (19, 33, 31, 6), (19, 12, 31, 8), (40, 33, 31, 13),
+                                        (40, 32, 31, 19)])
 def test_downsample_shapes(nz, ny, nx, s):
     import torch
     from paper_2603_09621_gb300 import gs
@@ -44,8 +46,8 @@ def _best_us(f):
 
 @pytest.mark.parametrize("shape,s", [((4, 2047, 2047), 4), ((4, 2047, 2047), 2), ((1_000_000, 4, 4), 1)])
 def test_downsample_time_follows_the_volume(shape, s):
-    """No more than three times what a volume of ordinary shape with as many voxels takes (once: 7 and 5 times for four
-    large planes of odd size; 4 and more for many small ones)."""
+    """No more than three times what a volume of ordinary shape with as many voxels takes (once: 7 and 5
+    times for four large planes of odd size; 4 and more for many small ones)."""
     import torch
     from paper_2603_09621_gb300 import gs
     ordinary = (64, 512, 512)
