@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(256) k_resample_adj_thin(const float* __restri
 
 // Shared memory of a tile (the kernel also holds the z run): 32 rows as long as five blocks fit an SM,
 // else 8 rows as long as two do, which takes volumes of up to about 1,000 columns (512 x 512 x 256 from
-// 512 x 512 x 64, 54 KB: 271 us by the run tables, 177 by the plane kernel).
+// 512 x 512 x 64, 54 KB: 271 us by the run tables, 128 by the plane kernel).
 constexpr int kPlaneSmem = 48 * 1024 - 512;
 constexpr int kPlaneSmemMax = 112 * 1024;
 
